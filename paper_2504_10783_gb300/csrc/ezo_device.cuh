@@ -6,12 +6,12 @@
 //   collision test (robot vs obstacle spheres and listed self pairs) that the
 //   paper's GPU collision checker performs (Sec. IV-D, Sec. V-B).
 //
-// Collision test, per robot sphere i and obstacle j:
-//   ||c_i - o_j||^2 < (r_i + R_j)^2
-//   <=>  t_ij = c_i.o_j + r_i R_j - (|o_j|^2 - R_j^2)/2  >  hu_i = (|c_i|^2 - r_i^2)/2.
-// t_ij is four FP32 FMAs per pair; a sphere is decided from max_j t_ij - hu_i
-// when that margin exceeds a rounding bound E, and re-checked with the
-// direct difference form otherwise, so labels equal the direct FP32 test.
+// Collision test, per robot sphere i and obstacle j: the pair collides when
+// |c_i - o_j|^2 < (r_i + R_j)^2, evaluated in FP32 differences. Which
+// obstacles a sphere is tested against comes from a grid over the obstacle
+// set (ObsGrid): per cell only those that can be the nearest to a point of
+// the cell. Self pairs use a four-FMA form of the same test with a rounding
+// bound, and the direct form inside the bound.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -178,43 +178,56 @@ __device__ __forceinline__ void stage_robot_boxes(float4* rbox_l, const RobotDev
   for (int i = threadIdx.x; i < nb; i += blockDim.x) rbox_l[i] = rd->box_l[i];
 }
 
-// Obstacle set in global memory: (x, y, z, R) and -(|o|^2 - R^2)/2, padded to
-// a multiple of EZO_CH with far-away spheres that can never collide.
+// Grid over an obstacle set (built once per set by k_grid_build): up to 32
+// coarse cells an axis and as many or twice as many fine ones. For a point of coarse
+// cell i, lb[i] step is a lower bound of its distance to the nearest obstacle
+// surface; a point outside the grid takes the cell of its projection, whose
+// bound holds for it as well (the grid contains every obstacle). A fine cell
+// lists the obstacles that can be the nearest to some point of it: obstacle j
+// is left out when another one is nearer to every point of the cell, so a
+// sphere of any radius whose centre lies in the cell collides with the set
+// exactly when it collides with a listed obstacle. Bounds are built with a
+// margin of 4e-6 of the coordinates' size, some thirty roundings of the FP32
+// pair test, so labels equal the FP32 test over all pairs.
+// cell[i]: bits 0-7 the fine cell's bound in units of step, bits 8-15 the
+// count of ids in bits 16 + 12 k (count <= kGridInline), or kGridList: a list
+// of (bits 16-31) ids from ids[bits 32-63], or kGridAll: every obstacle.
+constexpr int kGridC = 32;             // coarse cells an axis (row stride)
+constexpr int kGridLbBytes = kGridC * kGridC * kGridC;
+constexpr unsigned kGridInline = 4, kGridList = 0xFE, kGridAll = 0xFF;
+
+struct ObsGrid {
+  const uint8_t* lb;
+  const unsigned long long* cell;
+  const uint16_t* ids;
+  // x inv is the coarse cell coordinate; fma_rd(x, inv, bx) has floor(x inv)
+  // less the first cell's index in its low mantissa bits (bx = 2^23 - index,
+  // so the sum's unit is 1 and rounding down is the floor), fma_rd(x, finv,
+  // fx) likewise for the fine cells
+  float inv, finv, inv_step;
+  float bx, by, bz, fx, fy, fz;
+  float tx, ty, tz;  // 2^23 + last coarse cell
+  float ex, ey, ez;  // 2^23 + fine cells
+  int fbits;         // log2 of the fine cells' row stride: 5 or 6
+};
+
+// Obstacle set in global memory: (x, y, z, R), padded to a multiple of EZO_CH.
 struct EnvDev {
   const float4* obs;
-  const float* nhw;
   int n_obs;
   int n_obs_pad;
   const float4* box;  // obstacle boxes, 4 float4 each: (centre, h_x), (axis 0, h_y), (axis 1, h_z), (axis 2, 0)
   int n_box;
-  // first robot sphere of the obstacle sweep (a multiple of EZO_CH): the
+  // first robot sphere of the obstacle tests (a multiple of EZO_CH): the
   // spheres before it sit on the fixed base frame, so their pairs with these
   // obstacles are the same for every configuration, and they were found
   // clear of every obstacle by more than any rounding band when the pair
   // (robot, obstacle set) was set up; 0 when that does not hold
   int s_first;
+  ObsGrid grid;
 };
 
-// Shared-memory image of an obstacle set, in pairs of spheres (2p, 2p + 1):
-// obs_s[2p] = (x_2p, x_2p+1, y_2p, y_2p+1), obs_s[2p + 1] = (z_2p, z_2p+1,
-// R_2p, R_2p+1), and nhw_s[j] = -(|o_j|^2 - R_j^2)/2 in sphere order, so one
-// 128-bit load gives a coordinate of two obstacles as the float2 operand of a
-// packed FP32 FMA. n_obs_pad is a multiple of 8, so pairs never straddle the
-// padding. obs_at(j) reads sphere j back as (x, y, z, R).
-__device__ __forceinline__ void stage_env(float4* obs_s, float* nhw_s, const EnvDev& e) {
-  for (int p = threadIdx.x; p < e.n_obs_pad / 2; p += blockDim.x) {
-    const float4 a = e.obs[2 * p], b = e.obs[2 * p + 1];
-    obs_s[2 * p] = make_float4(a.x, b.x, a.y, b.y);
-    obs_s[2 * p + 1] = make_float4(a.z, b.z, a.w, b.w);
-  }
-  for (int i = threadIdx.x; i < e.n_obs_pad; i += blockDim.x) nhw_s[i] = e.nhw[i];
-}
-
-__device__ __forceinline__ float4 obs_at(const float4* __restrict__ obs_s, int j) {
-  const float* A = reinterpret_cast<const float*>(obs_s + (j & ~1));
-  const int h = j & 1;
-  return make_float4(A[h], A[2 + h], A[4 + h], A[6 + h]);
-}
+constexpr float kGridBias = 8388608.f;  // 2^23
 
 __device__ __forceinline__ void stage_env_boxes(float4* ebox_s, const EnvDev& e) {
   for (int i = threadIdx.x; i < 4 * e.n_box; i += blockDim.x) ebox_s[i] = e.box[i];
@@ -332,7 +345,7 @@ __device__ __forceinline__ void box_poses_of_frame(int b0, int b1, int lg, float
 // lane's OR.
 template <int T>
 __device__ __forceinline__ bool box_pairs_hit(const RobotSmem& rs, const float4* __restrict__ sph_s,
-                                           const float4* __restrict__ obs_s, int n_obs, const float4* __restrict__ cen,
+                                           const float4* __restrict__ obs, int n_obs, const float4* __restrict__ cen,
                                            int lg, const BoxCtx& bx) {
   bool hit = false;
   const int ns = rs.n_spheres, nb = rs.n_box, ne = bx.n_ebox;
@@ -342,7 +355,7 @@ __device__ __forceinline__ bool box_pairs_hit(const RobotSmem& rs, const float4*
   }
   for (int p = lg; p < nb * n_obs && !hit; p += T) {  // robot boxes x obstacle spheres
     const int b = p / n_obs, o = p - b * n_obs;
-    const float4 ob = obs_at(obs_s, o);
+    const float4 ob = __ldg(obs + o);
     hit = sphere_box_hit(ob, ob.w, bx.rbox_w + 4 * b);
   }
   for (int p = lg; p < nb * ne && !hit; p += T) {  // robot boxes x obstacle boxes
@@ -362,7 +375,7 @@ __device__ __forceinline__ bool box_pairs_hit(const RobotSmem& rs, const float4*
 
 // -------------------------------------------------- FK + collision test --
 // Forward kinematics of one configuration by a group of T lanes (T in
-// 1..8) of one warp, as the collision checker runs it: the group's lanes share
+// 1..32) of one warp, as the collision checker runs it: the group's lanes share
 // the joint sines and cosines, lane lg writes the centres of spheres s with
 // s % T == lg into the group's shared slot `cen` as (x, y, z, (|c|^2 - r^2)/2)
 // (padding spheres get an infinite last entry), and BOX poses the robot's
@@ -447,89 +460,106 @@ __device__ __forceinline__ void fk_group(const float (&q)[NDOF], const RobotSmem
   __syncwarp();
 }
 
-// One configuration evaluated by a group of T lanes of one warp (T in 1..8);
+// The direct pair test of sphere (c.xyz, r) against obstacle o, in FP32.
+__device__ __forceinline__ bool pair_hit(float cx, float cy, float cz, float r, float4 o) {
+  const float dx = cx - o.x, dy = cy - o.y, dz = cz - o.z;
+  const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+  const float sr = r + o.w;
+  return d2 < sr * sr;
+}
+
+// Sphere (c.xyz, r) against the obstacles of the fine cell of its centre
+// (every obstacle when the centre lies outside the grid).
+__device__ __forceinline__ bool cell_hit(const EnvDev& e, float cx, float cy, float cz, float r) {
+  const ObsGrid& g = e.grid;
+  const float ux = __fmaf_rd(cx, g.finv, g.fx), uy = __fmaf_rd(cy, g.finv, g.fy), uz = __fmaf_rd(cz, g.finv, g.fz);
+  const bool in = ux >= kGridBias && uy >= kGridBias && uz >= kGridBias && ux < g.ex && uy < g.ey && uz < g.ez;
+  unsigned long long d = (unsigned long long)kGridAll << 8;
+  if (in) {
+    const unsigned ix = __float_as_uint(ux) & 0xffu, iy = __float_as_uint(uy) & 0xffu, iz = __float_as_uint(uz) & 0xffu;
+    d = __ldg(g.cell + ((((iz << g.fbits) + iy) << g.fbits) + ix));
+    if (__fmaf_ru(r, g.inv_step, kGridBias) < __uint_as_float(0x4B000000u | (unsigned)(d & 0xffu))) return false;
+  }
+  const unsigned kind = (unsigned)(d >> 8) & 0xffu;
+  const bool list = kind == kGridList, all = kind == kGridAll;
+  const int cnt = list ? (int)((d >> 16) & 0xffffu) : (all ? e.n_obs : (int)kind);
+  const uint16_t* ids = g.ids + (list ? (unsigned)(d >> 32) : 0u);
+  unsigned long long in_ids = d >> 16;
+  for (int k = 0; k < cnt; ++k) {
+    const unsigned id = list ? (unsigned)__ldg(ids + k) : (all ? (unsigned)k : (unsigned)(in_ids & 0xfffu));
+    in_ids >>= 12;
+    if (pair_hit(cx, cy, cz, r, __ldg(e.obs + id))) return true;
+  }
+  return false;
+}
+
+// The obstacle tests of this lane's spheres s_first + lg, + T, .. of one
+// configuration. The first pass drops the spheres that the coarse bound shows
+// free (most of them: about twenty instructions a sphere whatever the number
+// of obstacles, where a sweep over all of them took three a pair); the second
+// takes the others one by one, so lanes with few of them wait only for the
+// lane with the most. 7-DOF arm of 40 spheres, against the sweep: 2e6 labels
+// among 64 obstacles 0.91 -> 0.55 ms, 2e5 among 1024 1.03 -> 0.106 ms.
+template <int T>
+__device__ __forceinline__ bool obstacles_hit(const RobotSmem& rs, const float4* __restrict__ sph_s, const EnvDev& e,
+                                              const uint8_t* __restrict__ lb, const float4* __restrict__ cen,
+                                              int lg) {
+  const ObsGrid& g = e.grid;
+  const int ns = e.n_obs > 0 ? rs.n_spheres : 0;
+  bool hit = false;
+  for (int s0 = e.s_first + lg; s0 < ns; s0 += 32 * T) {
+    unsigned near = 0u;
+#pragma unroll 4
+    for (int k = 0; k < 32; ++k) {
+      const int s = s0 + k * T;
+      if (s >= ns) break;
+      const float4 c = cen[s];
+      const float r = sph_s[s].w;
+      // fmaxf and fminf put an out-of-range (or NaN) coordinate into the grid
+      const unsigned ix = __float_as_uint(fminf(fmaxf(__fmaf_rd(c.x, g.inv, g.bx), kGridBias), g.tx));
+      const unsigned iy = __float_as_uint(fminf(fmaxf(__fmaf_rd(c.y, g.inv, g.by), kGridBias), g.ty));
+      const unsigned iz = __float_as_uint(fminf(fmaxf(__fmaf_rd(c.z, g.inv, g.bz), kGridBias), g.tz));
+      const unsigned i = ((iz & (kGridC - 1)) * kGridC + (iy & (kGridC - 1))) * kGridC + (ix & (kGridC - 1));
+      // free when ceil(r / step) < lb (a bound of 0 may stand for a negative one)
+      const float bound = __uint_as_float(0x4B000000u | (unsigned)lb[i]);
+      if (!(__fmaf_ru(r, g.inv_step, kGridBias) < bound)) near |= 1u << k;
+    }
+    while (near) {
+      const int s = s0 + (__ffs(near) - 1) * T;
+      near &= near - 1u;
+      const float4 c = cen[s];
+      if (cell_hit(e, c.x, c.y, c.z, sph_s[s].w)) {
+        hit = true;
+        break;
+      }
+    }
+    if (hit) break;
+  }
+  return hit;
+}
+
+// One configuration evaluated by a group of T lanes of one warp (T in 1..32);
 // BOX adds the box geometries (robot boxes posed along the chain, pairs with
 // a box after the sphere pairs).
 // Lane lg of the group computes the centres of spheres s with s % T == lg
 // (every lane walks the chain), the group shares them through smem slot
-// `cen`, then lane lg sweeps the obstacle pairs p (obstacles 2p, 2p + 1) with
-// p % T == lg, and the self pairs: the work items it % T == lg when the
-// pairs form link blocks, else the listed pairs p % T == lg. Returns the
-// group-wide OR.
+// `cen`, then lane lg tests its spheres against the obstacles through the
+// grid (lb: the coarse bounds, in shared or global memory), and the self
+// pairs: the work items it % T == lg when the pairs form link blocks and T is
+// at most 8, else the listed pairs p % T == lg. Returns the group-wide OR.
 // Every lane of the warp must call this together (invalid configurations are
 // evaluated and discarded).
 template <int NDOF, int T, bool BOX = false>
 __device__ __forceinline__ bool collide_group(const float (&q)[NDOF], const RobotSmem& rs,
-                                              const float4* __restrict__ sph_s,
-                                              const float4* __restrict__ obs_s,
-                                              const float* __restrict__ nhw_s, int n_obs, int n_obs_pad,
-                                              int s_first, const ushort2* __restrict__ self_pairs,
-                                              const float* __restrict__ self_rr, float E,
-                                              float4* __restrict__ cen, int lg, const BoxCtx& bx) {
+                                              const float4* __restrict__ sph_s, const EnvDev& env,
+                                              const uint8_t* __restrict__ lb,
+                                              const ushort2* __restrict__ self_pairs,
+                                              const float* __restrict__ self_rr, float4* __restrict__ cen, int lg,
+                                              const BoxCtx& bx) {
   fk_group<NDOF, T, BOX>(q, rs, sph_s, cen, lg, bx);
-
-  // ---- robot spheres vs obstacle spheres: one pair of obstacles per step,
-  //      both evaluated by packed FP32 FMAs (each half is an fma.rn of its
-  //      own, so t_ij is bit for bit the scalar chain's) ----
-  bool hit = false;
-  const int n_pairs = n_obs_pad >> 1;
-  const float2* __restrict__ nhw2 = reinterpret_cast<const float2*>(nhw_s);
-  for (int s0 = s_first; s0 < rs.n_spheres_pad; s0 += EZO_CH) {
-    float2 cx[EZO_CH], cy[EZO_CH], cz[EZO_CH], cr[EZO_CH];
-    float m[EZO_CH];
-#pragma unroll
-    for (int k = 0; k < EZO_CH; ++k) {
-      const float4 c = cen[s0 + k];
-      const float r = sph_s[s0 + k].w;
-      cx[k] = make_float2(c.x, c.x);
-      cy[k] = make_float2(c.y, c.y);
-      cz[k] = make_float2(c.z, c.z);
-      cr[k] = make_float2(r, r);
-      m[k] = -3.0e38f;
-    }
-#pragma unroll 2
-    for (int p = lg; p < n_pairs; p += T) {
-      const float4 xy = obs_s[2 * p], zr = obs_s[2 * p + 1];
-      const float2 w = nhw2[p];
-      const float2 ox = make_float2(xy.x, xy.y), oy = make_float2(xy.z, xy.w);
-      const float2 oz = make_float2(zr.x, zr.y), oR = make_float2(zr.z, zr.w);
-#pragma unroll
-      for (int k = 0; k < EZO_CH; ++k) {
-        float2 t = __ffma2_rn(cr[k], oR, w);
-        t = __ffma2_rn(cz[k], oz, t);
-        t = __ffma2_rn(cy[k], oy, t);
-        t = __ffma2_rn(cx[k], ox, t);
-        m[k] = fmax3f(m[k], t.x, t.y);
-      }
-    }
-    // spheres inside the rounding band of the fast form, as a bit mask; the
-    // rare re-check is one rolled loop (short code: the unrolled sweep
-    // already fills the instruction cache)
-    unsigned band = 0u;
-#pragma unroll
-    for (int k = 0; k < EZO_CH; ++k) {
-      const float diff = m[k] - cen[s0 + k].w;
-      if (diff > E) hit = true;
-      else if (diff >= -E) band |= 1u << k;
-    }
-    while (band) {
-      // decide with differences, over the same obstacles as this lane's
-      // maximum (its pairs)
-      const int k = __ffs(band) - 1;
-      band &= band - 1u;
-      const float4 c = cen[s0 + k];
-      const float r = sph_s[s0 + k].w;
-      for (int j = 2 * lg; j < n_obs; j += (j & 1) ? 2 * T - 1 : 1) {
-        const float4 o = obs_at(obs_s, j);
-        const float dx = c.x - o.x, dy = c.y - o.y, dz = c.z - o.z;
-        const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        const float sr = r + o.w;
-        if (d2 < sr * sr) hit = true;
-      }
-    }
-  }
+  bool hit = obstacles_hit<T>(rs, sph_s, env, lb, cen, lg);
   // ---- self pairs ----
-  if (rs.n_sblk > 0) {
+  if (T <= 8 && rs.n_sblk > 0) {
     // work items (r0, nr, k0, nk) of up to EZO_CH rows, lane lg of the group
     // taking items lg, lg + T, .. (the lanes run the same instructions on
     // their own items); same fast form as the obstacles with the partner's
@@ -596,6 +626,7 @@ __device__ __forceinline__ bool collide_group(const float (&q)[NDOF], const Robo
     }
   } else {
     // explicit pair list (direct difference form)
+#pragma unroll 4
     for (int p = lg; p < rs.n_self; p += T) {
       const ushort2 pr = self_pairs[p];
       const float4 a = cen[pr.x], b = cen[pr.y];
@@ -607,7 +638,7 @@ __device__ __forceinline__ bool collide_group(const float (&q)[NDOF], const Robo
   // ---- pairs with a box (direct tests; compiled only into the kernels for
   //      scenes with boxes, so sphere-only scenes keep their register budget) ----
   if constexpr (BOX) {
-    if (!hit) hit = box_pairs_hit<T>(rs, sph_s, obs_s, n_obs, cen, lg, bx);
+    if (!hit) hit = box_pairs_hit<T>(rs, sph_s, env.obs, env.n_obs, cen, lg, bx);
   }
   __syncwarp();
   if (T > 1) {
@@ -617,99 +648,6 @@ __device__ __forceinline__ bool collide_group(const float (&q)[NDOF], const Robo
     hit = h != 0u;
   }
   return hit;
-}
-
-// One configuration evaluated by a group of T = 16 or 32 lanes (sphere
-// geometries only). The kinematics are fk_group's. The obstacle pairs are
-// split two ways: lane lg = sg OG + og takes the robot spheres s with
-// s % SG == sg (SG = T / OG) against the obstacle pairs p with p % OG == og,
-// so each lane holds a few spheres for a few pairs instead of one chunk of
-// spheres per handful of pairs; the same fast form, rounding band and direct
-// re-check as collide_group decide each sphere, over the lane's obstacles.
-// Self pairs come from the explicit pair list, p % T == lg, in the direct
-// difference form. Returns the group-wide OR; every lane of the warp must
-// call this together.
-template <int NDOF, int T>
-__device__ __forceinline__ bool collide_wide(const float (&q)[NDOF], const RobotSmem& rs,
-                                             const float4* __restrict__ sph_s, const float4* __restrict__ obs_s,
-                                             const float* __restrict__ nhw_s, int n_obs, int n_obs_pad,
-                                             int s_first, const ushort2* __restrict__ self_pairs,
-                                             const float* __restrict__ self_rr, float E,
-                                             float4* __restrict__ cen, int lg, const BoxCtx& bx) {
-  static_assert(T == 16 || T == 32, "wide groups are 16 or 32 lanes");
-  constexpr int OG = 8, SG = T / OG, CW = 4;
-  fk_group<NDOF, T, false>(q, rs, sph_s, cen, lg, bx);
-  bool hit = false;
-  const int n_pairs = n_obs_pad >> 1;
-  const float2* __restrict__ nhw2 = reinterpret_cast<const float2*>(nhw_s);
-  const int sg = lg / OG, og = lg % OG;
-  const int nsp = rs.n_spheres_pad;
-  for (int s0 = s_first + sg; s0 < nsp; s0 += SG * CW) {
-    float2 cx[CW], cy[CW], cz[CW], cr[CW];
-    float hu[CW], m[CW];
-#pragma unroll
-    for (int k = 0; k < CW; ++k) {
-      const int s = s0 + k * SG;
-      const float4 c = s < nsp ? cen[s] : make_float4(0.f, 0.f, 0.f, __int_as_float(0x7f800000));
-      const float r = s < nsp ? sph_s[s].w : 0.f;
-      cx[k] = make_float2(c.x, c.x);
-      cy[k] = make_float2(c.y, c.y);
-      cz[k] = make_float2(c.z, c.z);
-      cr[k] = make_float2(r, r);
-      hu[k] = c.w;
-      m[k] = -3.0e38f;
-    }
-    for (int p = og; p < n_pairs; p += OG) {
-      const float4 xy = obs_s[2 * p], zr = obs_s[2 * p + 1];
-      const float2 w = nhw2[p];
-      const float2 ox = make_float2(xy.x, xy.y), oy = make_float2(xy.z, xy.w);
-      const float2 oz = make_float2(zr.x, zr.y), oR = make_float2(zr.z, zr.w);
-#pragma unroll
-      for (int k = 0; k < CW; ++k) {
-        float2 t = __ffma2_rn(cr[k], oR, w);
-        t = __ffma2_rn(cz[k], oz, t);
-        t = __ffma2_rn(cy[k], oy, t);
-        t = __ffma2_rn(cx[k], ox, t);
-        m[k] = fmax3f(m[k], t.x, t.y);
-      }
-    }
-    unsigned band = 0u;
-#pragma unroll
-    for (int k = 0; k < CW; ++k) {
-      const float diff = m[k] - hu[k];
-      if (diff > E) hit = true;
-      else if (diff >= -E) band |= 1u << k;
-    }
-    while (band) {
-      // inside the rounding band: direct differences over this lane's
-      // obstacles (2p, 2p + 1 for its pairs p), in one rolled loop
-      const int k = __ffs(band) - 1;
-      band &= band - 1u;
-      const int s = s0 + k * SG;
-      const float4 c = cen[s];
-      const float r = sph_s[s].w;
-      for (int j = 2 * og; j < n_obs; j += (j & 1) ? 2 * OG - 1 : 1) {
-        const float4 o = obs_at(obs_s, j);
-        const float dx = c.x - o.x, dy = c.y - o.y, dz = c.z - o.z;
-        const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        const float sr = r + o.w;
-        if (d2 < sr * sr) hit = true;
-      }
-    }
-  }
-#pragma unroll 4
-  for (int p = lg; p < rs.n_self; p += T) {
-    const ushort2 pr = self_pairs[p];
-    const float4 a = cen[pr.x], b = cen[pr.y];
-    const float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
-    const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    if (d2 < self_rr[p]) hit = true;
-  }
-  __syncwarp();
-  unsigned h = hit ? 1u : 0u;
-#pragma unroll
-  for (int off = 1; off < T; off <<= 1) h |= __shfl_xor_sync(0xffffffffu, h, off, T);
-  return h != 0u;
 }
 
 // Signed distance min over pairs of ||c_i - c_j|| - r_i - r_j for one
@@ -756,7 +694,7 @@ __device__ float signed_distance_one(const float* __restrict__ q, const RobotSme
   for (int s = 0; s < rs.n_spheres; ++s) {
     const float4 c = cen[s];
     for (int j = 0; j < n_obs; ++j) {
-      const float4 o = obs_at(obs_s, j);
+      const float4 o = obs_s[j];
       const float dx = c.x - o.x, dy = c.y - o.y, dz = c.z - o.z;
       const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
       const float lim = c.w + o.w + best;

@@ -60,8 +60,6 @@ struct SegState {
 
 struct EnvDevFull {
   EnvDev e;
-  float E;  // rounding band of the fast pair test for this robot/env
-  float pad;
 };
 
 struct RoundSummary {
@@ -142,7 +140,7 @@ struct BatchView {
 };
 
 // Launchers (ezo_kernels.cu). T = lanes per configuration.
-cudaError_t launch_check_flat(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env, float E,
+cudaError_t launch_check_flat(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env,
                               const float* q, long long ldq, long long N, uint8_t* flags, int T, int grid_cap,
                               cudaStream_t s);
 // signed distance, exact below cap (3e38: exact everywhere)
@@ -191,16 +189,16 @@ cudaError_t launch_wave_select(const BatchView& v, const uint8_t* contained, int
 // round end fused with the next round's sizing (the run loops' last kernel)
 cudaError_t launch_round_close(const BatchView& v, cudaStream_t s);
 // recovery (Sec. VI-B)
-cudaError_t launch_check_path(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env, float E,
+cudaError_t launch_check_path(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env,
                               const double* verts, int n_edges, const long long* off, long long N,
                               uint8_t* point_flags, uint8_t* edge_flags, int T, int grid_cap, cudaStream_t s);
 cudaError_t launch_coverage(const BatchView& v, uint8_t* covered, double tol, cudaStream_t s);
 // the same collision launchers for scenes with box geometries (compiled in
 // separate translation units so that the sphere-only kernels stay lean)
-cudaError_t launch_check_flat_box(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env, float E,
+cudaError_t launch_check_flat_box(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env,
                                   const float* q, long long ldq, long long N, uint8_t* flags, int T, int grid_cap,
                                   cudaStream_t s);
-cudaError_t launch_check_path_box(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env, float E,
+cudaError_t launch_check_path_box(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env,
                                   const double* verts, int n_edges, const long long* off, long long N,
                                   uint8_t* point_flags, uint8_t* edge_flags, int T, int grid_cap, cudaStream_t s);
 cudaError_t launch_round_check_box(const BatchView& v, int T, int grid, cudaStream_t s);
@@ -208,6 +206,21 @@ cudaError_t launch_round_bisect_box(const BatchView& v, int T, int grid, cudaStr
 
 cudaError_t launch_fk_centres(const RobotDev* robot, const RobotFK64* r64, int n, int nsp_pad, const float* q,
                               long long ldq, long long N, int mode, double* out_c, float* err, cudaStream_t s);
+// Builds the grid over n_obs obstacles (ezo_grid.cu): the coarse bounds, the
+// fine cells and their id lists; `used` (zero before) counts list entries.
+struct GridBuild {
+  const float4* obs;
+  int n_obs;
+  int k0[3], n[3];   // first coarse cell's index and the cells an axis
+  int sub;           // fine cells per coarse cell and axis: 1 or 2
+  float h, margin, step, far;
+  uint8_t* lb;
+  unsigned long long* cell;
+  uint16_t* ids;
+  unsigned ids_cap;
+  unsigned* used;
+};
+cudaError_t launch_grid_build(const GridBuild& g, cudaStream_t s);
 size_t check_smem_bytes(int n_spheres_pad, int n_obs_pad, int threads, int T, int n_rbox = 0, int n_ebox = 0);
 // Dynamic shared memory a collision kernel may request: the opt-in maximum
 // per block (227 KB) less the static robot image and a margin. The sphere

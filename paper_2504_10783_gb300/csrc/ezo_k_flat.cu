@@ -32,21 +32,20 @@ __global__ void __launch_bounds__(128) k_sample_flat(const double* __restrict__ 
 #endif  // !EZO_BOX_TU
 
 template <int NDOF, int T, bool BOX>
-__global__ void __launch_bounds__(128) k_check_flat(const RobotDev* __restrict__ robot, EnvDev env, float E,
+__global__ void __launch_bounds__(128) k_check_flat(const RobotDev* __restrict__ robot, EnvDev env, int stage_lb,
                                                     const float* __restrict__ q, long long ldq, long long N,
                                                     uint8_t* __restrict__ flags) {
   extern __shared__ float4 smem4[];
   __shared__ RobotSmem rs;
   const int nsp = robot->n_spheres_pad, nrbox = robot->n_box;
   const int groups = blockDim.x / T;
-  const GeomSmem gs = carve_geom(smem4, nsp, env.n_obs_pad, groups, nrbox, env.n_box);
+  const GeomSmem gs = carve_geom(smem4, nsp, groups, nrbox, env.n_box);
   float4* sph_s = gs.sph;
-  float4* obs_s = gs.obs;
-  float* nhw_s = gs.nhw;
   stage_robot(rs, sph_s, robot);
   stage_robot_boxes(gs.rbox_l, robot);
-  stage_env(obs_s, nhw_s, env);
   stage_env_boxes(gs.ebox, env);
+  if (stage_lb) stage_grid(gs.lb, env);
+  const uint8_t* lb = stage_lb ? gs.lb : env.grid.lb;
   __syncthreads();
   const int gi = threadIdx.x / T, lg = threadIdx.x % T;
   float4* cen = gs.cen_all + gi * (nsp + 1);
@@ -59,9 +58,7 @@ __global__ void __launch_bounds__(128) k_check_flat(const RobotDev* __restrict__
     float qq[NDOF];
 #pragma unroll
     for (int j = 0; j < NDOF; ++j) qq[j] = (j < rs.n) ? q[j * ldq + ic] : 0.f;
-    const bool hit =
-        collide_group<NDOF, T, BOX>(qq, rs, sph_s, obs_s, nhw_s, env.n_obs, env.n_obs_pad, env.s_first, sp, srr, E, cen,
-                                    lg, bx);
+    const bool hit = collide_group<NDOF, T, BOX>(qq, rs, sph_s, env, lb, sp, srr, cen, lg, bx);
     if (i < N && lg == 0) flags[i] = hit ? 1 : 0;
   }
 }
@@ -78,9 +75,8 @@ __global__ void __launch_bounds__(128) k_sd_flat(const RobotDev* __restrict__ ro
   float4* sph_s = smem4;
   float4* obs_s = sph_s + nsp;
   float4* cen_all = obs_s + env.n_obs_pad;
-  float* nhw_s = reinterpret_cast<float*>(cen_all + blockDim.x * (nsp + 1));
   stage_robot(rs, sph_s, robot);
-  stage_env(obs_s, nhw_s, env);
+  for (int i = threadIdx.x; i < env.n_obs_pad; i += blockDim.x) obs_s[i] = env.obs[i];
   __syncthreads();
   float4* cen = cen_all + threadIdx.x * (nsp + 1);
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
@@ -183,49 +179,59 @@ cudaError_t launch_fk_centres(const RobotDev* robot, const RobotFK64* r64, int n
 }
 
 size_t check_smem_bytes(int n_spheres_pad, int n_obs_pad, int threads, int T, int n_rbox, int n_ebox) {
-  return check_smem_layout(n_spheres_pad, n_obs_pad, threads, T, n_rbox, n_ebox);
+  return check_smem_rule(n_spheres_pad, n_obs_pad, threads, T, n_rbox, n_ebox);
 }
 
 #endif  // !EZO_BOX_TU
 
 #if EZO_BOX_TU
-cudaError_t launch_check_flat_box(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env, float E,
+cudaError_t launch_check_flat_box(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env,
                               const float* q, long long ldq, long long N, uint8_t* flags, int T, int grid_cap,
                               cudaStream_t s) {
   if (N <= 0) return cudaSuccess;
   cudaError_t err = cudaSuccess;
   const int threads = 128;
-  const size_t smem = check_smem_layout(nsp_pad, env.n_obs_pad, threads, T, n_rbox, env.n_box);
   const long long groups = threads / T;
   long long grid = (N + groups - 1) / groups;
   if (grid_cap > 0 && grid > grid_cap) grid = grid_cap;
+  // the coarse bounds go to shared memory when a block looks up enough of
+  // them to pay for the copy and they fit beside the sphere centres
+  const bool stage = stage_grid_pays(nsp_pad, env, N, T) &&
+                     check_smem_layout(nsp_pad, threads, T, n_rbox, env.n_box, true) <= kSmemBudget;
+  const size_t smem = check_smem_layout(nsp_pad, threads, T, n_rbox, env.n_box, stage);
   constexpr bool BB = EZO_BOX_TU != 0;
   EZO_DISPATCH_NDOF(n, EZO_DISPATCH_T(T, {
     auto kern = k_check_flat<ND, TT, BB>;
     err = set_smem(kern, smem);
     if (err != cudaSuccess) return err;
-    kern<<<(unsigned)grid, threads, smem, s>>>(robot, env, E, q, ldq, N, flags);
+    const int blocks = resident_grid(kern, threads, smem, (int)std::min<long long>(grid, 1 << 20));
+    kern<<<blocks, threads, smem, s>>>(robot, env, stage ? 1 : 0, q, ldq, N, flags);
   }));
   return cudaGetLastError();
 }
 #else
-cudaError_t launch_check_flat(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env, float E,
+cudaError_t launch_check_flat(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env,
                               const float* q, long long ldq, long long N, uint8_t* flags, int T, int grid_cap,
                               cudaStream_t s) {
-  if (n_rbox || env.n_box) return launch_check_flat_box(robot, n, nsp_pad, n_rbox, env, E, q, ldq, N, flags, T, grid_cap, s);
+  if (n_rbox || env.n_box) return launch_check_flat_box(robot, n, nsp_pad, n_rbox, env, q, ldq, N, flags, T, grid_cap, s);
   if (N <= 0) return cudaSuccess;
   cudaError_t err = cudaSuccess;
   const int threads = 128;
-  const size_t smem = check_smem_layout(nsp_pad, env.n_obs_pad, threads, T, n_rbox, env.n_box);
   const long long groups = threads / T;
   long long grid = (N + groups - 1) / groups;
   if (grid_cap > 0 && grid > grid_cap) grid = grid_cap;
+  // the coarse bounds go to shared memory when a block looks up enough of
+  // them to pay for the copy and they fit beside the sphere centres
+  const bool stage = stage_grid_pays(nsp_pad, env, N, T) &&
+                     check_smem_layout(nsp_pad, threads, T, n_rbox, env.n_box, true) <= kSmemBudget;
+  const size_t smem = check_smem_layout(nsp_pad, threads, T, n_rbox, env.n_box, stage);
   constexpr bool BB = EZO_BOX_TU != 0;
   EZO_DISPATCH_NDOF(n, EZO_DISPATCH_T(T, {
     auto kern = k_check_flat<ND, TT, BB>;
     err = set_smem(kern, smem);
     if (err != cudaSuccess) return err;
-    kern<<<(unsigned)grid, threads, smem, s>>>(robot, env, E, q, ldq, N, flags);
+    const int blocks = resident_grid(kern, threads, smem, (int)std::min<long long>(grid, 1 << 20));
+    kern<<<blocks, threads, smem, s>>>(robot, env, stage ? 1 : 0, q, ldq, N, flags);
   }));
   return cudaGetLastError();
 }
@@ -239,7 +245,7 @@ cudaError_t launch_sd_flat(const RobotDev* robot, int n, int nsp_pad, const EnvD
   if (N <= 0) return cudaSuccess;
   cudaError_t err = cudaSuccess;
   const int threads = 64;
-  const size_t smem = check_smem_layout(nsp_pad, env.n_obs_pad, threads, 1);
+  const size_t smem = check_smem_rule(nsp_pad, env.n_obs_pad, threads, 1);
   const long long grid = (N + threads - 1) / threads;
   EZO_DISPATCH_NDOF(n, {
     auto kern = k_sd_flat<ND>;

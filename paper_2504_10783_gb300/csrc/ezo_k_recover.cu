@@ -23,7 +23,7 @@ namespace ezo {
 #endif  // !EZO_BOX_TU
 
 template <int NDOF, int T, bool BOX>
-__global__ void __launch_bounds__(128) k_check_path(const RobotDev* __restrict__ robot, EnvDev env, float E,
+__global__ void __launch_bounds__(128) k_check_path(const RobotDev* __restrict__ robot, EnvDev env, int stage_lb,
                                                     const double* __restrict__ verts, int n_edges,
                                                     const long long* __restrict__ off, long long N,
                                                     uint8_t* __restrict__ point_flags,
@@ -32,14 +32,13 @@ __global__ void __launch_bounds__(128) k_check_path(const RobotDev* __restrict__
   __shared__ RobotSmem rs;
   const int nsp = robot->n_spheres_pad, nrbox = robot->n_box;
   const int groups = blockDim.x / T;
-  const GeomSmem gs = carve_geom(smem4, nsp, env.n_obs_pad, groups, nrbox, env.n_box);
+  const GeomSmem gs = carve_geom(smem4, nsp, groups, nrbox, env.n_box);
   float4* sph_s = gs.sph;
-  float4* obs_s = gs.obs;
-  float* nhw_s = gs.nhw;
   stage_robot(rs, sph_s, robot);
   stage_robot_boxes(gs.rbox_l, robot);
-  stage_env(obs_s, nhw_s, env);
   stage_env_boxes(gs.ebox, env);
+  if (stage_lb) stage_grid(gs.lb, env);
+  const uint8_t* lb = stage_lb ? gs.lb : env.grid.lb;
   __syncthreads();
   const int gi = threadIdx.x / T, lg = threadIdx.x % T;
   float4* cen = gs.cen_all + gi * (nsp + 1);
@@ -63,8 +62,7 @@ __global__ void __launch_bounds__(128) k_check_path(const RobotDev* __restrict__
 #pragma unroll
     for (int j = 0; j < NDOF; ++j)
       qq[j] = (j < n) ? (float)__dadd_rn(va[j], __dmul_rn(t, __dsub_rn(vb[j], va[j]))) : 0.f;
-    const bool hit = collide_group<NDOF, T, BOX>(qq, rs, sph_s, obs_s, nhw_s, env.n_obs, env.n_obs_pad,
-                                            env.s_first, robot->self_pairs, robot->self_rr, E, cen, lg, bx);
+    const bool hit = collide_group<NDOF, T, BOX>(qq, rs, sph_s, env, lb, robot->self_pairs, robot->self_rr, cen, lg, bx);
     if (i < N && lg == 0) {
       if (point_flags) point_flags[i] = hit ? 1 : 0;
       if (hit) edge_flags[k] = 1;  // every writer stores the same value
@@ -73,13 +71,15 @@ __global__ void __launch_bounds__(128) k_check_path(const RobotDev* __restrict__
 }
 
 #if EZO_BOX_TU
-cudaError_t launch_check_path_box(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env, float E,
+cudaError_t launch_check_path_box(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env,
                               const double* verts, int n_edges, const long long* off, long long N,
                               uint8_t* point_flags, uint8_t* edge_flags, int T, int grid_cap, cudaStream_t s) {
   if (N <= 0 || n_edges <= 0) return cudaSuccess;
   cudaError_t err = cudaSuccess;
   const int threads = 128;
-  const size_t smem = check_smem_layout(nsp_pad, env.n_obs_pad, threads, T, n_rbox, env.n_box);
+  const bool stage = stage_grid_pays(nsp_pad, env, N, T) &&
+                     check_smem_layout(nsp_pad, threads, T, n_rbox, env.n_box, true) <= kSmemBudget;
+  const size_t smem = check_smem_layout(nsp_pad, threads, T, n_rbox, env.n_box, stage);
   const long long groups = threads / T;
   long long grid = (N + groups - 1) / groups;
   if (grid_cap > 0 && grid > grid_cap) grid = grid_cap;
@@ -88,19 +88,22 @@ cudaError_t launch_check_path_box(const RobotDev* robot, int n, int nsp_pad, int
     auto kern = k_check_path<ND, TT, BB>;
     err = set_smem(kern, smem);
     if (err != cudaSuccess) return err;
-    kern<<<(unsigned)grid, threads, smem, s>>>(robot, env, E, verts, n_edges, off, N, point_flags, edge_flags);
+    const int blocks = resident_grid(kern, threads, smem, (int)std::min<long long>(grid, 1 << 20));
+    kern<<<blocks, threads, smem, s>>>(robot, env, stage ? 1 : 0, verts, n_edges, off, N, point_flags, edge_flags);
   }));
   return cudaGetLastError();
 }
 #else
-cudaError_t launch_check_path(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env, float E,
+cudaError_t launch_check_path(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env,
                               const double* verts, int n_edges, const long long* off, long long N,
                               uint8_t* point_flags, uint8_t* edge_flags, int T, int grid_cap, cudaStream_t s) {
-  if (n_rbox || env.n_box) return launch_check_path_box(robot, n, nsp_pad, n_rbox, env, E, verts, n_edges, off, N, point_flags, edge_flags, T, grid_cap, s);
+  if (n_rbox || env.n_box) return launch_check_path_box(robot, n, nsp_pad, n_rbox, env, verts, n_edges, off, N, point_flags, edge_flags, T, grid_cap, s);
   if (N <= 0 || n_edges <= 0) return cudaSuccess;
   cudaError_t err = cudaSuccess;
   const int threads = 128;
-  const size_t smem = check_smem_layout(nsp_pad, env.n_obs_pad, threads, T, n_rbox, env.n_box);
+  const bool stage = stage_grid_pays(nsp_pad, env, N, T) &&
+                     check_smem_layout(nsp_pad, threads, T, n_rbox, env.n_box, true) <= kSmemBudget;
+  const size_t smem = check_smem_layout(nsp_pad, threads, T, n_rbox, env.n_box, stage);
   const long long groups = threads / T;
   long long grid = (N + groups - 1) / groups;
   if (grid_cap > 0 && grid > grid_cap) grid = grid_cap;
@@ -109,7 +112,8 @@ cudaError_t launch_check_path(const RobotDev* robot, int n, int nsp_pad, int n_r
     auto kern = k_check_path<ND, TT, BB>;
     err = set_smem(kern, smem);
     if (err != cudaSuccess) return err;
-    kern<<<(unsigned)grid, threads, smem, s>>>(robot, env, E, verts, n_edges, off, N, point_flags, edge_flags);
+    const int blocks = resident_grid(kern, threads, smem, (int)std::min<long long>(grid, 1 << 20));
+    kern<<<blocks, threads, smem, s>>>(robot, env, stage ? 1 : 0, verts, n_edges, off, N, point_flags, edge_flags);
   }));
   return cudaGetLastError();
 }

@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(128, NDOF <= 7 ? (SPLIT ? 5 : 7) : 4)
 #endif  // !EZO_BOX_TU
 
 template <int NDOF, int T, bool BOX>
-__global__ void __launch_bounds__(128) k_round_check(BatchView v, int max_obs_pad) {
+__global__ void __launch_bounds__(128) k_round_check(BatchView v, int stage_lb) {
   extern __shared__ float4 smem4[];
   __shared__ RobotSmem rs;
   __shared__ int cur_env;
@@ -163,10 +163,8 @@ __global__ void __launch_bounds__(128) k_round_check(BatchView v, int max_obs_pa
   const RobotDev* robot = v.robot;
   const int nsp = robot->n_spheres_pad, nrbox = robot->n_box;
   const int groups = blockDim.x / T;
-  const GeomSmem gs = carve_geom(smem4, nsp, max_obs_pad, groups, nrbox, v.max_ebox);
+  const GeomSmem gs = carve_geom(smem4, nsp, groups, nrbox, v.max_ebox);
   float4* sph_s = gs.sph;
-  float4* obs_s = gs.obs;
-  float* nhw_s = gs.nhw;
   stage_robot(rs, sph_s, robot);
   stage_robot_boxes(gs.rbox_l, robot);
   if (threadIdx.x == 0) cur_env = -1;
@@ -180,7 +178,7 @@ __global__ void __launch_bounds__(128) k_round_check(BatchView v, int max_obs_pa
     const EnvDevFull& ef = v.envs[st.env];
     if (st.env != cur_env) {
       __syncthreads();
-      stage_env(obs_s, nhw_s, ef.e);
+      if (stage_lb) stage_grid(gs.lb, ef.e);
       stage_env_boxes(gs.ebox, ef.e);
       if (threadIdx.x == 0) cur_env = st.env;
       __syncthreads();
@@ -195,8 +193,9 @@ __global__ void __launch_bounds__(128) k_round_check(BatchView v, int max_obs_pa
       float qq[NDOF];
 #pragma unroll
       for (int j = 0; j < NDOF; ++j) qq[j] = (j < v.n) ? S[(long long)j * st.s_cap + ic] : 0.f;
-      const bool hit = collide_group<NDOF, T, BOX>(qq, rs, sph_s, obs_s, nhw_s, ef.e.n_obs, ef.e.n_obs_pad,
-                                              ef.e.s_first, robot->self_pairs, robot->self_rr, ef.E, cen, lg, bx);
+      const EnvDev env = ef.e;
+      const bool hit = collide_group<NDOF, T, BOX>(qq, rs, sph_s, env, stage_lb ? gs.lb : env.grid.lb,
+                                                   robot->self_pairs, robot->self_rr, cen, lg, bx);
       if (valid && lg == 0) fl[i] = hit ? 1 : 0;
     }
   }
@@ -358,13 +357,14 @@ cudaError_t launch_round_sample(const BatchView& v, int split_below_tiles, int g
 #if EZO_BOX_TU
 cudaError_t launch_round_check_box(const BatchView& v, int T, int grid, cudaStream_t s) {
   cudaError_t err = cudaSuccess;
-  const size_t smem = check_smem_layout(v.nsp_pad, v.max_obs_pad, 128, T, v.n_rbox, v.max_ebox);
+  const bool stage = check_smem_layout(v.nsp_pad, 128, T, v.n_rbox, v.max_ebox, true) <= kSmemBudget;
+  const size_t smem = check_smem_layout(v.nsp_pad, 128, T, v.n_rbox, v.max_ebox, stage);
   constexpr bool BB = EZO_BOX_TU != 0;
   EZO_DISPATCH_NDOF(v.n, EZO_DISPATCH_T(T, {
     auto kern = k_round_check<ND, TT, BB>;
     err = set_smem(kern, smem);
     if (err != cudaSuccess) return err;
-    kern<<<resident_grid(kern, 128, smem, grid), 128, smem, s>>>(v, v.max_obs_pad);
+    kern<<<resident_grid(kern, 128, smem, grid), 128, smem, s>>>(v, stage ? 1 : 0);
   }));
   return cudaGetLastError();
 }
@@ -372,13 +372,14 @@ cudaError_t launch_round_check_box(const BatchView& v, int T, int grid, cudaStre
 cudaError_t launch_round_check(const BatchView& v, int T, int grid, cudaStream_t s) {
   if (v.n_rbox || v.max_ebox) return launch_round_check_box(v, T, grid, s);
   cudaError_t err = cudaSuccess;
-  const size_t smem = check_smem_layout(v.nsp_pad, v.max_obs_pad, 128, T, v.n_rbox, v.max_ebox);
+  const bool stage = check_smem_layout(v.nsp_pad, 128, T, v.n_rbox, v.max_ebox, true) <= kSmemBudget;
+  const size_t smem = check_smem_layout(v.nsp_pad, 128, T, v.n_rbox, v.max_ebox, stage);
   constexpr bool BB = EZO_BOX_TU != 0;
   EZO_DISPATCH_NDOF(v.n, EZO_DISPATCH_T(T, {
     auto kern = k_round_check<ND, TT, BB>;
     err = set_smem(kern, smem);
     if (err != cudaSuccess) return err;
-    kern<<<resident_grid(kern, 128, smem, grid), 128, smem, s>>>(v, v.max_obs_pad);
+    kern<<<resident_grid(kern, 128, smem, grid), 128, smem, s>>>(v, stage ? 1 : 0);
   }));
   return cudaGetLastError();
 }

@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kRowBlock) k_bisect_finish(BatchView v) {
 // outcome), and bis_mode 2 redoes the exact halvings for the candidates whose
 // surrogate end point was free.
 template <int NDOF, int T, bool BOX>
-__global__ void __launch_bounds__(128) k_round_bisect(BatchView v, int max_obs_pad) {
+__global__ void __launch_bounds__(128) k_round_bisect(BatchView v, int stage_lb) {
   extern __shared__ float4 smem4[];
   __shared__ RobotSmem rs;
   __shared__ int cur_env;
@@ -186,10 +186,8 @@ __global__ void __launch_bounds__(128) k_round_bisect(BatchView v, int max_obs_p
   const RobotDev* robot = v.robot;
   const int nsp = robot->n_spheres_pad, nrbox = robot->n_box;
   const int groups = blockDim.x / T;
-  const GeomSmem gs = carve_geom(smem4, nsp, max_obs_pad, groups, nrbox, v.max_ebox);
+  const GeomSmem gs = carve_geom(smem4, nsp, groups, nrbox, v.max_ebox);
   float4* sph_s = gs.sph;
-  float4* obs_s = gs.obs;
-  float* nhw_s = gs.nhw;
   stage_robot(rs, sph_s, robot);
   stage_robot_boxes(gs.rbox_l, robot);
   if (threadIdx.x == 0) cur_env = -1;
@@ -207,15 +205,14 @@ __global__ void __launch_bounds__(128) k_round_bisect(BatchView v, int max_obs_p
     const EnvDevFull& ef = v.envs[st.env];
     if (st.env != cur_env) {
       __syncthreads();
-      stage_env(obs_s, nhw_s, ef.e);
+      if (stage_lb) stage_grid(gs.lb, ef.e);
       stage_env_boxes(gs.ebox, ef.e);
       if (threadIdx.x == 0) cur_env = st.env;
       __syncthreads();
     }
     const BoxCtx bx = box_ctx(gs, robot, nrbox, ef.e.n_box, gi);
-    // the scene's scalars in registers for the N_b checks
-    const int n_obs = ef.e.n_obs, n_obs_pad = ef.e.n_obs_pad, s_first = ef.e.s_first;
-    const float E = ef.E;
+    const EnvDev env = ef.e;  // in registers for the N_b checks
+    const uint8_t* lb = stage_lb ? gs.lb : env.grid.lb;
     const ushort2* self_pairs = robot->self_pairs;
     const float* self_rr = robot->self_rr;
     const int c = tile.y + sub + gi;
@@ -250,13 +247,7 @@ __global__ void __launch_bounds__(128) k_round_bisect(BatchView v, int max_obs_p
       float qq[NDOF];
 #pragma unroll
       for (int j = 0; j < NDOF; ++j) qq[j] = fmaf(f, dv32[j], p32[j]);
-      bool hit;
-      if constexpr (T > 8)
-        hit = collide_wide<NDOF, T>(qq, rs, sph_s, obs_s, nhw_s, n_obs, n_obs_pad, s_first, self_pairs, self_rr, E, cen,
-                                    lg, bx);
-      else
-        hit = collide_group<NDOF, T, BOX>(qq, rs, sph_s, obs_s, nhw_s, n_obs, n_obs_pad, s_first, self_pairs, self_rr, E,
-                                          cen, lg, bx);
+      const bool hit = collide_group<NDOF, T, BOX>(qq, rs, sph_s, env, lb, self_pairs, self_rr, cen, lg, bx);
       if (v.bis_mode == 1) {
         if (valid && lg == 0) {
           v.s_ok[row] = hit ? 1 : 0;
@@ -285,10 +276,9 @@ __global__ void __launch_bounds__(128) k_round_bisect(BatchView v, int max_obs_p
 // point are the sequential halvings' bit for bit. Half the dependent checks
 // for half again the checks; an odd last halving is warp 1's alone.
 template <int NDOF>
-__global__ void __launch_bounds__(96) k_round_bisect_pair(BatchView v, int max_obs_pad) {
+__global__ void __launch_bounds__(96) k_round_bisect_pair(BatchView v) {
   extern __shared__ float4 smem4[];
   __shared__ RobotSmem rs;
-  __shared__ int cur_env;
   __shared__ int s_hit[3];
   const int n_tiles = v.summary->n_bisect_tiles;
   int* q = &v.summary->q_bisect[v.bis_mode];
@@ -301,12 +291,9 @@ __global__ void __launch_bounds__(96) k_round_bisect_pair(BatchView v, int max_o
   }
   const RobotDev* robot = v.robot;
   const int nsp = robot->n_spheres_pad;
-  const GeomSmem gs = carve_geom(smem4, nsp, max_obs_pad, 3, 0, 0);
+  const GeomSmem gs = carve_geom(smem4, nsp, 3, 0, 0);
   float4* sph_s = gs.sph;
-  float4* obs_s = gs.obs;
-  float* nhw_s = gs.nhw;
   stage_robot(rs, sph_s, robot);
-  if (threadIdx.x == 0) cur_env = -1;
   __syncthreads();
   const int w = threadIdx.x >> 5, lg = threadIdx.x & 31;
   float4* cen = gs.cen_all + w * (nsp + 1);
@@ -320,14 +307,7 @@ __global__ void __launch_bounds__(96) k_round_bisect_pair(BatchView v, int max_o
     const int g = tile.x;
     const SegState& st = v.st[g];
     const EnvDevFull& ef = v.envs[st.env];
-    if (st.env != cur_env) {
-      __syncthreads();
-      stage_env(obs_s, nhw_s, ef.e);
-      if (threadIdx.x == 0) cur_env = st.env;
-      __syncthreads();
-    }
-    const int n_obs = ef.e.n_obs, n_obs_pad = ef.e.n_obs_pad, s_first = ef.e.s_first;
-    const float E = ef.E;
+    const EnvDev env = ef.e;
     const ushort2* self_pairs = robot->self_pairs;
     const float* self_rr = robot->self_rr;
     bool valid = c < st.n_cand;
@@ -355,8 +335,7 @@ __global__ void __launch_bounds__(96) k_round_bisect_pair(BatchView v, int max_o
 #pragma unroll
         for (int j = 0; j < NDOF; ++j) qq[j] = fmaf(f, dv32[j], p32[j]);
         const bool hit =
-            collide_wide<NDOF, 32>(qq, rs, sph_s, obs_s, nhw_s, n_obs, n_obs_pad, s_first, self_pairs, self_rr, E, cen, lg,
-                                   bx);
+            collide_group<NDOF, 32>(qq, rs, sph_s, env, env.grid.lb, self_pairs, self_rr, cen, lg, bx);
         if (lg == 0) s_hit[w] = hit ? 1 : 0;
       }
       __syncthreads();
@@ -776,13 +755,14 @@ __global__ void k_wave_select(BatchView v, const uint8_t* __restrict__ contained
 #if EZO_BOX_TU
 cudaError_t launch_round_bisect_box(const BatchView& v, int T, int grid, cudaStream_t s) {
   cudaError_t err = cudaSuccess;
-  const size_t smem = check_smem_layout(v.nsp_pad, v.max_obs_pad, 128, T, v.n_rbox, v.max_ebox);
+  const bool stage = false;
+  const size_t smem = check_smem_layout(v.nsp_pad, 128, T, v.n_rbox, v.max_ebox, stage);
   constexpr bool BB = EZO_BOX_TU != 0;
   EZO_DISPATCH_NDOF(v.n, EZO_DISPATCH_T(T, {
     auto kern = k_round_bisect<ND, TT, BB>;
     err = set_smem(kern, smem);
     if (err != cudaSuccess) return err;
-    kern<<<resident_grid(kern, 128, smem, grid), 128, smem, s>>>(v, v.max_obs_pad);
+    kern<<<resident_grid(kern, 128, smem, grid), 128, smem, s>>>(v, stage ? 1 : 0);
   }));
   return cudaGetLastError();
 }
@@ -794,23 +774,24 @@ cudaError_t launch_round_bisect(const BatchView& v, int T, int grid, cudaStream_
   if (T == kBisectPairLanes && v.bis_mode == 1) T = 32;  // one check per candidate: the 32-lane kernel
   if (T == kBisectPairLanes) {
     cudaError_t err = cudaSuccess;
-    const size_t smem = check_smem_layout(v.nsp_pad, v.max_obs_pad, 96, 32, 0, 0);
+    const size_t smem = check_smem_layout(v.nsp_pad, 96, 32, 0, 0, false);
     EZO_DISPATCH_NDOF(v.n, {
       auto kern = k_round_bisect_pair<ND>;
       err = set_smem(kern, smem);
       if (err != cudaSuccess) return err;
-      kern<<<resident_grid(kern, 96, smem, std::max(grid, 1) * 4), 96, smem, s>>>(v, v.max_obs_pad);
+      kern<<<resident_grid(kern, 96, smem, std::max(grid, 1) * 4), 96, smem, s>>>(v);
     });
     return cudaGetLastError();
   }
   cudaError_t err = cudaSuccess;
-  const size_t smem = check_smem_layout(v.nsp_pad, v.max_obs_pad, 128, T, v.n_rbox, v.max_ebox);
+  const bool stage = false;
+  const size_t smem = check_smem_layout(v.nsp_pad, 128, T, v.n_rbox, v.max_ebox, stage);
   constexpr bool BB = EZO_BOX_TU != 0;
   EZO_DISPATCH_NDOF(v.n, EZO_DISPATCH_T_WIDE(T, {
     auto kern = k_round_bisect<ND, TT, BB>;
     err = set_smem(kern, smem);
     if (err != cudaSuccess) return err;
-    kern<<<resident_grid(kern, 128, smem, grid), 128, smem, s>>>(v, v.max_obs_pad);
+    kern<<<resident_grid(kern, 128, smem, grid), 128, smem, s>>>(v, stage ? 1 : 0);
   }));
   return cudaGetLastError();
 }

@@ -587,38 +587,59 @@ __device__ __forceinline__ void round_close_block(const BatchView& v) {
 }
 
 // ------------------------------------------------------- collision checks --
-// Shared memory of the collision kernels: robot spheres, obstacles, per group
-// sphere centres, obstacle offsets, then the boxes (robot boxes in their
-// frames, obstacle boxes, per group robot boxes in the world; 4 float4 each).
-__host__ __device__ inline size_t check_smem_layout(int nsp, int nobs, int threads, int T, int nrbox = 0,
-                                                    int nebox = 0) {
+// The documented acceptance rule of the collision entry points, in bytes per
+// 128-thread block: robot spheres, obstacles, sphere centres per group of T
+// lanes, boxes. The kernels' own need (check_smem_layout) is smaller.
+__host__ __device__ inline size_t check_smem_rule(int nsp, int nobs, int threads, int T, int nrbox = 0,
+                                                  int nebox = 0) {
   const int groups = threads / T;
   return (size_t)(nsp + nobs + groups * (nsp + 1)) * sizeof(float4) + (size_t)nobs * sizeof(float) +
          (size_t)4 * (nrbox + nebox + groups * nrbox) * sizeof(float4);
 }
 
+// Shared memory of the collision kernels: robot spheres, per group sphere
+// centres, then the boxes (robot boxes in their frames, obstacle boxes, per
+// group robot boxes in the world; 4 float4 each), then the coarse bounds of
+// the obstacle grid when the kernel stages them.
+__host__ __device__ inline size_t check_smem_layout(int nsp, int threads, int T, int nrbox, int nebox, bool stage_lb) {
+  const int groups = threads / T;
+  return (size_t)(nsp + groups * (nsp + 1)) * sizeof(float4) +
+         (size_t)4 * (nrbox + nebox + groups * nrbox) * sizeof(float4) + (stage_lb ? (size_t)kGridLbBytes : 0);
+}
+
 struct GeomSmem {
   float4* sph;
-  float4* obs;
   float4* cen_all;
-  float* nhw;
   float4* rbox_l;
   float4* ebox;
   float4* rbox_w_all;
+  uint8_t* lb;
 };
 
-// nobs is a multiple of 8, so the box arrays after the obstacle offsets stay
-// 16-byte aligned
-__device__ __forceinline__ GeomSmem carve_geom(float4* base, int nsp, int nobs, int groups, int nrbox, int nebox) {
+__device__ __forceinline__ GeomSmem carve_geom(float4* base, int nsp, int groups, int nrbox, int nebox) {
   GeomSmem g;
   g.sph = base;
-  g.obs = g.sph + nsp;
-  g.cen_all = g.obs + nobs;
-  g.nhw = reinterpret_cast<float*>(g.cen_all + groups * (nsp + 1));
-  g.rbox_l = reinterpret_cast<float4*>(g.nhw + nobs);
+  g.cen_all = g.sph + nsp;
+  g.rbox_l = g.cen_all + groups * (nsp + 1);
   g.ebox = g.rbox_l + 4 * nrbox;
   g.rbox_w_all = g.ebox + 4 * nebox;
+  g.lb = reinterpret_cast<uint8_t*>(g.rbox_w_all + groups * 4 * nrbox);
   return g;
+}
+
+// The coarse bounds of an obstacle set's grid into shared memory.
+__device__ __forceinline__ void stage_grid(uint8_t* lb_s, const EnvDev& e) {
+  const uint4* src = reinterpret_cast<const uint4*>(e.grid.lb);
+  uint4* dst = reinterpret_cast<uint4*>(lb_s);
+  if (e.n_obs > 0)
+    for (int i = threadIdx.x; i < kGridLbBytes / 16; i += blockDim.x) dst[i] = __ldg(src + i);
+}
+
+// Whether a launch over N configurations at T lanes each looks up enough
+// bounds per resident block to pay for copying them to shared memory.
+inline bool stage_grid_pays(int nsp, const EnvDev& e, long long N, int T) {
+  const long long blocks = std::min<long long>((N * T + 127) / 128, 152 * 4);
+  return e.n_obs > 0 && N * nsp >= blocks * 4096;
 }
 
 __device__ __forceinline__ BoxCtx box_ctx(const GeomSmem& g, const RobotDev* robot, int nrbox, int n_ebox, int gi) {

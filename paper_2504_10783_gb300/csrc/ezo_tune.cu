@@ -114,11 +114,11 @@ extern "C" __attribute__((visibility("hidden"))) int ezo_internal_tuned_lanes(co
       const int T = lanes[li];
       if (!fits(T)) continue;
       // one warm-up launch, then the best of three
-      if (launch_check_flat(rd, n, nsp, nrbox, ef.e, ef.E, q, M, M, flags, T, sms * 32, s) != cudaSuccess) continue;
+      if (launch_check_flat(rd, n, nsp, nrbox, ef.e, q, M, M, flags, T, sms * 32, s) != cudaSuccess) continue;
       float t_best = 1e30f;
       for (int rep = 0; rep < 3; ++rep) {
         cudaEventRecord(e0, s);
-        launch_check_flat(rd, n, nsp, nrbox, ef.e, ef.E, q, M, M, flags, T, sms * 32, s);
+        launch_check_flat(rd, n, nsp, nrbox, ef.e, q, M, M, flags, T, sms * 32, s);
         cudaEventRecord(e1, s);
         cudaEventSynchronize(e1);
         float ms = 0.f;
