@@ -109,14 +109,13 @@ struct ezo_env {
 
 // The robot spheres on the fixed base frame sit where they are for every
 // configuration, so their pairs with a static obstacle set need no test per
-// configuration when every such pair is clear. The sweep then starts at the
-// first whole chunk of EZO_CH spheres past them; the clearance is checked in
+// configuration when every such pair is clear. The tests then start past
+// them; the clearance is checked in
 // FP64 on the FP32 values the kernels use, against 1e-4 m, far above the
 // rounding band of the FP32 test (the kernels place a base sphere exactly at
 // its FP32 local coordinates), so every label is what the full sweep gives.
 // Any base sphere within 1e-4 m of an obstacle keeps the full sweep.
-static int sweep_first(const ezo_robot* r, const ezo_env* e) {
-  const int cut = (r->n_base / EZO_CH) * EZO_CH;
+static int sweep_first(const ezo_robot* r, const ezo_env* e, int cut) {
   if (cut == 0) return 0;
   for (int s = 0; s < cut; ++s) {
     const float4 l = r->host.sph[s];
@@ -130,8 +129,112 @@ static int sweep_first(const ezo_robot* r, const ezo_env* e) {
 
 EnvDev ezo_env::dev_for(const ezo_robot* r) const {
   EnvDev d = dev();
-  d.s_first = sweep_first(r, this);
+  d.s_first = sweep_first(r, this, r->n_base);
   return d;
+}
+
+// collide_lane's plan of a robot (LaneRobot): the self pairs (i, j), i < j in
+// sorted order, as links: per sphere j the runs of its partners i on one
+// frame, and consecutive spheres of a frame with the same runs together.
+static void plan_lane(RobotDev& h, const std::vector<std::pair<int, int>>& pairs, bool ok, double reach) {
+  LaneRobot& L = h.lane;
+  L = LaneRobot{};
+  const int ns = h.n_spheres, n = h.n;
+  for (int f = 0; f <= n; ++f) {
+    int axis = 0;
+    for (int a = 3; a >= 1 && !axis; --a) {
+      bool on = true;
+      for (int s = h.frame_first[f]; s < h.frame_first[f + 1]; ++s) {
+        const float c[3] = {h.sph[s].x, h.sph[s].y, h.sph[s].z};
+        for (int k = 0; k < 3; ++k) on = on && (k == a - 1 || c[k] == 0.f);
+      }
+      if (on) axis = a;
+    }
+    L.axis[f] = axis;
+    L.slot[f] = -1;
+    for (int s = h.frame_first[f]; s < h.frame_first[f + 1]; ++s) L.frame[s] = f;
+    if (h.frame_first[f + 1] > h.frame_first[f]) {
+      L.slot[f] = L.n_slot++;
+      L.last = f;
+      if (!axis) L.general = 1;
+    }
+  }
+  std::vector<std::vector<std::pair<int, int>>> runs(ns);  // per sphere j: (first, count)
+  {
+    std::vector<std::vector<int>> partners(ns);
+    for (const auto& p : pairs) {
+      if (L.frame[p.first] >= L.frame[p.second]) return;  // on one frame: collide_group takes them
+      partners[p.second].push_back(p.first);
+    }
+    for (int j = 0; j < ns; ++j) {
+      auto& P = partners[j];
+      std::sort(P.begin(), P.end());
+      for (size_t a = 0; a < P.size();) {
+        size_t b = a + 1;
+        while (b < P.size() && P[b] == P[b - 1] + 1 && L.frame[P[b]] == L.frame[P[a]]) ++b;
+        runs[j].emplace_back(P[a], (int)(b - a));
+        a = b;
+      }
+    }
+  }
+  // the segment between a run's two farthest centres, and how far its spheres
+  // reach from it
+  auto capsule = [&](int s0, int cnt, float (&p)[3], float (&u)[3]) {
+    auto at = [&](int i, int k) { return (double)(k == 0 ? h.sph[i].x : (k == 1 ? h.sph[i].y : h.sph[i].z)); };
+    int e0 = s0, e1 = s0;
+    double far = 0.0;
+    for (int i = s0; i < s0 + cnt; ++i)
+      for (int j = i; j < s0 + cnt; ++j) {
+        double d2 = 0.0;
+        for (int k = 0; k < 3; ++k) d2 += (at(i, k) - at(j, k)) * (at(i, k) - at(j, k));
+        if (d2 > far) far = d2, e0 = i, e1 = j;
+      }
+    for (int k = 0; k < 3; ++k) p[k] = (float)at(e0, k), u[k] = (float)(at(e1, k) - at(e0, k));
+    double rad = 0.0;
+    for (int i = s0; i < s0 + cnt; ++i) {
+      double t = 0.0, d2 = 0.0;
+      for (int k = 0; k < 3; ++k) t += (at(i, k) - p[k]) * (double)u[k];
+      t = far > 0.0 ? std::min(1.0, std::max(0.0, t / far)) : 0.0;
+      for (int k = 0; k < 3; ++k) d2 += std::pow(at(i, k) - p[k] - t * (double)u[k], 2.0);
+      rad = std::max(rad, std::sqrt(d2) + (double)h.sph[i].w);
+    }
+    return rad;
+  };
+  for (int j = 0; j < ns && ok;) {
+    int e = j + 1;
+    while (e < ns && L.frame[e] == L.frame[j] && runs[e] == runs[j]) ++e;
+    for (const auto& run : runs[j]) {
+      if (L.n_link == kLinkPairs) return;
+      LinkPair& P = L.link[L.n_link++];
+      P.fa = (short)L.frame[run.first], P.fb = (short)L.frame[j];
+      P.a0 = (short)run.first, P.na = (short)run.second;
+      P.b0 = (short)j, P.nb = (short)(e - j);
+      double R = capsule(P.a0, P.na, P.pa, P.ua) + capsule(P.b0, P.nb, P.pb, P.ub);
+      auto len2 = [](const float (&u)[3]) { return (double)u[0] * u[0] + (double)u[1] * u[1] + (double)u[2] * u[2]; };
+      if (len2(P.ua) < len2(P.ub)) {  // b the shorter
+        std::swap(P.fa, P.fb), std::swap(P.a0, P.b0), std::swap(P.na, P.nb);
+        std::swap(P.pa, P.pb), std::swap(P.ua, P.ub);
+      }
+      P.inv = len2(P.ua) > 0.0 ? (float)(1.0 / len2(P.ua)) : 0.f;
+      for (int k = 0; k < 3; ++k) P.mb[k] = P.pb[k] + 0.5f * P.ub[k];
+      // the segments' ends are FP32 kinematics, their distance FP32
+      // arithmetic on coordinates up to the reach
+      const double slack = 1e-5 * (4.0 * reach * reach + R * R), M = R + 0.5 * std::sqrt(len2(P.ub));
+      P.r2 = (float)(R * R * (1.0 + 1e-4) + slack);
+      P.m2 = (float)(M * M * (1.0 + 1e-4) + slack);
+    }
+    j = e;
+  }
+  L.ok = ok;
+}
+
+// LaneRobot's slots and generality as the launchers take them (lane_smem_layout),
+// -1 where collide_lane does not apply: boxes, self pairs it cannot order,
+// spheres as large as the grid's edge.
+static int lane_code(const ezo_robot* r, const ezo_env* e) {
+  const LaneRobot& l = r->host.lane;
+  if (!l.ok || r->n_box || e->n_box || (e->n_obs > 0 && !(r->r_max < e->grid.r_out))) return -1;
+  return 2 * l.n_slot + l.general;
 }
 
 extern "C" {
@@ -306,6 +409,7 @@ ezo_status ezo_robot_create(int32_t n, const double* a, const double* alpha, con
     } else {
       h.n_sblk = 0;
     }
+    plan_lane(h, ok ? norm : std::vector<std::pair<int, int>>(), ok || norm.empty(), chain + loc_max);
     const double a2 = 2.0 * (chain + loc_max), b2 = 2.0 * r->r_max;
     h.E_self = (float)(8.0 * kU32 * (a2 * a2 + b2 * b2));
   }
@@ -454,10 +558,13 @@ ezo_status ezo_env_create(int32_t n_obs, const double* xyzr, ezo_env** out) {
     g.ey = kGridBias + (float)(gb.sub * gb.n[1]);
     g.ez = kGridBias + (float)(gb.sub * gb.n[2]);
     g.fbits = gb.sub == 2 ? 6 : 5;
+    g.r_out = (float)(0.99 * pad);
     g.tx = kGridBias + (float)(gb.n[0] - 1);
     g.ty = kGridBias + (float)(gb.n[1] - 1);
     g.tz = kGridBias + (float)(gb.n[2] - 1);
-    if ((err = launch_grid_build(gb, nullptr)) != cudaSuccess ||
+    // cells past the grid's last one an axis are outside: free (r_out)
+    if ((err = cudaMemsetAsync(gb.lb, 255, kGridLbBytes, nullptr)) != cudaSuccess ||
+        (err = launch_grid_build(gb, nullptr)) != cudaSuccess ||
         (err = cudaStreamSynchronize(nullptr)) != cudaSuccess) {
       ezo_env_free(e);
       return cuda_fail(err, "ezo_env_create: grid");
@@ -591,7 +698,7 @@ ezo_status ezo_check_collision(const ezo_robot* robot, const ezo_env* env, const
   if (check_smem_bytes(robot->nsp_pad, env->n_obs_pad, 128, lanes, robot->n_box, env->n_box) > kSmemBudget)
     return fail(EZO_ERR_INVALID_ARG,
                 "ezo_check_collision: robot and obstacle spheres exceed shared memory at this lanes_per_config");
-  cudaError_t e = launch_check_flat(robot->d_robot, robot->n, robot->nsp_pad, robot->n_box, env->dev_for(robot), q_dev, ldq, N,
+  cudaError_t e = launch_check_flat(robot->d_robot, robot->n, robot->nsp_pad, robot->n_box, lane_code(robot, env), env->dev_for(robot), q_dev, ldq, N,
                                     flags_dev, lanes, sm_count() * 32, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "ezo_check_collision");
   g_err.clear();
@@ -671,6 +778,10 @@ __attribute__((visibility("hidden"))) int ezo_internal_env_dev(const ezo_robot* 
   return 0;
 }
 
+__attribute__((visibility("hidden"))) int ezo_internal_lane(const ezo_robot* r, const ezo_env* e) {
+  return lane_code(r, e);
+}
+
 __attribute__((visibility("hidden"))) void ezo_internal_set_error(const char* msg) { g_err = msg ? msg : ""; }
 
 __attribute__((visibility("hidden"))) int ezo_internal_robot_prismatic(const ezo_robot* r) {
@@ -690,7 +801,7 @@ double ezo_check_flops(const ezo_robot* robot, const ezo_env* env) {
 }
 
 int32_t ezo_check_static_spheres(const ezo_robot* robot, const ezo_env* env) {
-  return (robot && env) ? sweep_first(robot, env) : 0;
+  return (robot && env) ? sweep_first(robot, env, (robot->n_base / EZO_CH) * EZO_CH) : 0;
 }
 
 // ------------------------------------------------------------------ batch --
@@ -1308,6 +1419,11 @@ ezo_status ezo_batch_create(const ezo_robot* robot, int32_t n_env, const ezo_env
   v.max_obs_pad = b->max_obs_pad;
   v.max_ebox = b->max_ebox;
   v.n_rbox = robot->n_box;
+  v.lane = 0;
+  for (int e2 = 0; e2 < n_env; ++e2) {
+    const int w = lane_code(robot, envs[e2]);
+    v.lane = w < 0 || v.lane < 0 ? -1 : w;
+  }
   v.nsp_pad = robot->nsp_pad;
   v.np_max = b->np_max;
   v.path_first = b->d_path_first;
@@ -1320,25 +1436,23 @@ ezo_status ezo_batch_create(const ezo_robot* robot, int32_t n_env, const ezo_env
     tot_np += s.n_p;
     tot_s1 += std::max(s.n_p, host_test_size(1, prm->eps, prm->delta, prm->tau));
   }
-  // lanes per configuration from the autotuner, at the first round's sample
+  // lanes per configuration, the autotuner's picks at the first round's sample
   // count (labels) and at a quarter of the candidate capacity (bisection)
   int e_big = 0;
   for (int e2 = 1; e2 < n_env; ++e2)
     if (envs[e2]->n_obs > envs[e_big]->n_obs) e_big = e2;
-  // the tuner times one flat launch of the round-1 size, but the round
-  // kernel's work units and the smaller later rounds favour two lanes per
-  // configuration below ~1e6 samples per round (1e5 samples per round, whole
-  // inflation: 0.22 ms at 2 lanes, 0.28 at 1, 0.24 at 4, while the flat
-  // tuner ranks them within its noise); larger rounds take the tuner's pick
-  b->T_check = tot_s1 < (1ll << 20) ? 2 : ezo_internal_tuned_lanes(robot, envs[e_big], tot_s1, nullptr);
-  // Bisection runs N_b dependent checks per candidate on the few thousand
-  // candidates of a round, so it is latency bound: sixteen lanes per
-  // candidate (the wide check; eight in scenes with boxes), unless a round
-  // can hold enough candidates to fill the GPU at fewer lanes. Measured on
-  // the 7-DOF arm's path (800 to 14,000 candidates a round), 16 lanes beat 8
-  // by 5-30% in every round but the largest.
-  b->T_bisect = tot_np >= (1ll << 20) ? ezo_internal_tuned_lanes(robot, envs[e_big], tot_np / 4, nullptr)
-                                      : ((robot->n_box || b->max_ebox) ? 8 : 16);
+  if (v.lane >= 0) {
+    b->T_check = lane_check_lanes(tot_s1);
+    b->T_bisect = lane_bisect_lanes(tot_np);
+  } else {
+    // collide_group: two lanes per label below ~1e6 samples a round (whole
+    // inflations ran faster than at the flat tuner's pick there), and for the
+    // N_b dependent checks of a candidate sixteen (eight in scenes with
+    // boxes), unless a round can hold enough candidates to fill the GPU
+    b->T_check = tot_s1 < (1ll << 20) ? 2 : ezo_internal_tuned_lanes(robot, envs[e_big], tot_s1, nullptr);
+    b->T_bisect = tot_np >= (1ll << 20) ? ezo_internal_tuned_lanes(robot, envs[e_big], tot_np / 4, nullptr)
+                                        : ((robot->n_box || b->max_ebox) ? 8 : 16);
+  }
   b->T_check = std::max(b->T_check, b->t_min);
   b->T_bisect = std::max(b->T_bisect, b->t_min);
   // walks share eight lanes in rounds with fewer walks than one warp per
@@ -1999,7 +2113,7 @@ ezo_status ezo_check_path(const ezo_robot* robot, const ezo_env* env, const doub
   if (e == cudaSuccess) e = cudaMemsetAsync(d_edge, 0, (size_t)K, s);
   if (e == cudaSuccess) {
     const int lanes = ezo_internal_tuned_lanes(robot, env, N, s);
-    e = launch_check_path(robot->d_robot, n, robot->nsp_pad, robot->n_box, env->dev_for(robot), d_verts, K, d_off, N,
+    e = launch_check_path(robot->d_robot, n, robot->nsp_pad, robot->n_box, lane_code(robot, env), env->dev_for(robot), d_verts, K, d_off, N,
                           point_flags_dev, d_edge, lanes, sm_count() * 32, s);
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(edge_flags, d_edge, (size_t)K, cudaMemcpyDeviceToHost, s);

@@ -85,6 +85,31 @@ __device__ __forceinline__ float u01_co(uint32_t x) { return (float)(x >> 8) * 5
 __device__ __forceinline__ float u01_oc(uint32_t x) { return (float)((x >> 8) + 1u) * 5.9604644775390625e-8f; }
 
 // ------------------------------------------------------------------ robot --
+// The robot as collide_lane walks it. axis[f] = 1, 2, 3 when every sphere of
+// frame f lies on its x, y or z axis, else 0; slot[f] numbers the frames with
+// spheres (-1: none), whose poses a group of lanes keeps: the axis and the
+// origin, or three axes and the origin where some frame is general. The chain
+// is walked to frame `last`, the last with spheres. The self pairs are a list
+// of links, runs of spheres on one frame each (a0, na on frame fa; b0, nb on
+// fb), every sphere of one against every sphere of the other, each run with
+// the segment p + t u through it (in its frame): axes of two capsules whose
+// radii together are sqrt(r2), so links whose segments are farther apart than
+// that have no colliding pair; nor have those where the middle mb of the
+// shorter segment b is farther than sqrt(m2), r2's root and half of b, from
+// segment a (inv = 1/|ua|^2).
+constexpr int kLinkPairs = 32;
+struct LinkPair {
+  short fa, fb, a0, na, b0, nb;
+  float r2, m2, inv;
+  float pa[3], ua[3], pb[3], ub[3], mb[3];
+};
+struct LaneRobot {
+  int ok, n_link, n_slot, general, last;
+  int axis[EZO_MAX_DOF + 2], slot[EZO_MAX_DOF + 2];
+  LinkPair link[kLinkPairs];
+  int frame[EZO_MAX_SPHERES];  // of each sorted sphere
+};
+
 // Device image of a robot: DH chain plus spheres sorted by the frame they are
 // attached to. Lives in global memory; kernels stage the small part in smem.
 struct RobotDev {
@@ -116,6 +141,7 @@ struct RobotDev {
   int n_sbp, n_bbp;
   const ushort2* sb_pairs;  // (sorted sphere, sorted box)
   const ushort2* bb_pairs;  // (sorted box, sorted box)
+  LaneRobot lane;
 };
 
 // The chain and the spheres in FP64 as given at creation (spheres sorted as
@@ -209,6 +235,7 @@ struct ObsGrid {
   float tx, ty, tz;  // 2^23 + last coarse cell
   float ex, ey, ez;  // 2^23 + fine cells
   int fbits;         // log2 of the fine cells' row stride: 5 or 6
+  float r_out;       // a smaller sphere whose centre lies outside the grid is free
 };
 
 // Obstacle set in global memory: (x, y, z, R), padded to a multiple of EZO_CH.
@@ -218,7 +245,7 @@ struct EnvDev {
   int n_obs_pad;
   const float4* box;  // obstacle boxes, 4 float4 each: (centre, h_x), (axis 0, h_y), (axis 1, h_z), (axis 2, 0)
   int n_box;
-  // first robot sphere of the obstacle tests (a multiple of EZO_CH): the
+  // first robot sphere of the obstacle tests: the
   // spheres before it sit on the fixed base frame, so their pairs with these
   // obstacles are the same for every configuration, and they were found
   // clear of every obstacle by more than any rounding band when the pair
@@ -481,13 +508,25 @@ __device__ __forceinline__ bool cell_hit(const EnvDev& e, float cx, float cy, fl
     if (__fmaf_ru(r, g.inv_step, kGridBias) < __uint_as_float(0x4B000000u | (unsigned)(d & 0xffu))) return false;
   }
   const unsigned kind = (unsigned)(d >> 8) & 0xffu;
-  const bool list = kind == kGridList, all = kind == kGridAll;
-  const int cnt = list ? (int)((d >> 16) & 0xffffu) : (all ? e.n_obs : (int)kind);
+  if (kind <= kGridInline) {
+    // the word's one to four ids, their obstacles loaded together
+    unsigned id[kGridInline];
+    bool hit = false;
+#pragma unroll
+    for (unsigned k = 0; k < kGridInline; ++k)
+      id[k] = (k < kind ? (unsigned)(d >> (16 + 12 * k)) : (unsigned)(d >> 16)) & 0xfffu;
+    float4 o[kGridInline];
+#pragma unroll
+    for (unsigned k = 0; k < kGridInline; ++k) o[k] = __ldg(e.obs + id[k]);
+#pragma unroll
+    for (unsigned k = 0; k < kGridInline; ++k) hit = pair_hit(cx, cy, cz, r, o[k]) || hit;
+    return hit;
+  }
+  const bool list = kind == kGridList;
+  const int cnt = list ? (int)((d >> 16) & 0xffffu) : e.n_obs;
   const uint16_t* ids = g.ids + (list ? (unsigned)(d >> 32) : 0u);
-  unsigned long long in_ids = d >> 16;
   for (int k = 0; k < cnt; ++k) {
-    const unsigned id = list ? (unsigned)__ldg(ids + k) : (all ? (unsigned)k : (unsigned)(in_ids & 0xfffu));
-    in_ids >>= 12;
+    const unsigned id = list ? (unsigned)__ldg(ids + k) : (unsigned)k;
     if (pair_hit(cx, cy, cz, r, __ldg(e.obs + id))) return true;
   }
   return false;
@@ -534,6 +573,425 @@ __device__ __forceinline__ bool obstacles_hit(const RobotSmem& rs, const float4*
       }
     }
     if (hit) break;
+  }
+  return hit;
+}
+
+// ---------------------------------------- spheres formed in registers --
+// The robot in shared memory for collide_lane, followed by the spheres
+// (float4), per sphere (coordinate along its frame's axis, ceil(r / step) for
+// the obstacle set's grid) and frame, the grid's coarse bounds when staged,
+// and per group of lanes its words.
+struct LaneSmem {
+  float4 joint[2 * EZO_MAX_DOF];  // (ca, sa, a, d), (toff, kth, kd, 0)
+  int frame_first[EZO_MAX_DOF + 2], axis[EZO_MAX_DOF + 2], slot[EZO_MAX_DOF + 2];
+  int n, n_spheres, last, n_link, general;
+  LinkPair link[kLinkPairs];
+};
+
+// Floats of a group: one lane keeps the joint values and each pose's numbers
+// at the block's stride; more lanes keep poses as float4s (origin, axis[, two
+// columns]), an odd number of them, so that the groups of a warp read
+// different banks.
+__host__ __device__ inline int lane_group_words(int n, int n_slot, int general, int T) {
+  if (T == 1) return n + n_slot * (general ? 12 : 6);
+  return 4 * ((n_slot * (general ? 4 : 2)) | 1);
+}
+
+__device__ __forceinline__ void stage_lane_robot(LaneSmem& ls, float4* sph, int* frame,
+                                                 const RobotDev* __restrict__ rd) {
+  const LaneRobot& lr = rd->lane;
+  for (int i = threadIdx.x; i < EZO_MAX_DOF; i += blockDim.x) {
+    ls.joint[2 * i] = make_float4(rd->ca[i], rd->sa[i], rd->a[i], rd->d[i]);
+    ls.joint[2 * i + 1] = make_float4(rd->toff[i], rd->kth[i], rd->kd[i], 0.f);
+  }
+  for (int i = threadIdx.x; i < EZO_MAX_DOF + 2; i += blockDim.x) {
+    ls.frame_first[i] = rd->frame_first[i];
+    ls.axis[i] = lr.axis[i];
+    ls.slot[i] = lr.slot[i];
+  }
+  for (int i = threadIdx.x; i < lr.n_link * (int)(sizeof(LinkPair) / 4); i += blockDim.x)
+    reinterpret_cast<int*>(ls.link)[i] = reinterpret_cast<const int*>(lr.link)[i];
+  if (threadIdx.x == 0) {
+    ls.n = rd->n;
+    ls.n_spheres = rd->n_spheres;
+    ls.last = lr.last;
+    ls.n_link = lr.n_link;
+    ls.general = lr.general;
+  }
+  for (int i = threadIdx.x; i < rd->n_spheres; i += blockDim.x) {
+    sph[i] = rd->sph[i];
+    frame[i] = lr.frame[i];
+  }
+}
+
+// (coordinate on the axis, ceil(r / step)) of every sphere; a sphere before
+// s_first, or any when there are no obstacles, gets -1: free whatever the bound
+__device__ __forceinline__ void stage_lane_env(float2* sa, const RobotDev* __restrict__ rd, const EnvDev& e) {
+  for (int i = threadIdx.x; i < rd->n_spheres; i += blockDim.x) {
+    const float4 l = rd->sph[i];
+    const int axis = rd->lane.axis[rd->lane.frame[i]];
+    const int q = e.n_obs == 0 || i < e.s_first ? -1 : (int)fminf(ceilf(__fmul_ru(l.w, e.grid.inv_step)), 1.0e6f);
+    sa[i] = make_float2(axis == 1 ? l.x : (axis == 2 ? l.y : l.z), __int_as_float(q));
+  }
+}
+
+// A frame's pose as collide_lane uses it: origin p, the axis v its spheres lie
+// on, and for a general frame the other two columns.
+struct LanePose {
+  float px, py, pz, vx, vy, vz;
+  float ax, ay, az, bx, by, bz;  // columns 0 and 1 (axis 0 only; v is column 2 then)
+};
+
+// Centre of a sphere: one multiply-add a coordinate on an axis (the other two
+// products of fk_group's chain are exact zeros there), its whole chain else.
+__device__ __forceinline__ void lane_centre(const LanePose& P, int axis, float la, const float4* __restrict__ l,
+                                            float& cx, float& cy, float& cz) {
+  cx = fmaf(P.vx, la, P.px);
+  cy = fmaf(P.vy, la, P.py);
+  cz = fmaf(P.vz, la, P.pz);
+  if (axis == 0) {
+    const float lx = l->x, ly = l->y;
+    cx = fmaf(P.ax, lx, fmaf(P.bx, ly, cx));
+    cy = fmaf(P.ay, lx, fmaf(P.by, ly, cy));
+    cz = fmaf(P.az, lx, fmaf(P.bz, ly, cz));
+  }
+}
+
+// Keeps and reads the pose of slot k (lane_group_words).
+template <int T>
+__device__ __forceinline__ void lane_keep(const LanePose& P, int k, int general, float* mine, int stride) {
+  if (T == 1) {
+    float* o = mine + k * (general ? 12 : 6) * stride;
+    o[0] = P.px, o[stride] = P.py, o[2 * stride] = P.pz;
+    o[3 * stride] = P.vx, o[4 * stride] = P.vy, o[5 * stride] = P.vz;
+    if (general) {
+      o[6 * stride] = P.ax, o[7 * stride] = P.ay, o[8 * stride] = P.az;
+      o[9 * stride] = P.bx, o[10 * stride] = P.by, o[11 * stride] = P.bz;
+    }
+  } else {
+    float4* o = reinterpret_cast<float4*>(mine) + k * (general ? 4 : 2);
+    o[0] = make_float4(P.px, P.py, P.pz, 0.f);
+    o[1] = make_float4(P.vx, P.vy, P.vz, 0.f);
+    if (general) {
+      o[2] = make_float4(P.ax, P.ay, P.az, 0.f);
+      o[3] = make_float4(P.bx, P.by, P.bz, 0.f);
+    }
+  }
+}
+template <int T>
+__device__ __forceinline__ LanePose lane_pose(int k, int general, const float* mine, int stride) {
+  LanePose P;
+  P.ax = P.ay = P.az = P.bx = P.by = P.bz = 0.f;
+  if (T == 1) {
+    const float* o = mine + k * (general ? 12 : 6) * stride;
+    P.px = o[0], P.py = o[stride], P.pz = o[2 * stride];
+    P.vx = o[3 * stride], P.vy = o[4 * stride], P.vz = o[5 * stride];
+    if (general) {
+      P.ax = o[6 * stride], P.ay = o[7 * stride], P.az = o[8 * stride];
+      P.bx = o[9 * stride], P.by = o[10 * stride], P.bz = o[11 * stride];
+    }
+  } else {
+    const float4* o = reinterpret_cast<const float4*>(mine) + k * (general ? 4 : 2);
+    const float4 p = o[0], v = o[1];
+    P.px = p.x, P.py = p.y, P.pz = p.z;
+    P.vx = v.x, P.vy = v.y, P.vz = v.z;
+    if (general) {
+      const float4 a = o[2], b = o[3];
+      P.ax = a.x, P.ay = a.y, P.az = a.z;
+      P.bx = b.x, P.by = b.y, P.bz = b.z;
+    }
+  }
+  return P;
+}
+
+// The next frame of the chain (fk_group's operations, in its order).
+struct LaneChain {
+  float c0x, c0y, c0z, c1x, c1y, c1z, c2x, c2y, c2z, px, py, pz;
+  __device__ __forceinline__ void start() {
+    c0x = 1.f, c0y = 0.f, c0z = 0.f, c1x = 0.f, c1y = 1.f, c1z = 0.f, c2x = 0.f, c2y = 0.f, c2z = 1.f;
+    px = py = pz = 0.f;
+  }
+  __device__ __forceinline__ void step(float4 J, float4 K, float qj, float s, float c) {
+    const float n0x = fmaf(c, c0x, s * c1x), n0y = fmaf(c, c0y, s * c1y), n0z = fmaf(c, c0z, s * c1z);
+    const float n1x = fmaf(c, c1x, -s * c0x), n1y = fmaf(c, c1y, -s * c0y), n1z = fmaf(c, c1z, -s * c0z);
+    const float aj = J.z, dj = fmaf(qj, K.z, J.w);
+    px = fmaf(aj, n0x, fmaf(dj, c2x, px));
+    py = fmaf(aj, n0y, fmaf(dj, c2y, py));
+    pz = fmaf(aj, n0z, fmaf(dj, c2z, pz));
+    const float ca = J.x, sn = J.y;
+    const float m1x = fmaf(ca, n1x, sn * c2x), m1y = fmaf(ca, n1y, sn * c2y), m1z = fmaf(ca, n1z, sn * c2z);
+    const float m2x = fmaf(ca, c2x, -sn * n1x), m2y = fmaf(ca, c2y, -sn * n1y), m2z = fmaf(ca, c2z, -sn * n1z);
+    c0x = n0x, c0y = n0y, c0z = n0z;
+    c1x = m1x, c1y = m1y, c1z = m1z;
+    c2x = m2x, c2y = m2y, c2z = m2z;
+  }
+  __device__ __forceinline__ LanePose pose(int axis) const {
+    LanePose P;
+    P.px = px, P.py = py, P.pz = pz;
+    P.vx = axis == 1 ? c0x : (axis == 2 ? c1x : c2x);
+    P.vy = axis == 1 ? c0y : (axis == 2 ? c1y : c2y);
+    P.vz = axis == 1 ? c0z : (axis == 2 ? c1z : c2z);
+    P.ax = c0x, P.ay = c0y, P.az = c0z, P.bx = c1x, P.by = c1y, P.bz = c1z;
+    return P;
+  }
+};
+
+// Whether the coarse bound leaves a sphere (centre c, q = ceil(r / step)) to
+// be tested: its centre in the grid and its radius not below the bound.
+__device__ __forceinline__ bool lane_near(const ObsGrid& g, const uint8_t* __restrict__ lb, float cx, float cy,
+                                          float cz, int q) {
+  const unsigned ix = __float_as_uint(__fmaf_rd(cx, g.inv, g.bx)), iy = __float_as_uint(__fmaf_rd(cy, g.inv, g.by)),
+                 iz = __float_as_uint(__fmaf_rd(cz, g.inv, g.bz));
+  // all three in [2^23, 2^23 + 32): no bit but the low five differs from 2^23's
+  const unsigned off = (ix ^ 0x4B000000u) | (iy ^ 0x4B000000u) | (iz ^ 0x4B000000u);
+  return off < (unsigned)kGridC && q >= (int)lb[((iz * kGridC + iy) * kGridC + ix) & (kGridLbBytes - 1)];
+}
+
+// Point or vector (w = 1 or 0 for the origin) of a run's segment in the world.
+__device__ __forceinline__ void lane_world(const LanePose& P, int axis, const float (&l)[3], float w, float& x,
+                                           float& y, float& z) {
+  const float a = axis == 1 ? l[0] : (axis == 2 ? l[1] : l[2]);
+  x = fmaf(P.vx, a, w * P.px);
+  y = fmaf(P.vy, a, w * P.py);
+  z = fmaf(P.vz, a, w * P.pz);
+  if (axis == 0) {
+    x = fmaf(P.ax, l[0], fmaf(P.bx, l[1], x));
+    y = fmaf(P.ay, l[0], fmaf(P.by, l[1], y));
+    z = fmaf(P.az, l[0], fmaf(P.bz, l[1], z));
+  }
+}
+
+// The self pairs from the kept poses, links lg, lg + T, ..: the squared
+// distance of the two segments (any point pair on them bounds it from above,
+// and the pair found is the nearest to second order in its rounding, which
+// r2's margin covers); the pairs of links nearer than their radii one by one.
+template <int T>
+__device__ __forceinline__ bool links_hit(const LaneSmem& ls, const float4* __restrict__ sph,
+                                          const float2* __restrict__ sa, const float* mine, int stride, int lg) {
+  const int general = ls.general;
+#pragma unroll 1
+  for (int i = lg; i < ls.n_link; i += T) {
+    const LinkPair& L = ls.link[i];
+    const LanePose A = lane_pose<T>(ls.slot[L.fa], general, mine, stride),
+                   B = lane_pose<T>(ls.slot[L.fb], general, mine, stride);
+    const int xa = ls.axis[L.fa], xb = ls.axis[L.fb];
+    float px, py, pz, ux, uy, uz, qx, qy, qz, vx, vy, vz;
+    lane_world(A, xa, L.pa, 1.f, px, py, pz);
+    lane_world(A, xa, L.ua, 0.f, ux, uy, uz);
+    {
+      // the middle of b against segment a: leaves one link in two hundred of
+      // the 7-DOF arm at a third of the whole test's work
+      float mx, my, mz;
+      lane_world(B, xb, L.mb, 1.f, mx, my, mz);
+      mx -= px, my -= py, mz -= pz;
+      const float t = __saturatef(fmaf(mx, ux, fmaf(my, uy, mz * uz)) * L.inv);
+      mx = fmaf(-t, ux, mx), my = fmaf(-t, uy, my), mz = fmaf(-t, uz, mz);
+      if (!(fmaf(mx, mx, fmaf(my, my, mz * mz)) < L.m2)) continue;
+    }
+    lane_world(B, xb, L.pb, 1.f, qx, qy, qz);
+    lane_world(B, xb, L.ub, 0.f, vx, vy, vz);
+    const float rx = px - qx, ry = py - qy, rz = pz - qz;
+    const float uu = fmaf(ux, ux, fmaf(uy, uy, uz * uz)), vv = fmaf(vx, vx, fmaf(vy, vy, vz * vz));
+    const float uv = fmaf(ux, vx, fmaf(uy, vy, uz * vz));
+    const float ur = fmaf(ux, rx, fmaf(uy, ry, uz * rz)), vr = fmaf(vx, rx, fmaf(vy, ry, vz * rz));
+    const float det = fmaf(uu, vv, -uv * uv);
+    // s on the first segment for the nearest points of the two lines (0 when
+    // they are parallel), t the nearest on the second to it, then s to t
+    const float iu = uu > 0.f ? __fdividef(1.f, uu) : 0.f, iv = vv > 0.f ? __fdividef(1.f, vv) : 0.f;
+    float s = det > 1e-6f * uu * vv ? __saturatef(__fdividef(fmaf(uv, vr, -ur * vv), det)) : 0.f;
+    const float t = __saturatef(fmaf(s, uv, vr) * iv);
+    s = __saturatef(fmaf(t, uv, -ur) * iu);
+    const float dx = rx + fmaf(s, ux, -t * vx), dy = ry + fmaf(s, uy, -t * vy), dz = rz + fmaf(s, uz, -t * vz);
+    if (!(fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < L.r2)) continue;
+    for (int j = L.b0; j < L.b0 + L.nb; ++j) {
+      const float4 lj = sph[j];
+      float cx, cy, cz;
+      lane_centre(B, xb, sa[j].x, sph + j, cx, cy, cz);
+      for (int k = L.a0; k < L.a0 + L.na; ++k) {
+        float ox, oy, oz;
+        lane_centre(A, xa, sa[k].x, sph + k, ox, oy, oz);
+        if (pair_hit(cx, cy, cz, lj.w, make_float4(ox, oy, oz, sph[k].w))) return true;
+      }
+    }
+  }
+  return false;
+}
+
+// A warp's queue of spheres to test against their cells: the lanes put in
+// those that the coarse bound did not free, and 32 at a time are tested, one
+// a lane, from their owner's kept pose. Few spheres are left (0.7 of 29 a
+// configuration among 64 obstacles), in a few lanes at a time, so each lane
+// going through its own cost six passes a warp where this takes one.
+// mine, stride: this lane's poses (lane_pose), a group's pitch for T > 1.
+constexpr int kNearQueue = 64;  // entries of a warp: sphere | lane << 16
+template <int T>
+struct NearQueue {
+  int* q;
+  int count;
+  // Tests the first 32 entries; true for a lane one of whose spheres hit.
+  __device__ __forceinline__ bool test(const LaneSmem& ls, const float4* __restrict__ sph,
+                                       const float2* __restrict__ sa, const int* __restrict__ frame, const EnvDev& e,
+                                       const float* mine, int stride) {
+    __syncwarp();
+    const int lane = threadIdx.x & 31;
+    unsigned owner = 0u;
+    if (lane < count) {
+      const int w = q[lane], s = w & 0xffff, o = w >> 16, f = frame[s];
+      const float* theirs = T == 1 ? mine + (o - lane) : mine + (o / T - lane / T) * stride;
+      const LanePose P = lane_pose<T>(ls.slot[f], ls.general, theirs, stride);
+      float cx, cy, cz;
+      lane_centre(P, ls.axis[f], sa[s].x, sph + s, cx, cy, cz);
+      if (cell_hit(e, cx, cy, cz, sph[s].w)) owner = 1u << o;
+    }
+    owner = __reduce_or_sync(0xffffffffu, owner);
+    const int left = max(0, count - 32);
+    int w = 0;
+    if (lane < left) w = q[32 + lane];
+    __syncwarp();
+    if (lane < left) q[lane] = w;
+    count = left;
+    return (owner >> lane) & 1u;
+  }
+  // Adds sphere s of this lane (put = false: none); the warp's lanes together.
+  __device__ __forceinline__ void add(bool put, int s) {
+    const int lane = threadIdx.x & 31;
+    const unsigned m = __ballot_sync(0xffffffffu, put);
+    if (put) q[count + __popc(m & ((1u << lane) - 1u))] = s | (lane << 16);
+    count += __popc(m);
+  }
+};
+
+// One configuration by a group of T lanes of one warp (T in 1..32). A
+// sphere's centre is formed in registers from its frame's pose, looked up in
+// the obstacle grid, and formed again where it is needed; only the poses of
+// the frames with spheres are stored (collide_group keeps every centre in
+// shared memory, which held it to 12 warps an SM), and the self pairs are
+// screened link against link. The spheres that a coarse bound does not free go
+// through the warp's queue.
+// One lane (T = 1): the chain is one rolled loop over the frames, with the
+// joint values in mine[j * stride] (unrolled, half the time went to waiting
+// for instructions), each frame's spheres taken as it is reached. More lanes:
+// every lane walks the unrolled chain (the group shares the sines and
+// cosines), lane 0 writes the poses, and the spheres of all frames are dealt
+// to the lanes; the rolled form was a quarter slower there, where few warps
+// hide its latency.
+// Needs the robot's largest sphere to be smaller than the grid's edge: a
+// centre outside the grid is then free. All lanes of the warp call it
+// together; returns the group-wide OR.
+// Measured at one lane, 7-DOF arm of 40 spheres (kernel time, collide_group at
+// its best lane count before): 2e6 labels among 64 obstacles 0.53 -> 0.179 ms,
+// of which the chain takes 0.05, the 29 lookups 0.04, the spheres left to
+// test 0.03, the links 0.03; 2e5 labels among 1024 obstacles 0.077 -> 0.039
+// ms. Bound by instruction issue (73%), 20 warps an SM.
+template <int NDOF, int T>
+__device__ __forceinline__ bool collide_lane(const float (&q)[NDOF], const LaneSmem& ls,
+                                             const float4* __restrict__ sph, const float2* __restrict__ sa,
+                                             const int* __restrict__ frame, const EnvDev& e,
+                                             const uint8_t* __restrict__ lb, float* mine, int stride, int lg,
+                                             int* queue) {
+  const ObsGrid& g = e.grid;
+  const int last = ls.last, general = ls.general;
+  bool hit = false;
+  NearQueue<T> nq{queue, 0};
+  LaneChain C;
+  C.start();
+  if constexpr (T == 1) {
+    float* poses = mine + ls.n * stride;
+#pragma unroll
+    for (int j = 0; j < NDOF; ++j)
+      if (j < ls.n) mine[j * stride] = q[j];
+#pragma unroll 1
+    for (int f = 0; f <= last; ++f) {
+      if (f > 0) {
+        const float4 J = ls.joint[2 * f - 2], K = ls.joint[2 * f - 1];
+        const float qj = mine[(f - 1) * stride];
+        float s, c;
+        sincosf(fmaf(qj, K.y, K.x), &s, &c);
+        C.step(J, K, qj, s, c);
+      }
+      const int s_end = ls.frame_first[f + 1];
+      if (ls.slot[f] < 0) continue;
+      const int axis = ls.axis[f];
+      const LanePose P = C.pose(axis);
+      lane_keep<1>(P, ls.slot[f], general, poses, stride);
+      // the base frame's spheres before s_first have nothing left to test
+#pragma unroll 1
+      for (int s0 = f == 0 ? max(ls.frame_first[0], e.s_first) : ls.frame_first[f]; s0 < s_end; s0 += 32) {
+        unsigned near = 0u, bit = 1u;
+        const int cnt = min(32, s_end - s0);
+#pragma unroll 4
+        for (int k = 0; k < cnt; ++k, bit += bit) {
+          const float2 a = sa[s0 + k];
+          float cx, cy, cz;
+          lane_centre(P, axis, a.x, sph + s0 + k, cx, cy, cz);
+          if (lane_near(g, lb, cx, cy, cz, __float_as_int(a.y))) near |= bit;
+        }
+        if (hit) near = 0u;
+        while (__any_sync(0xffffffffu, near != 0u)) {
+          const bool put = near != 0u;
+          nq.add(put, s0 + __ffs(near) - 1);
+          near &= near - 1u;
+          if (nq.count >= 32 && nq.test(ls, sph, sa, frame, e, poses, stride)) hit = true;
+        }
+      }
+    }
+    if (nq.count && nq.test(ls, sph, sa, frame, e, poses, stride)) hit = true;
+    if (!hit) hit = links_hit<1>(ls, sph, sa, poses, stride, 0);
+  } else {
+    constexpr int JPL = (NDOF + T - 1) / T;
+    float ms[JPL], mc[JPL];
+#pragma unroll
+    for (int k = 0; k < JPL; ++k) {
+      const int jm = lg + k * T;
+      float ang = 0.f;
+#pragma unroll
+      for (int j = 0; j < NDOF; ++j)
+        if (j == jm && j < last) ang = fmaf(q[j], ls.joint[2 * j + 1].y, ls.joint[2 * j + 1].x);
+      sincosf(ang, &ms[k], &mc[k]);
+    }
+#pragma unroll
+    for (int f = 0; f <= NDOF; ++f) {
+      if (f > last) break;
+      if (f > 0) {
+        const int j = f - 1;
+        const float s = __shfl_sync(0xffffffffu, ms[j / T], j % T, T), c = __shfl_sync(0xffffffffu, mc[j / T], j % T, T);
+        C.step(ls.joint[2 * j], ls.joint[2 * j + 1], q[j], s, c);
+      }
+      if (ls.slot[f] >= 0 && lg == 0) lane_keep<T>(C.pose(ls.axis[f]), ls.slot[f], general, mine, stride);
+    }
+    __syncwarp();
+    const int ns = ls.n_spheres;
+#pragma unroll 1
+    for (int s1 = e.s_first; s1 < ns; s1 += 32 * T) {
+      const int s0 = s1 + lg;
+      unsigned near = 0u;
+#pragma unroll 2
+      for (int k = 0; k < 32; ++k) {
+        const int s = s0 + k * T;
+        if (s >= ns) break;
+        const int f = frame[s];
+        const LanePose P = lane_pose<T>(ls.slot[f], general, mine, stride);
+        const float2 a = sa[s];
+        float cx, cy, cz;
+        lane_centre(P, ls.axis[f], a.x, sph + s, cx, cy, cz);
+        if (lane_near(g, lb, cx, cy, cz, __float_as_int(a.y))) near |= 1u << k;
+      }
+      if (hit) near = 0u;
+      while (__any_sync(0xffffffffu, near != 0u)) {
+        const bool put = near != 0u;
+        nq.add(put, s0 + (__ffs(near) - 1) * T);
+        near &= near - 1u;
+        if (nq.count >= 32 && nq.test(ls, sph, sa, frame, e, mine, stride)) hit = true;
+      }
+    }
+    if (nq.count && nq.test(ls, sph, sa, frame, e, mine, stride)) hit = true;
+    if (!hit) hit = links_hit<T>(ls, sph, sa, mine, stride, lg);
+    unsigned h = hit ? 1u : 0u;
+#pragma unroll
+    for (int off = 1; off < T; off <<= 1) h |= __shfl_xor_sync(0xffffffffu, h, off, T);
+    hit = h != 0u;
+    __syncwarp();  // the group's poses may be overwritten
   }
   return hit;
 }

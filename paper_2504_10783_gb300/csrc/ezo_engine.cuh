@@ -137,10 +137,13 @@ struct BatchView {
   int* q_claim;      // [1 + q_claim_cap]: launch count, then the epoch that claimed each work unit
   int q_claim_cap;   // work units of the largest launch
   int n_sm;          // SMs of the device
+  int lane;          // collide_lane's layout code, -1: not for this batch
 };
 
-// Launchers (ezo_kernels.cu). T = lanes per configuration.
-cudaError_t launch_check_flat(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env,
+// Launchers. T = lanes per configuration; lane: collide_lane's layout code, -1
+// when the robot or the obstacle set does not admit it.
+cudaError_t launch_check_flat(const RobotDev* robot, int n, int nsp_pad, int n_rbox, int lane,
+                              const EnvDev& env,
                               const float* q, long long ldq, long long N, uint8_t* flags, int T, int grid_cap,
                               cudaStream_t s);
 // signed distance, exact below cap (3e38: exact everywhere)
@@ -189,7 +192,8 @@ cudaError_t launch_wave_select(const BatchView& v, const uint8_t* contained, int
 // round end fused with the next round's sizing (the run loops' last kernel)
 cudaError_t launch_round_close(const BatchView& v, cudaStream_t s);
 // recovery (Sec. VI-B)
-cudaError_t launch_check_path(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env,
+cudaError_t launch_check_path(const RobotDev* robot, int n, int nsp_pad, int n_rbox, int lane,
+                              const EnvDev& env,
                               const double* verts, int n_edges, const long long* off, long long N,
                               uint8_t* point_flags, uint8_t* edge_flags, int T, int grid_cap, cudaStream_t s);
 cudaError_t launch_coverage(const BatchView& v, uint8_t* covered, double tol, cudaStream_t s);
@@ -222,6 +226,16 @@ struct GridBuild {
 };
 cudaError_t launch_grid_build(const GridBuild& g, cudaStream_t s);
 size_t check_smem_bytes(int n_spheres_pad, int n_obs_pad, int threads, int T, int n_rbox = 0, int n_ebox = 0);
+// Lanes per configuration of a round's labels and bisection by collide_lane,
+// from the samples and candidates of a round. Labels are bound by throughput:
+// one lane repeats no kinematics (1e5 samples: 0.028 ms a round at one lane,
+// 0.033 at two, 0.036 at four, 0.047 at eight) unless that leaves schedulers
+// without a warp. A candidate's N_b checks depend on one another: eight lanes
+// are fastest at the few thousand candidates of a path's round (0.054 ms;
+// 0.060 at four and sixteen), four where a round holds hundreds of thousands
+// (24 paths: 3.0 ms; 3.2 at eight, 3.6 at one).
+inline int lane_check_lanes(long long samples) { return samples >= (1ll << 16) ? 1 : (samples >= (1ll << 14) ? 2 : 4); }
+inline int lane_bisect_lanes(long long candidates) { return candidates >= (1ll << 20) ? 4 : 8; }
 // Dynamic shared memory a collision kernel may request: the opt-in maximum
 // per block (227 KB) less the static robot image and a margin. The sphere
 // centres take (spheres + 1) x 16 bytes per group of lanes, so more lanes per

@@ -31,35 +31,25 @@ __global__ void __launch_bounds__(128) k_sample_flat(const double* __restrict__ 
 
 #endif  // !EZO_BOX_TU
 
-template <int NDOF, int T, bool BOX>
-__global__ void __launch_bounds__(128) k_check_flat(const RobotDev* __restrict__ robot, EnvDev env, int stage_lb,
-                                                    const float* __restrict__ q, long long ldq, long long N,
-                                                    uint8_t* __restrict__ flags) {
+template <int NDOF, int T, bool BOX, bool LANE>
+__global__ void __launch_bounds__(LANE ? 256 : 128) k_check_flat(const RobotDev* __restrict__ robot, EnvDev env,
+                                                                 int stage_lb, const float* __restrict__ q,
+                                                                 long long ldq, long long N,
+                                                                 uint8_t* __restrict__ flags) {
   extern __shared__ float4 smem4[];
-  __shared__ RobotSmem rs;
-  const int nsp = robot->n_spheres_pad, nrbox = robot->n_box;
-  const int groups = blockDim.x / T;
-  const GeomSmem gs = carve_geom(smem4, nsp, groups, nrbox, env.n_box);
-  float4* sph_s = gs.sph;
-  stage_robot(rs, sph_s, robot);
-  stage_robot_boxes(gs.rbox_l, robot);
-  stage_env_boxes(gs.ebox, env);
-  if (stage_lb) stage_grid(gs.lb, env);
-  const uint8_t* lb = stage_lb ? gs.lb : env.grid.lb;
+  __shared__ typename CheckRobot<LANE>::type rs;
+  Checker<NDOF, T, BOX, LANE> chk(rs, smem4, robot, env.n_box, stage_lb);
+  chk.set_env(env);
   __syncthreads();
-  const int gi = threadIdx.x / T, lg = threadIdx.x % T;
-  float4* cen = gs.cen_all + gi * (nsp + 1);
-  const BoxCtx bx = box_ctx(gs, robot, nrbox, env.n_box, gi);
-  const ushort2* sp = robot->self_pairs;
-  const float* srr = robot->self_rr;
+  const int groups = blockDim.x / T, gi = threadIdx.x / T;
   for (long long base = (long long)blockIdx.x * groups; base < N; base += (long long)gridDim.x * groups) {
     const long long i = base + gi;
     const long long ic = i < N ? i : N - 1;
     float qq[NDOF];
 #pragma unroll
     for (int j = 0; j < NDOF; ++j) qq[j] = (j < rs.n) ? q[j * ldq + ic] : 0.f;
-    const bool hit = collide_group<NDOF, T, BOX>(qq, rs, sph_s, env, lb, sp, srr, cen, lg, bx);
-    if (i < N && lg == 0) flags[i] = hit ? 1 : 0;
+    const bool hit = chk(qq);
+    if (i < N && chk.lg == 0) flags[i] = hit ? 1 : 0;
   }
 }
 
@@ -194,45 +184,39 @@ cudaError_t launch_check_flat_box(const RobotDev* robot, int n, int nsp_pad, int
   const long long groups = threads / T;
   long long grid = (N + groups - 1) / groups;
   if (grid_cap > 0 && grid > grid_cap) grid = grid_cap;
-  // the coarse bounds go to shared memory when a block looks up enough of
-  // them to pay for the copy and they fit beside the sphere centres
-  const bool stage = stage_grid_pays(nsp_pad, env, N, T) &&
-                     check_smem_layout(nsp_pad, threads, T, n_rbox, env.n_box, true) <= kSmemBudget;
-  const size_t smem = check_smem_layout(nsp_pad, threads, T, n_rbox, env.n_box, stage);
-  constexpr bool BB = EZO_BOX_TU != 0;
+  const CheckPlan pl =
+      check_plan(nsp_pad, n, threads, T, n_rbox, env.n_box, -1, stage_grid_pays(nsp_pad, env, N, T));
   EZO_DISPATCH_NDOF(n, EZO_DISPATCH_T(T, {
-    auto kern = k_check_flat<ND, TT, BB>;
-    err = set_smem(kern, smem);
+    auto kern = k_check_flat<ND, TT, true, false>;
+    err = set_smem(kern, pl.smem);
     if (err != cudaSuccess) return err;
-    const int blocks = resident_grid(kern, threads, smem, (int)std::min<long long>(grid, 1 << 20));
-    kern<<<blocks, threads, smem, s>>>(robot, env, stage ? 1 : 0, q, ldq, N, flags);
+    const int blocks = resident_grid(kern, threads, pl.smem, (int)std::min<long long>(grid, 1 << 20));
+    kern<<<blocks, threads, pl.smem, s>>>(robot, env, pl.stage ? 1 : 0, q, ldq, N, flags);
   }));
   return cudaGetLastError();
 }
 #else
-cudaError_t launch_check_flat(const RobotDev* robot, int n, int nsp_pad, int n_rbox, const EnvDev& env,
+cudaError_t launch_check_flat(const RobotDev* robot, int n, int nsp_pad, int n_rbox, int lane,
+                              const EnvDev& env,
                               const float* q, long long ldq, long long N, uint8_t* flags, int T, int grid_cap,
                               cudaStream_t s) {
   if (n_rbox || env.n_box) return launch_check_flat_box(robot, n, nsp_pad, n_rbox, env, q, ldq, N, flags, T, grid_cap, s);
   if (N <= 0) return cudaSuccess;
   cudaError_t err = cudaSuccess;
-  const int threads = 128;
+  // 256 threads where a block shares the staged bounds and has work for them
+  const int threads = lane >= 0 && N * T >= 256ll * 152 ? 256 : 128;
   const long long groups = threads / T;
   long long grid = (N + groups - 1) / groups;
   if (grid_cap > 0 && grid > grid_cap) grid = grid_cap;
-  // the coarse bounds go to shared memory when a block looks up enough of
-  // them to pay for the copy and they fit beside the sphere centres
-  const bool stage = stage_grid_pays(nsp_pad, env, N, T) &&
-                     check_smem_layout(nsp_pad, threads, T, n_rbox, env.n_box, true) <= kSmemBudget;
-  const size_t smem = check_smem_layout(nsp_pad, threads, T, n_rbox, env.n_box, stage);
-  constexpr bool BB = EZO_BOX_TU != 0;
-  EZO_DISPATCH_NDOF(n, EZO_DISPATCH_T(T, {
-    auto kern = k_check_flat<ND, TT, BB>;
-    err = set_smem(kern, smem);
+  const CheckPlan pl =
+      check_plan(nsp_pad, n, threads, T, n_rbox, env.n_box, lane, stage_grid_pays(nsp_pad, env, N, T));
+  EZO_DISPATCH_NDOF(n, EZO_DISPATCH_T(T, EZO_DISPATCH_LANE(pl.lane, {
+    auto kern = k_check_flat<ND, TT, false, LL>;
+    err = set_smem(kern, pl.smem);
     if (err != cudaSuccess) return err;
-    const int blocks = resident_grid(kern, threads, smem, (int)std::min<long long>(grid, 1 << 20));
-    kern<<<blocks, threads, smem, s>>>(robot, env, stage ? 1 : 0, q, ldq, N, flags);
-  }));
+    const int blocks = resident_grid(kern, threads, pl.smem, (int)std::min<long long>(grid, 1 << 20));
+    kern<<<blocks, threads, pl.smem, s>>>(robot, env, pl.stage ? 1 : 0, q, ldq, N, flags);
+  })));
   return cudaGetLastError();
 }
 #endif

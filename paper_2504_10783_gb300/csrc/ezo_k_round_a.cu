@@ -144,11 +144,10 @@ __global__ void __launch_bounds__(128, NDOF <= 7 ? (SPLIT ? 5 : 7) : 4)
 
 #endif  // !EZO_BOX_TU
 
-template <int NDOF, int T, bool BOX>
+template <int NDOF, int T, bool BOX, bool LANE>
 __global__ void __launch_bounds__(128) k_round_check(BatchView v, int stage_lb) {
   extern __shared__ float4 smem4[];
-  __shared__ RobotSmem rs;
-  __shared__ int cur_env;
+  __shared__ typename CheckRobot<LANE>::type rs;
   const int n_tiles = v.summary->n_sample_tiles;
   constexpr int PASSES = kTile / (128 / T);
   // work units are (tile, pass), taken from the round's work queue; a block
@@ -160,44 +159,29 @@ __global__ void __launch_bounds__(128) k_round_check(BatchView v, int stage_lb) 
     queue_leave(v, q, &v.summary->left_check, units);
     return;
   }
-  const RobotDev* robot = v.robot;
-  const int nsp = robot->n_spheres_pad, nrbox = robot->n_box;
-  const int groups = blockDim.x / T;
-  const GeomSmem gs = carve_geom(smem4, nsp, groups, nrbox, v.max_ebox);
-  float4* sph_s = gs.sph;
-  stage_robot(rs, sph_s, robot);
-  stage_robot_boxes(gs.rbox_l, robot);
-  if (threadIdx.x == 0) cur_env = -1;
-  __syncthreads();
-  const int gi = threadIdx.x / T, lg = threadIdx.x % T;
-  float4* cen = gs.cen_all + gi * (nsp + 1);
+  Checker<NDOF, T, BOX, LANE> chk(rs, smem4, v.robot, v.max_ebox, stage_lb);
+  int cur_env = -1;  // the same in every thread
+  const int groups = blockDim.x / T, gi = threadIdx.x / T;
   for (; u < units; u = queue_take(v, q, units)) {
     const int2 tile = v.sample_tiles[u / PASSES];
     const int sub = (u % PASSES) * groups;
     const SegState& st = v.st[tile.x];
-    const EnvDevFull& ef = v.envs[st.env];
     if (st.env != cur_env) {
       __syncthreads();
-      if (stage_lb) stage_grid(gs.lb, ef.e);
-      stage_env_boxes(gs.ebox, ef.e);
-      if (threadIdx.x == 0) cur_env = st.env;
+      chk.set_env(v.envs[st.env].e);
+      cur_env = st.env;
       __syncthreads();
     }
-    const BoxCtx bx = box_ctx(gs, robot, nrbox, ef.e.n_box, gi);
     const float* S = v.S + (long long)v.n * st.sample_off;
     uint8_t* fl = v.flags + st.sample_off;
-    {
-      const int i = tile.y + sub + gi;
-      const bool valid = i < st.n_samples;
-      const int ic = valid ? i : tile.y;
-      float qq[NDOF];
+    const int i = tile.y + sub + gi;
+    const bool valid = i < st.n_samples;
+    const int ic = valid ? i : tile.y;
+    float qq[NDOF];
 #pragma unroll
-      for (int j = 0; j < NDOF; ++j) qq[j] = (j < v.n) ? S[(long long)j * st.s_cap + ic] : 0.f;
-      const EnvDev env = ef.e;
-      const bool hit = collide_group<NDOF, T, BOX>(qq, rs, sph_s, env, stage_lb ? gs.lb : env.grid.lb,
-                                                   robot->self_pairs, robot->self_rr, cen, lg, bx);
-      if (valid && lg == 0) fl[i] = hit ? 1 : 0;
-    }
+    for (int j = 0; j < NDOF; ++j) qq[j] = (j < v.n) ? S[(long long)j * st.s_cap + ic] : 0.f;
+    const bool hit = chk(qq);
+    if (valid && chk.lg == 0) fl[i] = hit ? 1 : 0;
   }
   queue_leave(v, q, &v.summary->left_check, units);
 }
@@ -357,14 +341,12 @@ cudaError_t launch_round_sample(const BatchView& v, int split_below_tiles, int g
 #if EZO_BOX_TU
 cudaError_t launch_round_check_box(const BatchView& v, int T, int grid, cudaStream_t s) {
   cudaError_t err = cudaSuccess;
-  const bool stage = check_smem_layout(v.nsp_pad, 128, T, v.n_rbox, v.max_ebox, true) <= kSmemBudget;
-  const size_t smem = check_smem_layout(v.nsp_pad, 128, T, v.n_rbox, v.max_ebox, stage);
-  constexpr bool BB = EZO_BOX_TU != 0;
+  const CheckPlan pl = check_plan(v.nsp_pad, v.n, 128, T, v.n_rbox, v.max_ebox, -1, true);
   EZO_DISPATCH_NDOF(v.n, EZO_DISPATCH_T(T, {
-    auto kern = k_round_check<ND, TT, BB>;
-    err = set_smem(kern, smem);
+    auto kern = k_round_check<ND, TT, true, false>;
+    err = set_smem(kern, pl.smem);
     if (err != cudaSuccess) return err;
-    kern<<<resident_grid(kern, 128, smem, grid), 128, smem, s>>>(v, stage ? 1 : 0);
+    kern<<<resident_grid(kern, 128, pl.smem, grid), 128, pl.smem, s>>>(v, pl.stage ? 1 : 0);
   }));
   return cudaGetLastError();
 }
@@ -372,15 +354,13 @@ cudaError_t launch_round_check_box(const BatchView& v, int T, int grid, cudaStre
 cudaError_t launch_round_check(const BatchView& v, int T, int grid, cudaStream_t s) {
   if (v.n_rbox || v.max_ebox) return launch_round_check_box(v, T, grid, s);
   cudaError_t err = cudaSuccess;
-  const bool stage = check_smem_layout(v.nsp_pad, 128, T, v.n_rbox, v.max_ebox, true) <= kSmemBudget;
-  const size_t smem = check_smem_layout(v.nsp_pad, 128, T, v.n_rbox, v.max_ebox, stage);
-  constexpr bool BB = EZO_BOX_TU != 0;
-  EZO_DISPATCH_NDOF(v.n, EZO_DISPATCH_T(T, {
-    auto kern = k_round_check<ND, TT, BB>;
-    err = set_smem(kern, smem);
+  const CheckPlan pl = check_plan(v.nsp_pad, v.n, 128, T, v.n_rbox, v.max_ebox, v.lane, true);
+  EZO_DISPATCH_NDOF(v.n, EZO_DISPATCH_T(T, EZO_DISPATCH_LANE(pl.lane, {
+    auto kern = k_round_check<ND, TT, false, LL>;
+    err = set_smem(kern, pl.smem);
     if (err != cudaSuccess) return err;
-    kern<<<resident_grid(kern, 128, smem, grid), 128, smem, s>>>(v, stage ? 1 : 0);
-  }));
+    kern<<<resident_grid(kern, 128, pl.smem, grid), 128, pl.smem, s>>>(v, pl.stage ? 1 : 0);
+  })));
   return cudaGetLastError();
 }
 #endif

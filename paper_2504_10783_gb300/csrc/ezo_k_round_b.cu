@@ -167,12 +167,11 @@ __global__ void __launch_bounds__(kRowBlock) k_bisect_finish(BatchView v) {
 // bis_mode 1 instead checks the surrogate's end point once (s_ok records the
 // outcome), and bis_mode 2 redoes the exact halvings for the candidates whose
 // surrogate end point was free.
-template <int NDOF, int T, bool BOX>
+template <int NDOF, int T, bool BOX, bool LANE>
 __global__ void __launch_bounds__(128) k_round_bisect(BatchView v, int stage_lb) {
   extern __shared__ float4 smem4[];
-  __shared__ RobotSmem rs;
-  __shared__ int cur_env;
-  const int n_tiles = v.summary->n_bisect_tiles;
+  __shared__ typename CheckRobot<LANE>::type rs;
+    const int n_tiles = v.summary->n_bisect_tiles;
   // work units are (tile, pass), taken from this mode's work queue; a block
   // that finds none leaves before staging anything
   int* q = &v.summary->q_bisect[v.bis_mode];
@@ -183,17 +182,9 @@ __global__ void __launch_bounds__(128) k_round_bisect(BatchView v, int stage_lb)
     queue_leave(v, q, left, units);
     return;
   }
-  const RobotDev* robot = v.robot;
-  const int nsp = robot->n_spheres_pad, nrbox = robot->n_box;
-  const int groups = blockDim.x / T;
-  const GeomSmem gs = carve_geom(smem4, nsp, groups, nrbox, v.max_ebox);
-  float4* sph_s = gs.sph;
-  stage_robot(rs, sph_s, robot);
-  stage_robot_boxes(gs.rbox_l, robot);
-  if (threadIdx.x == 0) cur_env = -1;
-  __syncthreads();
-  const int gi = threadIdx.x / T, lg = threadIdx.x % T;
-  float4* cen = gs.cen_all + gi * (nsp + 1);
+  Checker<NDOF, T, BOX, LANE> chk(rs, smem4, v.robot, v.max_ebox, stage_lb);
+  int cur_env = -1;  // the same in every thread
+  const int groups = blockDim.x / T, gi = threadIdx.x / T, lg = chk.lg;
   const int ld = v.s_ld;
   const float scale = ldexpf(1.f, -v.n_b);
   static_assert(kTile % (128 / T) == 0, "tile must be a whole number of passes");
@@ -202,19 +193,12 @@ __global__ void __launch_bounds__(128) k_round_bisect(BatchView v, int stage_lb)
     const int sub = (u % T) * groups;
     const int g = tile.x;
     const SegState& st = v.st[g];
-    const EnvDevFull& ef = v.envs[st.env];
     if (st.env != cur_env) {
       __syncthreads();
-      if (stage_lb) stage_grid(gs.lb, ef.e);
-      stage_env_boxes(gs.ebox, ef.e);
-      if (threadIdx.x == 0) cur_env = st.env;
+      chk.set_env(v.envs[st.env].e);
+      cur_env = st.env;
       __syncthreads();
     }
-    const BoxCtx bx = box_ctx(gs, robot, nrbox, ef.e.n_box, gi);
-    const EnvDev env = ef.e;  // in registers for the N_b checks
-    const uint8_t* lb = stage_lb ? gs.lb : env.grid.lb;
-    const ushort2* self_pairs = robot->self_pairs;
-    const float* self_rr = robot->self_rr;
     const int c = tile.y + sub + gi;
     const int row = (u / T) * kTile + sub + gi;
     bool valid = c < st.n_cand;
@@ -247,7 +231,7 @@ __global__ void __launch_bounds__(128) k_round_bisect(BatchView v, int stage_lb)
       float qq[NDOF];
 #pragma unroll
       for (int j = 0; j < NDOF; ++j) qq[j] = fmaf(f, dv32[j], p32[j]);
-      const bool hit = collide_group<NDOF, T, BOX>(qq, rs, sph_s, env, lb, self_pairs, self_rr, cen, lg, bx);
+      const bool hit = chk(qq);
       if (v.bis_mode == 1) {
         if (valid && lg == 0) {
           v.s_ok[row] = hit ? 1 : 0;
@@ -275,10 +259,11 @@ __global__ void __launch_bounds__(128) k_round_bisect(BatchView v, int stage_lb)
 // exactly as the two halvings would take them, so the record and the end
 // point are the sequential halvings' bit for bit. Half the dependent checks
 // for half again the checks; an odd last halving is warp 1's alone.
-template <int NDOF>
+template <int NDOF, bool LANE>
 __global__ void __launch_bounds__(96) k_round_bisect_pair(BatchView v) {
   extern __shared__ float4 smem4[];
-  __shared__ RobotSmem rs;
+  __shared__ typename CheckRobot<LANE>::type rs;
+  __shared__ int cur_env;
   __shared__ int s_hit[3];
   const int n_tiles = v.summary->n_bisect_tiles;
   int* q = &v.summary->q_bisect[v.bis_mode];
@@ -289,15 +274,10 @@ __global__ void __launch_bounds__(96) k_round_bisect_pair(BatchView v) {
     queue_leave(v, q, left, units);
     return;
   }
-  const RobotDev* robot = v.robot;
-  const int nsp = robot->n_spheres_pad;
-  const GeomSmem gs = carve_geom(smem4, nsp, 3, 0, 0);
-  float4* sph_s = gs.sph;
-  stage_robot(rs, sph_s, robot);
+  Checker<NDOF, 32, false, LANE> chk(rs, smem4, v.robot, 0, false);
+  if (threadIdx.x == 0) cur_env = -1;
   __syncthreads();
-  const int w = threadIdx.x >> 5, lg = threadIdx.x & 31;
-  float4* cen = gs.cen_all + w * (nsp + 1);
-  const BoxCtx bx{};
+  const int w = threadIdx.x >> 5, lg = chk.lg;
   const int ld = v.s_ld;
   const int nb = v.n_b;
   const float scale = ldexpf(1.f, -nb);
@@ -306,10 +286,12 @@ __global__ void __launch_bounds__(96) k_round_bisect_pair(BatchView v) {
     const int c = tile.y + u % kTile;
     const int g = tile.x;
     const SegState& st = v.st[g];
-    const EnvDevFull& ef = v.envs[st.env];
-    const EnvDev env = ef.e;
-    const ushort2* self_pairs = robot->self_pairs;
-    const float* self_rr = robot->self_rr;
+    if (st.env != cur_env) {
+      __syncthreads();
+      chk.set_env(v.envs[st.env].e);
+      if (threadIdx.x == 0) cur_env = st.env;
+      __syncthreads();
+    }
     bool valid = c < st.n_cand;
     if (v.bis_mode == 2) valid = valid && !v.s_ok[u];
     if (!valid) continue;  // the whole block: u is the block's
@@ -334,8 +316,7 @@ __global__ void __launch_bounds__(96) k_round_bisect_pair(BatchView v) {
         float qq[NDOF];
 #pragma unroll
         for (int j = 0; j < NDOF; ++j) qq[j] = fmaf(f, dv32[j], p32[j]);
-        const bool hit =
-            collide_group<NDOF, 32>(qq, rs, sph_s, env, env.grid.lb, self_pairs, self_rr, cen, lg, bx);
+        const bool hit = chk(qq);
         if (lg == 0) s_hit[w] = hit ? 1 : 0;
       }
       __syncthreads();
@@ -755,14 +736,12 @@ __global__ void k_wave_select(BatchView v, const uint8_t* __restrict__ contained
 #if EZO_BOX_TU
 cudaError_t launch_round_bisect_box(const BatchView& v, int T, int grid, cudaStream_t s) {
   cudaError_t err = cudaSuccess;
-  const bool stage = false;
-  const size_t smem = check_smem_layout(v.nsp_pad, 128, T, v.n_rbox, v.max_ebox, stage);
-  constexpr bool BB = EZO_BOX_TU != 0;
+  const CheckPlan pl = check_plan(v.nsp_pad, v.n, 128, T, v.n_rbox, v.max_ebox, -1, false);
   EZO_DISPATCH_NDOF(v.n, EZO_DISPATCH_T(T, {
-    auto kern = k_round_bisect<ND, TT, BB>;
-    err = set_smem(kern, smem);
+    auto kern = k_round_bisect<ND, TT, true, false>;
+    err = set_smem(kern, pl.smem);
     if (err != cudaSuccess) return err;
-    kern<<<resident_grid(kern, 128, smem, grid), 128, smem, s>>>(v, stage ? 1 : 0);
+    kern<<<resident_grid(kern, 128, pl.smem, grid), 128, pl.smem, s>>>(v, pl.stage ? 1 : 0);
   }));
   return cudaGetLastError();
 }
@@ -774,25 +753,23 @@ cudaError_t launch_round_bisect(const BatchView& v, int T, int grid, cudaStream_
   if (T == kBisectPairLanes && v.bis_mode == 1) T = 32;  // one check per candidate: the 32-lane kernel
   if (T == kBisectPairLanes) {
     cudaError_t err = cudaSuccess;
-    const size_t smem = check_smem_layout(v.nsp_pad, 96, 32, 0, 0, false);
-    EZO_DISPATCH_NDOF(v.n, {
-      auto kern = k_round_bisect_pair<ND>;
-      err = set_smem(kern, smem);
+    const CheckPlan pl = check_plan(v.nsp_pad, v.n, 96, 32, 0, 0, v.lane, false);
+    EZO_DISPATCH_NDOF(v.n, EZO_DISPATCH_LANE(pl.lane, {
+      auto kern = k_round_bisect_pair<ND, LL>;
+      err = set_smem(kern, pl.smem);
       if (err != cudaSuccess) return err;
-      kern<<<resident_grid(kern, 96, smem, std::max(grid, 1) * 4), 96, smem, s>>>(v);
-    });
+      kern<<<resident_grid(kern, 96, pl.smem, std::max(grid, 1) * 4), 96, pl.smem, s>>>(v);
+    }));
     return cudaGetLastError();
   }
   cudaError_t err = cudaSuccess;
-  const bool stage = false;
-  const size_t smem = check_smem_layout(v.nsp_pad, 128, T, v.n_rbox, v.max_ebox, stage);
-  constexpr bool BB = EZO_BOX_TU != 0;
-  EZO_DISPATCH_NDOF(v.n, EZO_DISPATCH_T_WIDE(T, {
-    auto kern = k_round_bisect<ND, TT, BB>;
-    err = set_smem(kern, smem);
+  const CheckPlan pl = check_plan(v.nsp_pad, v.n, 128, T, v.n_rbox, v.max_ebox, v.lane, false);
+  EZO_DISPATCH_NDOF(v.n, EZO_DISPATCH_T_WIDE(T, EZO_DISPATCH_LANE(pl.lane, {
+    auto kern = k_round_bisect<ND, TT, false, LL>;
+    err = set_smem(kern, pl.smem);
     if (err != cudaSuccess) return err;
-    kern<<<resident_grid(kern, 128, smem, grid), 128, smem, s>>>(v, stage ? 1 : 0);
-  }));
+    kern<<<resident_grid(kern, 128, pl.smem, grid), 128, pl.smem, s>>>(v, pl.stage ? 1 : 0);
+  })));
   return cudaGetLastError();
 }
 #endif

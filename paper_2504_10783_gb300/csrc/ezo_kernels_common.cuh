@@ -635,6 +635,37 @@ __device__ __forceinline__ void stage_grid(uint8_t* lb_s, const EnvDev& e) {
     for (int i = threadIdx.x; i < kGridLbBytes / 16; i += blockDim.x) dst[i] = __ldg(src + i);
 }
 
+// Shared memory of collide_lane beside LaneSmem: the warps' queues, the groups'
+// words, spheres, axis records and frames, the grid's coarse bounds when staged.
+// `lane` is
+// LaneRobot's (slots, general) as lane_code packs them, -1 where collide_lane
+// does not apply.
+__host__ __device__ inline size_t lane_smem_layout(int nsp, int n, int threads, int T, int lane, bool stage) {
+  return (size_t)nsp * (sizeof(float4) + sizeof(float2) + sizeof(int)) +
+         (size_t)(threads / 32) * kNearQueue * sizeof(int) +
+         (size_t)(threads / T) * lane_group_words(n, lane >> 1, lane & 1, T) * sizeof(float) +
+         (stage ? kGridLbBytes : 0);
+}
+
+// A collision kernel's form (collide_lane where the robot and the obstacle
+// sets admit it: lane >= 0), its dynamic shared memory and whether it stages
+// the grid's bounds: when `pays` and they fit.
+struct CheckPlan {
+  bool lane, stage;
+  size_t smem;
+};
+inline CheckPlan check_plan(int nsp, int n, int threads, int T, int n_rbox, int n_ebox, int lane, bool pays) {
+  CheckPlan p;
+  p.lane = lane >= 0;
+  auto bytes = [&](bool st) {
+    return p.lane ? lane_smem_layout(nsp, n, threads, T, lane, st)
+                  : check_smem_layout(nsp, threads, T, n_rbox, n_ebox, st);
+  };
+  p.stage = pays && bytes(true) <= kSmemBudget;
+  p.smem = bytes(p.stage);
+  return p;
+}
+
 // Whether a launch over N configurations at T lanes each looks up enough
 // bounds per resident block to pay for copying them to shared memory.
 inline bool stage_grid_pays(int nsp, const EnvDev& e, long long N, int T) {
@@ -653,6 +684,81 @@ __device__ __forceinline__ BoxCtx box_ctx(const GeomSmem& g, const RobotDev* rob
   return b;
 }
 
+
+// The collision test as the kernels call it, T lanes per configuration:
+// collide_lane (LANE) or collide_group. Constructed by all threads of the
+// block; the caller synchronises after the constructor and around set_env.
+template <bool LANE>
+struct CheckRobot {
+  using type = RobotSmem;
+};
+template <>
+struct CheckRobot<true> {
+  using type = LaneSmem;
+};
+
+template <int NDOF, int T, bool BOX, bool LANE>
+struct Checker {
+  typename CheckRobot<LANE>::type& rs;
+  const RobotDev* robot;
+  GeomSmem gs;
+  float4* cen;
+  int lg;
+  BoxCtx bx;
+  float2* sa;
+  int* frame;
+  float* mine;
+  int* queue;
+  int stride;
+  bool stage_lb;
+  EnvDev env;
+  const uint8_t* lb;
+
+  __device__ __forceinline__ Checker(typename CheckRobot<LANE>::type& shared, float4* smem, const RobotDev* r,
+                                     int max_ebox, bool stage)
+      : rs(shared), robot(r), lg(threadIdx.x % T), stage_lb(stage) {
+    const int nsp = r->n_spheres_pad;
+    if constexpr (LANE) {
+      const int words = lane_group_words(r->n, r->lane.n_slot, r->lane.general, T), g = threadIdx.x / T;
+      gs.sph = smem;
+      int* queues = reinterpret_cast<int*>(smem + nsp);
+      queue = queues + (threadIdx.x / 32) * kNearQueue;
+      float* w = reinterpret_cast<float*>(queues + (blockDim.x / 32) * kNearQueue);
+      stride = T == 1 ? blockDim.x : words;
+      mine = T == 1 ? w + g : w + g * words;
+      gs.lb = reinterpret_cast<uint8_t*>(w + (blockDim.x / T) * words);
+      sa = reinterpret_cast<float2*>(gs.lb + (stage ? kGridLbBytes : 0));
+      frame = reinterpret_cast<int*>(sa + nsp);
+      stage_lane_robot(rs, gs.sph, frame, r);
+    } else {
+      const int nrbox = r->n_box, groups = blockDim.x / T;
+      gs = carve_geom(smem, nsp, groups, nrbox, max_ebox);
+      cen = gs.cen_all + (threadIdx.x / T) * (nsp + 1);
+      stage_robot(rs, gs.sph, r);
+      stage_robot_boxes(gs.rbox_l, r);
+    }
+  }
+
+  __device__ __forceinline__ void set_env(const EnvDev& e) {
+    env = e;
+    if (stage_lb) stage_grid(gs.lb, e);
+    lb = stage_lb ? gs.lb : e.grid.lb;
+    if constexpr (LANE) {
+      stage_lane_env(sa, robot, e);
+    } else {
+      stage_env_boxes(gs.ebox, e);
+      bx = box_ctx(gs, robot, robot->n_box, e.n_box, threadIdx.x / T);
+    }
+  }
+
+  __device__ __forceinline__ bool operator()(const float (&q)[NDOF]) const {
+    if constexpr (LANE) {
+      return collide_lane<NDOF, T>(q, rs, gs.sph, sa, frame, env, lb, mine, stride, lg, queue);
+    } else {
+      return collide_group<NDOF, T, BOX>(q, rs, gs.sph, env, lb, robot->self_pairs, robot->self_rr, cen, lg, bx);
+    }
+  }
+};
 
 // Projection of Eqs. (6)-(7) in FP64: c_proj = (1 - alpha) v1 + alpha v2.
 template <int NDOF>
@@ -717,6 +823,18 @@ __device__ __forceinline__ void project_fp64(const double (&c)[NDOF], const doub
       constexpr int TT = 8;                  \
       __VA_ARGS__;                           \
     }                                        \
+  } while (0)
+
+// LL = whether the kernel runs collide_lane
+#define EZO_DISPATCH_LANE(lane, ...) \
+  do {                               \
+    if (lane) {                      \
+      constexpr bool LL = true;      \
+      __VA_ARGS__;                   \
+    } else {                         \
+      constexpr bool LL = false;     \
+      __VA_ARGS__;                   \
+    }                                \
   } while (0)
 
 // EZO_DISPATCH_T with the wide groups of 16 and 32 lanes (the bisection)

@@ -84,8 +84,8 @@ int na_test_size(int k, double eps, double delta, double tau) {
   return (int)std::ceil(2.0 * std::log(1.0 / dk) / (eps * tau * tau));
 }
 
-// Lanes per configuration of the label and bisection kernels: the rule of
-// ezo_batch_create for rounds of this size (two lanes per configuration below
+// Lanes per configuration of the label and bisection kernels by collide_group:
+// the rule of ezo_batch_create for rounds of this size (two lanes per configuration below
 // 2^20 samples, sixteen per bisection candidate below 2^20 candidates, eight
 // with boxes; labels do not depend on the choice); above that, the size rule
 // of the collision checker, since the tuner would allocate.
@@ -103,6 +103,7 @@ int bisect_lanes(long long np, bool boxes) { return np >= (1ll << 20) ? lanes_fo
 // The robot and env handles are defined in ezo_capi.cu; these accessors give
 // this file the device images it needs without touching that code path.
 extern "C" int ezo_internal_robot_boxes(const ezo_robot* r);
+extern "C" int ezo_internal_lane(const ezo_robot* r, const ezo_env* e);
 extern "C" const ezo::RobotDev* ezo_internal_robot_dev(const ezo_robot* r, int* n, int* nsp_pad, double* q_lo,
                                                        double* q_hi);
 extern "C" int ezo_internal_env_dev(const ezo_robot* r, const ezo_env* e, ezo::EnvDevFull* out);
@@ -287,8 +288,11 @@ extern "C" ezo_status ezo_inflate_segment_noalloc(const ezo_robot* robot, const 
   NA_CUDA(cudaGetDevice(&dev));
   NA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   v.n_sm = sms;
-  const int T_check = std::max(check_lanes(s_cap), t_min);
-  const int T_bis = std::max(bisect_lanes(np, ezo_internal_robot_boxes(robot) || envf.e.n_box), t_min);
+  v.lane = ezo_internal_lane(robot, env);
+  const bool lane = v.lane >= 0;
+  const int T_check = std::max(lane ? lane_check_lanes(s_cap) : check_lanes(s_cap), t_min);
+  const int T_bis = std::max(
+      lane ? lane_bisect_lanes(np) : bisect_lanes(np, ezo_internal_robot_boxes(robot) || envf.e.n_box), t_min);
   const int grid_s = (int)std::max<long long>(1, std::min<long long>(st_tiles * 8, (long long)sms * 16));
   const int grid_c = (int)std::max<long long>(1, std::min<long long>(st_tiles * T_check, (long long)sms * 16));
   const int grid_b = (int)std::max<long long>(1, std::min<long long>(bi_tiles * T_bis, (long long)sms * 16));

@@ -25,6 +25,7 @@ extern "C" const ezo::RobotDev* ezo_internal_robot_dev(const ezo_robot* r, int* 
 extern "C" int ezo_internal_env_dev(const ezo_robot* r, const ezo_env* e, ezo::EnvDevFull* out);
 extern "C" void ezo_internal_set_error(const char* msg);
 extern "C" int ezo_internal_robot_boxes(const ezo_robot* r);
+extern "C" int ezo_internal_lane(const ezo_robot* r, const ezo_env* e);
 
 namespace {
 
@@ -39,7 +40,7 @@ __global__ void k_uniform_configs(float* q, long long N, int n, const float* lo,
 }
 
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int, int, int, int, int>, int> g_tune_cache;
+std::map<std::tuple<int, int, int, int, int, int, int, int, int>, int> g_tune_cache;
 bool g_autotune = true;
 
 int size_class(long long N) {
@@ -65,7 +66,7 @@ extern "C" __attribute__((visibility("hidden"))) int ezo_internal_tuned_lanes(co
   const RobotDev* rd = ezo_internal_robot_dev(robot, &n, &nsp, lo, hi);
   EnvDevFull ef{};
   if (!rd || ezo_internal_env_dev(robot, env, &ef) != 0) return rule(N);
-  const int nrbox = ezo_internal_robot_boxes(robot);
+  const int nrbox = ezo_internal_robot_boxes(robot), lane = ezo_internal_lane(robot, env);
   // only lane counts whose sphere centres fit in shared memory (more lanes,
   // fewer groups per block, less memory); 8 when none does, which the entry
   // points reject before launching
@@ -82,7 +83,7 @@ extern "C" __attribute__((visibility("hidden"))) int ezo_internal_tuned_lanes(co
   int dev = 0;
   cudaGetDevice(&dev);
   const int cls = size_class(N);
-  const auto key = std::make_tuple(dev, n, nsp, head.n_self, ef.e.n_obs_pad, cls, nrbox, ef.e.n_box);
+  const auto key = std::make_tuple(dev, n, nsp, head.n_self, ef.e.n_obs_pad, cls, nrbox, ef.e.n_box, lane);
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune_cache.find(key);
@@ -114,11 +115,11 @@ extern "C" __attribute__((visibility("hidden"))) int ezo_internal_tuned_lanes(co
       const int T = lanes[li];
       if (!fits(T)) continue;
       // one warm-up launch, then the best of three
-      if (launch_check_flat(rd, n, nsp, nrbox, ef.e, q, M, M, flags, T, sms * 32, s) != cudaSuccess) continue;
+      if (launch_check_flat(rd, n, nsp, nrbox, lane, ef.e, q, M, M, flags, T, sms * 32, s) != cudaSuccess) continue;
       float t_best = 1e30f;
       for (int rep = 0; rep < 3; ++rep) {
         cudaEventRecord(e0, s);
-        launch_check_flat(rd, n, nsp, nrbox, ef.e, q, M, M, flags, T, sms * 32, s);
+        launch_check_flat(rd, n, nsp, nrbox, lane, ef.e, q, M, M, flags, T, sms * 32, s);
         cudaEventRecord(e1, s);
         cudaEventSynchronize(e1);
         float ms = 0.f;

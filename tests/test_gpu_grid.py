@@ -64,3 +64,67 @@ def test_grid_labels_equal_all_pairs(kind, n):
         assert not ((flags != hit.to(torch.uint8)) & ~near).any(), lanes
     if kind in ("box", "plane"):
         assert 0 < int(hit.sum()) and (n > 64 or int(hit.sum()) < N)
+
+
+@pytest.mark.parametrize("layout", ["links", "one_axis_each", "general", "many_links", "same_frame", "base"])
+def test_lane_walk_equals_group_form(layout):
+    """Labels with self pairs at every lane count, for robots that the one-walk
+    form orders differently (spheres on one axis of their frames, off the axes,
+    more links than its list holds, pairs on one frame, base spheres with
+    pairs), against the pair tests on the FP32 sphere centres, and the round
+    kernels' labels and bisections at every lane count against one another."""
+    import torch
+
+    from paper_2504_10783_gb300 import ezo
+    from paper_2504_10783_gb300 import workloads as wl
+    rng = np.random.default_rng(5)
+    n = 11 if layout == "many_links" else 5
+    rd = wl.chain_robot(n, a=0.3, r=0.05, per_link=5)
+    link = rd.sphere_frame
+    if layout == "one_axis_each":
+        for f in range(1, n + 1):
+            m = link == f
+            rd.sphere_xyz[m] = 0.0
+            rd.sphere_xyz[m, f % 3] = rng.uniform(-0.25, 0.1, int(m.sum()))
+    elif layout == "general":
+        rd.sphere_xyz = rd.sphere_xyz + rng.normal(0.0, 0.03, rd.sphere_xyz.shape)
+    elif layout == "base":
+        rd.sphere_frame = rd.sphere_frame - 1  # the first link's spheres sit on the fixed base frame
+        link = rd.sphere_frame
+    pairs = [(i, j) for i in range(rd.n_spheres) for j in range(i + 1, rd.n_spheres) if link[j] - link[i] >= 2]
+    if layout == "same_frame":
+        pairs.append((0, 4))
+    rd.self_pairs = np.asarray(pairs, dtype=np.int32)
+    obs = np.column_stack([rng.uniform((0.3, -0.8, -0.2), (1.4, 0.8, 1.0), (40, 3)), rng.uniform(0.02, 0.08, 40)])
+    robot, env = ezo.Robot(rd), ezo.Env(obs)
+    N = 4099
+    qd = torch.from_numpy(np.ascontiguousarray(wl.uniform_configs(3, rd, N).astype(np.float32).T)).cuda()
+    cen = torch.empty((rd.n_spheres, 3, N), dtype=torch.float64, device="cuda")
+    ezo.sphere_centres(robot, qd, cen)
+    order = np.argsort(robot.sphere_order)
+    c = cen.permute(2, 0, 1).float()[:, torch.from_numpy(order).cuda()]
+    r = torch.tensor(rd.sphere_r, dtype=torch.float32, device="cuda")
+    o = torch.tensor(obs, dtype=torch.float32, device="cuda")
+    p = torch.from_numpy(rd.self_pairs.astype(np.int64)).cuda()
+    ratio = torch.cat([((c[:, :, None] - o[:, :3]).double().square().sum(-1)
+                        / (r[:, None] + o[:, 3]).double().square()).flatten(1),
+                       (c[:, p[:, 0]] - c[:, p[:, 1]]).double().square().sum(-1)
+                       / (r[p[:, 0]] + r[p[:, 1]]).double().square()], 1)
+    hit, near = (ratio < 1).any(1).to(torch.uint8), ((ratio - 1).abs() < 1e-6).any(1)
+    assert int(near.sum()) <= 3 and 0.05 < hit.float().mean().item() < 0.95
+    assert (ratio[:, 40 * rd.n_spheres:] < 1).any(1).sum().item() > 20  # self collisions among them
+    for lanes in (1, 2, 4, 8):
+        flags = torch.full((N,), 7, dtype=torch.uint8, device="cuda")
+        ezo.check_collision(robot, env, qd, flags, lanes=lanes)
+        assert not ((flags != hit) & ~near).any(), lanes
+    free = torch.nonzero((ratio > 1.05).all(1)).flatten()[0].item()
+    v = qd[:, free].cpu().numpy().astype(np.float64)
+    prm = ezo.Params.make(eps=0.2, delta=0.2, n_p=700, n_f=10, n_b=10, n_mix=10, n_it_max=2, seed=3)
+    ref = None
+    for lanes in (1, 2, 4, 8, 16, 32, 96):
+        bt = ezo.Batch(robot, [env], v, v + 1e-3, prm)
+        bt.set_shape(bt.shape()["sample_fill_tiles"], min(lanes, 8), lanes)
+        bt.run()
+        got = (bt.read(0, "labels"), bt.read(0, "bits"), bt.segment(0).A)
+        ref = ref or got
+        assert all(np.array_equal(a, b) for a, b in zip(ref, got)), lanes
