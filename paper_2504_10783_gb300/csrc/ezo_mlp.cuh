@@ -1,40 +1,82 @@
-// Training GEMMs of the learned surrogate: arguments shared by the kernels
-// that compute C[M x N] = A[M x K] B[N x K]^T (both operands BF16, K
-// contiguous, row-major with leading dimensions lda, ldb; FP32 accumulation)
-// with the epilogues of the forward and backward passes.
+// Training of the learned surrogate: the operand images and the arguments of
+// the kernels in ezo_mlp_gemm_tc.cu.
+//
+// An operand image holds rows of 64 BF16 values (one K-chunk) in the K-major
+// 128-byte swizzled layout of the tensor cores (sw128, ezo_tc.cuh), so a
+// range of its rows is one contiguous copy. Batch-major operands (features x
+// rows of the next product's K) are [tile of 128 batch rows][K-chunk of 64
+// features][128 rows]; transposed ones [chunk of 64 batch rows][feature];
+// weights [K-chunk][256 rows]. Pre-activations are FP32 [tile][feature][128
+// batch rows].
 #pragma once
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <cstddef>
+#include <cstdint>
+
 namespace ezo {
 
-enum Epi : int {
-  EPI_F32 = 0,        // C (FP32) = acc
-  EPI_BIAS_SILU = 1,  // Z = acc + bias (FP32), H = SiLU(Z) (BF16, and transposed)
-  EPI_DSILU = 2       // D = acc * SiLU'(Z) (BF16, and transposed)
+constexpr int kMlpChunk = 256 * 128;                 // bytes of a K-chunk of 256 rows
+constexpr int kMlpWeights = 2 * 65536 + 256 * 64;    // hidden weights: W3, W2, W1 in a workspace
+// flat parameter layout: W1 [256 x 64] | b1 | W2 [256 x 256] | b2 | W3 | b3 | w4 [256] | b4 [1]
+constexpr long long kOffW1 = 0, kOffB1 = kOffW1 + 256 * 64, kOffW2 = kOffB1 + 256, kOffB2 = kOffW2 + 65536,
+                    kOffW3 = kOffB2 + 256, kOffB3 = kOffW3 + 65536, kOffW4 = kOffB3 + 256, kOffB4 = kOffW4 + 256,
+                    kNumParams = kOffB4 + 1;
+constexpr int kOutPart = 258;    // a block's partial sums: dw4, db4, loss
+constexpr int kOutBlocks = 256;  // blocks of the output layer's kernel at most
+
+inline int mlp_splits(int rows) { return (rows + 127) / 128; }
+inline int mlp_out_blocks(int rows) { return rows / 8 < kOutBlocks ? rows / 8 : kOutBlocks; }
+
+struct LayerArgs {
+  const uint8_t* A;   // batch-major image of the input (not the first layer)
+  const uint8_t* B;   // weight image (backward: the transposed one)
+  int rows;           // batch rows, a multiple of 64
+  const float* bias;  // forward
+  float* Z;           // pre-activations: written forward, read backward
+  uint8_t* H;         // batch-major image of the result, or null
+  uint8_t* Ht;        // transposed image of the result
+  const float* q;     // first layer: configurations, value j of row i at q[j * ldq + i]
+  long long ldq;
+  int n;
+  uint8_t* Xt;        // first layer: transposed feature image, 64 features a chunk
+  int* err;           // set when a bounded wait gave up
+};
+struct WgradArgs {
+  const uint8_t *Xt, *H1t, *H2t, *dZ1t, *dZ2t, *dZ3t;
+  int rows;
+  float* ws;  // [128 batch rows][kMlpWeights]
+  int* err;
+};
+struct OutputArgs {
+  const uint8_t* H3t;
+  const float *Z3, *w4, *b4, *t;
+  int rows;
+  uint8_t *dZ3, *dZ3t;
+  float* part;  // [block][kOutPart]
+};
+struct UpdateArgs {
+  const float* ws;
+  int splits;
+  const uint8_t *dZ1t, *dZ2t, *dZ3t;
+  int rows;
+  const float* part;
+  int out_blocks;
+  float *g, *loss;
+  float lr;  // 0: gradients only
+  float beta1, beta2, eps, c1, c2;
+  float *p, *m, *v;
+  uint8_t *img, *timg;  // weight images
 };
 
-struct GemmArgs {
-  const __nv_bfloat16* A;
-  const __nv_bfloat16* B;
-  int M, N, K, lda, ldb;
-  const int* m_dev;  // optional device row count (rows >= *m_dev are skipped)
-  float* C;          // EPI_F32 output, ldc
-  int ldc;
-  const float* bias;
-  float* Z;          // EPI_BIAS_SILU: pre-activation out; EPI_DSILU: pre-activation in (ldz = N)
-  __nv_bfloat16* H;  // BF16 output, row-major (ldh = N)
-  __nv_bfloat16* Ht; // BF16 output, transposed [N x ldt]
-  int ldt;
-};
-
-// The same products on tcgen05 (ezo_mlp_gemm_tc.cu): K and lda, ldb multiples
-// of 64; M any; N a multiple of 64 up to 256. EPI_F32 splits K over blocks
-// when `ws` (FP32 workspace of gemm_tc_ws_floats(M, N, K) values) is given and
-// adds the partial products in a fixed order, so results are reproducible.
-// `err` (device int) is set when a bounded wait gave up.
-size_t gemm_tc_ws_floats(int M, int N, int K);
-cudaError_t gemm_tc(int epi, const GemmArgs& a, float* ws, int* err, cudaStream_t s);
+cudaError_t mlp_layer_first(const LayerArgs& g, cudaStream_t s);
+cudaError_t mlp_layer_forward(const LayerArgs& g, cudaStream_t s);
+cudaError_t mlp_layer_backward(const LayerArgs& g, cudaStream_t s);
+cudaError_t mlp_output(const OutputArgs& g, cudaStream_t s);
+cudaError_t mlp_wgrad(const WgradArgs& g, cudaStream_t s);
+cudaError_t mlp_update(const UpdateArgs& u, cudaStream_t s);
+cudaError_t mlp_weight_images(const float* p, void* img, void* timg, cudaStream_t s);
 
 }  // namespace ezo

@@ -35,8 +35,9 @@
 // Shared-memory operands use the K-major 128-byte swizzled layout: a row of
 // 64 BF16 values is 128 bytes, 8 rows form a 1024-byte atom, and 16-byte
 // chunk c of row r sits at chunk position c ^ (r % 8). The weights are kept
-// in global memory as images of that layout (built once per weight update),
-// so each chunk is one contiguous bulk copy.
+// in global memory as images of that layout (written with every weight
+// update: chunk 0 = W1 [256 x 64], chunks 1..4 = W2 columns 64 (j - 1) ..,
+// chunks 5..8 = W3 likewise), so each chunk is one contiguous bulk copy.
 //
 // Every wait on an mbarrier gives up after about two seconds: the kernel
 // then records an error code, writes NaN for the rows it has not finished
@@ -403,33 +404,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_forward_tc(TcArgs g) {
   }
 }
 
-// image of the three hidden-layer weight matrices in the swizzled K-major
-// layout: chunk 0 = W1 [256 x 64], chunks 1..4 = W2 columns 64 (j - 1) ..,
-// chunks 5..8 = W3 likewise; element (n, k) of a chunk at byte
-// sw128(n, k / 8) + 2 (k % 8)
-__global__ void k_mlp_tc_image(const __nv_bfloat16* __restrict__ W1, const __nv_bfloat16* __restrict__ W2,
-                               const __nv_bfloat16* __restrict__ W3, uint8_t* __restrict__ img) {
-  const int total = kChunksPerTile * kTcH * 64;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-    const int j = i / (kTcH * 64), rem = i % (kTcH * 64), n = rem / 64, k = rem % 64;
-    __nv_bfloat16 w;
-    if (j == 0) w = W1[n * kTcF + k];
-    else if (j <= 4) w = W2[n * kTcH + (j - 1) * 64 + k];
-    else w = W3[n * kTcH + (j - 5) * 64 + k];
-    *reinterpret_cast<__nv_bfloat16*>(img + j * kChunkBytes + sw128(n, k >> 3) + (k & 7) * 2) = w;
-  }
-}
-
 }  // namespace
 
 size_t mlp_tc_image_bytes() { return (size_t)kChunksPerTile * kChunkBytes; }
-
-cudaError_t mlp_tc_build_image(const void* W1, const void* W2, const void* W3, void* img, cudaStream_t s) {
-  k_mlp_tc_image<<<(kChunksPerTile * kTcH * 64 + 255) / 256, 256, 0, s>>>(
-      static_cast<const __nv_bfloat16*>(W1), static_cast<const __nv_bfloat16*>(W2),
-      static_cast<const __nv_bfloat16*>(W3), static_cast<uint8_t*>(img));
-  return cudaGetLastError();
-}
 
 // y[i] = sd_hat of configuration i (q: n x rows_cap, stride ldq) for rows
 // i < min(*m_dev, rows_cap) (all rows_cap rows when m_dev is null).

@@ -354,3 +354,40 @@ def test_surrogate_wavefront_graph_equals_host_loop(ezo, trained):
             np.testing.assert_array_equal(a.A, b.A)
             np.testing.assert_array_equal(a.b, b.b)
     assert any(r.status == ezo.SEG_ACCEPTED for r in res[ezo.RUN_GRAPH])
+
+
+@pytest.mark.parametrize("batch", [64, 128, 192, 320, 2112])
+def test_gradient_at_tile_edges(batch):
+    """One gradient at batch sizes around the 128-row tiles and the 64-row
+    chunks of the training kernels, after a larger batch has left its rows in
+    the buffers, against FP64 autograd on the same weights: the BF16 roundings
+    of the pass (2^-8 relative each, a dozen in a chain, averaged over the
+    batch) stay within 3% of each tensor's norm, a wrong or missing row is at
+    least 1 / batch of it in the output layer's gradient."""
+    import torch
+
+    from paper_2504_10783_gb300 import ezo
+    from paper_2504_10783_gb300 import workloads as wl
+    robot = ezo.Robot(wl.dh7_robot())
+    sur = ezo.Surrogate(robot, seed=3)
+    g = torch.Generator(device="cuda").manual_seed(batch)
+    q = torch.rand((7, 2496), generator=g, device="cuda") * 4 - 2
+    t = torch.rand(2496, generator=g, device="cuda") * 0.4 - 0.1
+    sur.grad(q, t)
+    q, t = q[:, :batch], t[:batch]
+    loss, got = sur.grad(q, t)
+    p = torch.tensor(sur.params(), dtype=torch.float64, requires_grad=True)
+    x = torch.cat([torch.sin(q.T), torch.cos(q.T), q.new_zeros(batch, 50)], 1).double().cpu()
+    at, cuts = 0, []
+    for rows, cols in ((256, 64), (256, 256), (256, 256)):
+        W, at = p[at:at + rows * cols].reshape(rows, cols), at + rows * cols
+        x = torch.nn.functional.silu(x @ W.T + p[at:at + rows])
+        cuts += [at, at + rows]
+        at += rows
+    y = x @ p[at:at + 256] + p[at + 256]
+    ref_loss = ((y - t.double().cpu()) ** 2).mean()
+    ref_loss.backward()
+    assert abs(loss - ref_loss.item()) <= 0.03 * ref_loss.item()
+    for a, b in zip(np.split(got.astype(np.float64), cuts + [at + 256]),
+                    np.split(p.grad.numpy(), cuts + [at + 256])):
+        assert np.linalg.norm(a - b) <= 0.03 * np.linalg.norm(b)
