@@ -147,8 +147,8 @@ cudaError_t launch_check_flat(const RobotDev* robot, int n, int nsp_pad, int n_r
                               const float* q, long long ldq, long long N, uint8_t* flags, int T, int grid_cap,
                               cudaStream_t s);
 // signed distance, exact below cap (3e38: exact everywhere)
-cudaError_t launch_sd_flat(const RobotDev* robot, int n, int nsp_pad, const EnvDev& env, const float* q, long long ldq,
-                           long long N, float* sd, cudaStream_t s, float cap = 3.0e38f);
+cudaError_t launch_sd_flat(const RobotDev* robot, int n, int nsp_pad, int lane, const EnvDev& env,
+                           const WideGrid& wide, const float* q, long long ldq, long long N, float* sd, cudaStream_t s, float cap = 3.0e38f);
 cudaError_t launch_sample_flat(const double* A, const double* b, int m, int lda, int n, const double* v1h,
                                const double* v2h, long long N, int n_mix, uint64_t seed, uint32_t stream, int k,
                                float* out, long long ldo, cudaStream_t s);
@@ -210,8 +210,9 @@ cudaError_t launch_round_bisect_box(const BatchView& v, int T, int grid, cudaStr
 
 cudaError_t launch_fk_centres(const RobotDev* robot, const RobotFK64* r64, int n, int nsp_pad, const float* q,
                               long long ldq, long long N, int mode, double* out_c, float* err, cudaStream_t s);
-// Builds the grid over n_obs obstacles (ezo_grid.cu): the coarse bounds, the
-// fine cells and their id lists; `used` (zero before) counts list entries.
+// Builds a grid over n_obs obstacles (ezo_grid.cu): the coarse bounds (unless
+// null), the fine cells and their id lists, which cells farther than `far`
+// from every obstacle go without; `used` (zero before) counts list entries.
 struct GridBuild {
   const float4* obs;
   int n_obs;

@@ -102,8 +102,8 @@ __global__ void __launch_bounds__(64) k_grid_build(GridBuild g) {
     }
     unsigned kind = (unsigned)m;
     if (m > (int)kGridInline) {
-      // cells farther from every obstacle than the grid's edge need no list:
-      // a sphere that large is tested against every obstacle
+      // the collision grid's cells farther from every obstacle than its edge
+      // need no list: a sphere that large is tested against every obstacle
       kind = kGridAll;
       if (low <= g.far) {
         const unsigned off = atomicAdd(g.used, (unsigned)m);
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(64) k_grid_build(GridBuild g) {
     atomicMin(&s_lb[sub == 2 ? t & 0x2a : t], lb8);
   }
   __syncthreads();
-  if (in && (sub == 1 || (t & ~0x2a) == 0))
+  if (in && g.lb && (sub == 1 || (t & ~0x2a) == 0))
     g.lb[((z / sub) * kGridC + y / sub) * kGridC + x / sub] = (uint8_t)s_lb[t];
 }
 

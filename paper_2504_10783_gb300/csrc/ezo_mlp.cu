@@ -73,11 +73,13 @@ cudaError_t dal(T** p, size_t n) {
 
 extern "C" int ezo_internal_robot_boxes(const ezo_robot* r);
 extern "C" int ezo_internal_env_boxes(const ezo_env* e);
+extern "C" int ezo_internal_sd_lane(const ezo_robot* r);
+extern "C" int ezo_internal_env_dev(const ezo_robot* r, const ezo_env* e, ezo::EnvDevFull* out);
+extern "C" ezo::WideGrid ezo_internal_sd_grid(const ezo_env* e, long long N, cudaStream_t s);
 extern "C" int ezo_internal_robot_prismatic(const ezo_robot* r);
 extern "C" void ezo_internal_set_error(const char* msg);
 extern "C" const ezo::RobotDev* ezo_internal_robot_dev(const ezo_robot* r, int* n, int* nsp_pad, double* q_lo,
                                                        double* q_hi);
-extern "C" int ezo_internal_env_dev(const ezo_robot* r, const ezo_env* e, ezo::EnvDevFull* out);
 
 struct ezo_surrogate {
   int n = 0;
@@ -367,6 +369,7 @@ ezo_status ezo_surrogate_train(ezo_surrogate* S, const ezo_env* env, int64_t n_s
   const RobotDev* rd = ezo_internal_robot_dev(S->robot, &n, &nsp, lo, hi);
   EnvDevFull ef{};
   ezo_internal_env_dev(S->robot, env, &ef);
+  const int lane = ezo_internal_sd_lane(S->robot);
   const long long N = n_samples / batch * batch;
   // one block: the configurations, their labels, the joint limits
   float* q = nullptr;
@@ -383,7 +386,7 @@ ezo_status ezo_surrogate_train(ezo_surrogate* S, const ezo_env* env, int64_t n_s
     // signed distance, clamped to [label_lo, label_hi]
     k_uniform_q<<<blocks_for(N, 256), 256, 0, s>>>(q, N, n, bnd, bnd + EZO_MAX_DOF, (uint32_t)data_seed,
                                                      (uint32_t)(data_seed >> 32));
-    e = launch_sd_flat(rd, n, nsp, ef.e, q, N, N, t, s, label_hi);
+    e = launch_sd_flat(rd, n, nsp, lane, ef.e, lane >= 0 ? ezo_internal_sd_grid(env, N, s) : WideGrid{}, q, N, N, t, s, label_hi);
     k_clamp_labels<<<blocks_for(N, 256), 256, 0, s>>>(t, N, label_lo, label_hi);
   }
   for (int ep = 0; ep < epochs && e == cudaSuccess; ++ep) {

@@ -128,3 +128,44 @@ def test_lane_walk_equals_group_form(layout):
         got = (bt.read(0, "labels"), bt.read(0, "bits"), bt.segment(0).A)
         ref = ref or got
         assert all(np.array_equal(a, b) for a, b in zip(ref, got)), lanes
+
+
+@pytest.mark.parametrize("kind,n", [("box", 1), ("box", 5), ("box", 64), ("box", 1023), ("cluster", 300),
+                                    ("plane", 700), ("spread", 100), ("far", 33), ("none", 0)])
+def test_signed_distance_equals_all_pairs(kind, n):
+    """The signed distance (bounds of the obstacle grid, sphere by sphere)
+    against the minimum over every pair on the checker's FP32 sphere centres:
+    both round the same expression, 2e-7 of the coordinates' size apart at
+    most (1e-6 m of a 1.7 m reach; of 1e6 m where the set lies that far out)."""
+    import torch
+
+    from paper_2504_10783_gb300 import ezo
+    from paper_2504_10783_gb300 import workloads as wl
+    rng = np.random.default_rng(n)
+    rd = wl.chain_robot(7, a=0.2, r=0.05)
+    rd.sphere_r = np.concatenate([[0.0, 0.35], rng.uniform(0.01, 0.1, rd.n_spheres - 2)])
+    obs = _obstacles(kind, n, rng) if n else np.zeros((0, 4))
+    robot, env = ezo.Robot(rd), ezo.Env(obs)
+    N = 1021
+    q = wl.uniform_configs(n + 1, rd, N).astype(np.float32)
+    q[5, 3] = np.nan
+    qd = torch.from_numpy(np.ascontiguousarray(q.T)).cuda()
+    cen = torch.empty((rd.n_spheres, 3, N), dtype=torch.float64, device="cuda")
+    ezo.sphere_centres(robot, qd, cen)
+    c = cen.permute(2, 0, 1)[:, torch.from_numpy(np.argsort(robot.sphere_order)).cuda()]
+    r = torch.tensor(rd.sphere_r, dtype=torch.float32, device="cuda").double()
+    o = torch.tensor(obs, dtype=torch.float32, device="cuda").double()
+    p = torch.from_numpy(rd.self_pairs.astype(np.int64)).cuda()
+    ref = ((c[:, p[:, 0]] - c[:, p[:, 1]]).norm(dim=2) - r[p[:, 0]] - r[p[:, 1]])
+    for j0 in range(0, n, 128):
+        d = (c[:, :, None, :] - o[None, None, j0: j0 + 128, :3]).norm(dim=3) - r[:, None] - o[j0: j0 + 128, 3]
+        ref = torch.cat([ref, d.flatten(1)], 1)
+    ref = torch.where(ref.isnan(), torch.full_like(ref, 3.0e38), ref).amin(1)
+    tol = 1e-6 if kind != "far" else 0.25
+    for reps in (1, 17):  # small calls go by the collision grid's bounds, large ones by a grid of their own
+        sd = torch.empty(N * reps, dtype=torch.float32, device="cuda")
+        ezo.signed_distance(robot, env, qd.repeat(1, reps).contiguous(), sd)
+        torch.cuda.synchronize()
+        want = ref.repeat(reps)
+        bad = ((sd.double() - want).abs() > tol) & ~((sd > 1e37) & (want > 1e37))
+        assert not bad.any(), (reps, sd[bad][:5], want[bad][:5])
