@@ -12,7 +12,10 @@ namespace ezo {
 
 #if !EZO_BOX_TU
 
-template <int NDOF>
+// Walks shared by TS lanes each (the same samples bit for bit): a call with
+// few walks is a chain of dependent steps that leaves the GPU idle, and TS
+// lanes draw the coming directions and scan the rows together.
+template <int NDOF, int TS>
 __global__ void __launch_bounds__(128) k_sample_flat(const double* __restrict__ A, const double* __restrict__ b,
                                                      int m, int lda, int n, SampleParams p,
                                                      float* __restrict__ out, long long ldo, long long N) {
@@ -20,9 +23,15 @@ __global__ void __launch_bounds__(128) k_sample_flat(const double* __restrict__ 
   float* A32 = reinterpret_cast<float*>(smf4);
   stage_polytope<NDOF>(A32, A, b, m, lda, n);
   __syncthreads();
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+  const int gi = threadIdx.x / TS, lw = threadIdx.x % TS, groups = blockDim.x / TS;
+  for (long long base = (long long)blockIdx.x * groups; base < N; base += (long long)gridDim.x * groups) {
+    const long long i = base + gi, ic = i < N ? i : N - 1;
     float x[NDOF];
-    hnr_walk<NDOF>(A32, m, n, p.v1f, p.ef, p.n_mix, p.keys, (uint32_t)i, p.round_k, p.stream, x);
+    if constexpr (TS == 1)
+      hnr_walk<NDOF>(A32, m, n, p.v1f, p.ef, p.n_mix, p.keys, (uint32_t)ic, p.round_k, p.stream, x);
+    else
+      hnr_walk_split<NDOF, TS>(A32, m, n, p.v1f, p.ef, p.n_mix, p.keys, (uint32_t)ic, p.round_k, p.stream, lw, x);
+    if (i >= N || lw != 0) continue;
 #pragma unroll
     for (int j = 0; j < NDOF; ++j)
       if (j < n) out[(long long)j * ldo + i] = x[j];
@@ -303,15 +312,21 @@ cudaError_t launch_sample_flat(const double* A, const double* b, int m, int lda,
   p.stream = stream;
   p.round_k = (uint32_t)k;
   const int threads = 128;
-  const long long grid = (N + threads - 1) / threads;
+  // Lanes per walk from the count of walks (us at 1, 2, 4, 8 lanes, 60 steps,
+  // 40 rows, 7 joints): 1000 walks 87, 64, 44, 33; 10007 87, 74, 56, 56; 20000
+  // 107, 89, 77, 95; 30000 107, 107, 102, 124; 50000 138, 151, 153, 191. Two
+  // lanes pay between only where rows beyond a joint box split (30000 walks,
+  // 10 joints, 60 rows: 292, 264, 332; 14 rows: 38, 47, 38).
+  const int TS = N < 10240 ? 8 : (N < 24576 ? 4 : (N < 40960 && m > 2 * n + 8 ? 2 : 1));
+  const long long grid = (N * TS + threads - 1) / threads;
   cudaError_t err = cudaSuccess;
-  EZO_DISPATCH_NDOF(n, {
+  EZO_DISPATCH_NDOF(n, EZO_DISPATCH_T(TS, {
     const size_t smem = hnr_smem_bytes<ND>(m);
-    auto kern = k_sample_flat<ND>;
+    auto kern = k_sample_flat<ND, TT>;
     err = set_smem(kern, smem);
     if (err != cudaSuccess) return err;
-    kern<<<(unsigned)grid, threads, smem, s>>>(A, b, m, lda, n, p, out, ldo, N);
-  });
+    kern<<<(unsigned)std::min<long long>(grid, 1ll << 20), threads, smem, s>>>(A, b, m, lda, n, p, out, ldo, N);
+  }));
   return cudaGetLastError();
 }
 
