@@ -13,8 +13,11 @@
 #include <vector>
 
 #include "../../include/ezo.h"
+#include "ezo_engine.cuh"
 
 extern "C" void ezo_internal_set_error(const char* msg);
+ezo_status ezo_internal_batch_take(const ezo_batch* b, const std::vector<int>& segs, std::vector<ezo::SegState>& states,
+                                   std::vector<double>& A, std::vector<double>& bv, int* rows, cudaStream_t s);
 
 struct ezo_polytope {
   int32_t m = 0, n = 0, segment = -1;
@@ -51,30 +54,33 @@ int severity(ezo_status s) {
   return 2;
 }
 
-// Segment g of a finished batch as a host polytope with its statistics.
-ezo_status take_polytope(const ezo_batch* b, int32_t g, int32_t n, int32_t m_cap, ezo_polytope** out) {
-  ezo_polytope* p = new (std::nothrow) ezo_polytope();
-  if (!p) return api_fail(EZO_ERR_CAPACITY, "out of host memory");
-  p->n = n;
-  p->segment = g;
-  p->A.resize((size_t)m_cap * n);
-  p->b.resize((size_t)m_cap);
-  ezo_status st = ezo_batch_get_polytope(b, g, &p->m, p->A.data(), p->b.data());
-  int64_t work[3] = {0, 0, 0}, evals = 0;
-  if (st == EZO_OK)
-    st = ezo_batch_get_segment(b, g, &p->stats.status, &p->stats.rounds, &p->stats.m, &p->stats.planes,
-                               &p->stats.checks);
-  if (st == EZO_OK) st = ezo_batch_read(b, g, 9, work, sizeof(work));
-  if (st == EZO_OK) st = ezo_batch_read(b, g, 11, &evals, sizeof(evals));
-  if (st != EZO_OK) {
-    delete p;
-    return st;
+// The segments segs of a finished batch as host polytopes with their
+// statistics.
+ezo_status take_polytopes(const ezo_batch* b, const std::vector<int>& segs, int32_t n, cudaStream_t s,
+                          std::vector<ezo_polytope*>& out) {
+  std::vector<ezo::SegState> st;
+  std::vector<double> A, bv;
+  int rows = 0;
+  const ezo_status e = ezo_internal_batch_take(b, segs, st, A, bv, &rows, s);
+  if (e != EZO_OK) return e;
+  for (size_t i = 0; i < segs.size(); ++i) {
+    ezo_polytope* p = new (std::nothrow) ezo_polytope();
+    if (!p) return api_fail(EZO_ERR_CAPACITY, "out of host memory");
+    out.push_back(p);
+    const ezo::SegState& t = st[i];
+    p->n = n;
+    p->m = t.m;
+    p->segment = segs[i];
+    p->A.assign(A.begin() + i * rows * n, A.begin() + (i * rows + t.m) * n);
+    p->b.assign(bv.begin() + i * rows, bv.begin() + i * rows + t.m);
+    p->stats.status = t.status;
+    p->stats.rounds = t.rounds;
+    p->stats.m = t.m;
+    p->stats.planes = t.planes;
+    p->stats.checks = t.checks;
+    p->stats.checks_bisect = t.checks_bisect;
+    p->stats.surrogate_evals = t.sur_evals;
   }
-  p->A.resize((size_t)p->m * n);
-  p->b.resize((size_t)p->m);
-  p->stats.checks_bisect = work[1];
-  p->stats.surrogate_evals = evals;
-  *out = p;
   return EZO_OK;
 }
 
@@ -95,12 +101,14 @@ ezo_status ezo_inflate_segment(const ezo_robot* robot, const ezo_env* env, const
                                    params, &b);
   if (st != EZO_OK) return st;
   st = ezo_batch_run(b, EZO_RUN_HOST_LOOP, cuda_stream);
-  int32_t m_cap = 0;
-  if (st == EZO_OK) st = ezo_batch_capacity(b, &m_cap, nullptr);
-  ezo_polytope* p = nullptr;
-  if (st == EZO_OK) st = take_polytope(b, 0, ezo_robot_dof(robot), m_cap, &p);
+  std::vector<ezo_polytope*> got;
+  if (st == EZO_OK) st = take_polytopes(b, {0}, ezo_robot_dof(robot), (cudaStream_t)cuda_stream, got);
   ezo_batch_free(b);
-  if (st != EZO_OK) return st;
+  if (st != EZO_OK) {
+    for (ezo_polytope* q : got) delete q;
+    return st;
+  }
+  ezo_polytope* p = got[0];
   if (stats) *stats = p->stats;
   *out = p;
   const ezo_status outcome = segment_outcome(p->stats.status);
@@ -149,11 +157,15 @@ ezo_status ezo_inflate_batch(const ezo_robot* robot, int32_t n_env, const ezo_en
   // segment speculatively in one graph, the skip rule afterwards
   const int32_t seq = mode == 0 ? 1 : (mode == 1 ? 2 : 0);
   st = ezo_batch_run_path(b, seq, mode == 0 ? EZO_RUN_HOST_LOOP : EZO_RUN_GRAPH, cuda_stream);
-  int32_t m_cap = 0;
-  if (st == EZO_OK) st = ezo_batch_capacity(b, &m_cap, nullptr);
   std::vector<int32_t> status(B), mm(B);
   if (st == EZO_OK) st = ezo_batch_get_polytopes(b, status.data(), mm.data(), nullptr, nullptr, 0, nullptr, cuda_stream);
+  std::vector<int> segs;
+  for (int32_t g = 0; g < B && st == EZO_OK; ++g)
+    if (status[g] != EZO_SEG_SKIPPED && status[g] != EZO_SEG_IDLE) segs.push_back(g);
+  std::vector<ezo_polytope*> got;
+  if (st == EZO_OK) st = take_polytopes(b, segs, n, (cudaStream_t)cuda_stream, got);
   ezo_status worst = EZO_OK;
+  size_t next = 0;
   for (int32_t i = 0; i < n_path && st == EZO_OK; ++i) {
     ezo_scs* scs = new (std::nothrow) ezo_scs();
     if (!scs) {
@@ -161,18 +173,16 @@ ezo_status ezo_inflate_batch(const ezo_robot* robot, int32_t n_env, const ezo_en
       break;
     }
     out[i] = scs;
-    for (int32_t k = 0; k < path_len[i] && st == EZO_OK; ++k) {
-      const int32_t g = first_seg[i] + k;
-      if (status[g] == EZO_SEG_SKIPPED || status[g] == EZO_SEG_IDLE) continue;
-      ezo_polytope* p = nullptr;
-      st = take_polytope(b, g, n, m_cap, &p);
-      if (st != EZO_OK) break;
-      p->segment = k;
+    for (; next < segs.size() && segs[next] < first_seg[i] + path_len[i]; ++next) {
+      ezo_polytope* p = got[next];
+      got[next] = nullptr;
+      p->segment = segs[next] - first_seg[i];
       scs->sets.push_back(p);
-      const ezo_status o = segment_outcome(status[g]);
+      const ezo_status o = segment_outcome(status[segs[next]]);
       if (severity(o) > severity(worst)) worst = o;
     }
   }
+  for (ezo_polytope* p : got) delete p;
   ezo_batch_free(b);
   if (st != EZO_OK) {
     for (int32_t i = 0; i < n_path; ++i) {

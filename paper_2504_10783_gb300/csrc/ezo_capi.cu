@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -16,6 +17,7 @@
 
 #include "../../include/ezo.h"
 #include "ezo_engine.cuh"
+#include "ezo_pool.cuh"
 
 using namespace ezo;
 
@@ -39,6 +41,26 @@ ezo_status cuda_fail(cudaError_t e, const char* where) {
     cudaError_t e_ = (call);                            \
     if (e_ != cudaSuccess) return cuda_fail(e_, #call); \
   } while (0)
+
+// Working memory kept between calls; freed with the last handle.
+BlockPool& device_pool() {
+  static BlockPool* p = new BlockPool(false);  // never destroyed: the driver may be gone at exit
+  return *p;
+}
+BlockPool& host_pool() {
+  static BlockPool* p = new BlockPool(true);
+  return *p;
+}
+std::atomic<int> g_handles{0};
+struct HandleCount {
+  HandleCount() { ++g_handles; }
+  ~HandleCount() {
+    if (--g_handles == 0) {
+      device_pool().trim();
+      host_pool().trim();
+    }
+  }
+};
 
 constexpr double kU32 = 5.9604644775390625e-8;  // 2^-24
 
@@ -78,6 +100,7 @@ struct EventPool {
 }  // namespace
 
 struct ezo_robot {
+  HandleCount alive;
   RobotDev host{};
   RobotDev* d_robot = nullptr;
   RobotFK64* d_fk64 = nullptr;  // FP64 chain for the kinematics error
@@ -87,6 +110,7 @@ struct ezo_robot {
   std::vector<int> sphere_sorted;              // caller's sphere index -> sorted index
   int n = 0, n_spheres = 0, nsp_pad = 0, n_self = 0;
   int n_base = 0;  // sorted spheres on frame 0 (the fixed base), the first n_base
+  double base_lo[3] = {0, 0, 0}, base_hi[3] = {0, 0, 0};  // the box around them
   std::vector<double> q_lo, q_hi;
   double r_max = 0.0;
   double fk_flops = 0.0;
@@ -95,6 +119,7 @@ struct ezo_robot {
 };
 
 struct ezo_env {
+  HandleCount alive;
   // one block: obstacles, the grid's list counter, coarse bounds, cells, lists
   char* d_mem = nullptr;
   float4* d_obs = nullptr;
@@ -125,6 +150,10 @@ struct ezo_env {
 // Any base sphere within 1e-4 m of an obstacle keeps the full sweep.
 static int sweep_first(const ezo_robot* r, const ezo_env* e, int cut) {
   if (cut == 0) return 0;
+  // apart along an axis by the box around the base spheres and the one around
+  // the obstacles: clear without a look at the pairs
+  for (int k = 0; k < 3 && e->n_obs > 0; ++k)
+    if (e->lo[k] - r->base_hi[k] > 1e-4 || r->base_lo[k] - e->hi[k] > 1e-4) return cut;
   for (int s = 0; s < cut; ++s) {
     const float4 l = r->host.sph[s];
     for (const float4& o : e->h_obs) {
@@ -419,6 +448,13 @@ ezo_status ezo_robot_create(int32_t n, const double* a, const double* alpha, con
     h.frame_first[n + 1] = n_spheres;
   }
   r->n_base = h.frame_first[1];
+  for (int s = 0; s < r->n_base; ++s) {
+    const double c[3] = {h.sph[s].x, h.sph[s].y, h.sph[s].z}, w = h.sph[s].w;
+    for (int k = 0; k < 3; ++k) {
+      r->base_lo[k] = s ? std::min(r->base_lo[k], c[k] - w) : c[k] - w;
+      r->base_hi[k] = s ? std::max(r->base_hi[k], c[k] + w) : c[k] + w;
+    }
+  }
   r->sphere_sorted = inv;
   std::vector<ushort2> pairs(std::max(1, n_self_pairs));
   std::vector<float> rr(std::max(1, n_self_pairs));
@@ -872,6 +908,8 @@ __attribute__((visibility("hidden"))) int ezo_internal_env_dev(const ezo_robot* 
   return 0;
 }
 
+__attribute__((visibility("hidden"))) int ezo_internal_robot_self(const ezo_robot* r) { return r->n_self; }
+
 __attribute__((visibility("hidden"))) int ezo_internal_lane(const ezo_robot* r, const ezo_env* e) {
   return lane_code(r, e);
 }
@@ -909,6 +947,7 @@ int32_t ezo_check_static_spheres(const ezo_robot* robot, const ezo_env* env) {
 }  // extern "C"
 
 struct ezo_batch {
+  HandleCount alive;
   const ezo_robot* robot = nullptr;
   int B = 0, n = 0, m0 = 0, m_cap = 0, s_cap_max = 0, np_max = 0, max_path_len = 1, max_obs_pad = 0, max_ebox = 0;
   ezo_params prm{};
@@ -936,7 +975,8 @@ struct ezo_batch {
   int* d_path_first = nullptr;
   uint8_t* d_contained = nullptr;
   SegState* d_st0 = nullptr;    // initial state, for resets
-  double *d_A0 = nullptr, *d_b0 = nullptr;  // initial polytopes
+  double *d_A0 = nullptr, *d_b0 = nullptr;  // the domain, m0 rows: every segment's initial polytope
+  char* mem = nullptr;  // one block of the device pool: all of the above
   std::vector<double> v1h, v2h;
   BatchView view{};
   int T_check = 1, T_bisect = 4, split_below = 0;
@@ -978,15 +1018,14 @@ void drop_graphs(ezo_batch* b) {
 ezo_status batch_free_device(ezo_batch* b) {
   drop_graphs(b);
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
-  void* ptrs[] = {b->d_st,    b->d_v1,    b->d_v2,   b->d_A,    b->d_b,      b->d_S,      b->d_flags,
-                  b->d_cidx,  b->d_cstar, b->d_dist, b->d_c32,  b->d_cn,     b->d_bits,   b->d_pidx, b->d_ga, b->d_gb,
-                  b->d_pdelta, b->d_stiles, b->d_btiles, b->d_sum, b->d_envs, b->d_path_first, b->d_contained, b->d_st0, b->d_A0, b->d_b0,
-                  b->view.s_p32, b->view.s_d32, b->view.s_lo, b->view.s_hi,
-                  b->view.s_bits, b->view.s_ok, b->view.s_rows, b->view.sm_seats, b->view.q_claim,
+  void* ptrs[] = {b->view.s_lo, b->view.s_hi, b->view.s_bits, b->view.s_ok, b->view.s_rows,
                   b->d_wnext, b->d_wlast, b->d_wkept};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  if (b->h_sum) cudaFreeHost(b->h_sum);
+  // work queued on the batch's buffers ends before they are handed on
+  if (b->mem) cudaDeviceSynchronize();
+  device_pool().give(b->mem);
+  host_pool().give(b->h_sum);
   for (auto e : b->events.ev) cudaEventDestroy(e);
   return EZO_OK;
 }
@@ -1405,75 +1444,76 @@ ezo_status ezo_batch_create(const ezo_robot* robot, int32_t n_env, const ezo_env
     return fail(EZO_ERR_INVALID_ARG, "ezo_batch_create: robot spheres and obstacles exceed shared memory at 8 lanes");
   }
   const long long B = n_seg, mc = b->m_cap;
-  cudaError_t e = cudaSuccess;
-#define EZO_ALLOC(p, cnt) \
-  if (e == cudaSuccess) e = dalloc(&(p), (size_t)(cnt))
-  EZO_ALLOC(b->d_st, B);
-  EZO_ALLOC(b->d_v1, B * n);
-  EZO_ALLOC(b->d_v2, B * n);
-  EZO_ALLOC(b->d_A, B * mc * n);
-  EZO_ALLOC(b->d_b, B * mc);
-  EZO_ALLOC(b->d_S, b->total_s * n);
-  EZO_ALLOC(b->d_flags, b->total_s);
-  EZO_ALLOC(b->d_cidx, b->total_c);
-  EZO_ALLOC(b->d_cstar, b->total_c * n);
-  EZO_ALLOC(b->d_dist, b->total_c);
-  EZO_ALLOC(b->d_c32, b->total_c * n);
-  EZO_ALLOC(b->d_cn, b->total_c);
-  EZO_ALLOC(b->d_bits, b->total_c);
-  EZO_ALLOC(b->d_ga, b->total_c * n);
-  EZO_ALLOC(b->d_gb, b->total_c);
-  EZO_ALLOC(b->d_pidx, B * prm->n_f);
-  EZO_ALLOC(b->d_pdelta, B * prm->n_f);
-  EZO_ALLOC(b->d_stiles, b->max_sample_tiles);
-  EZO_ALLOC(b->d_btiles, b->max_bisect_tiles);
-  EZO_ALLOC(b->d_sum, 1);
-  EZO_ALLOC(b->d_envs, n_env);
-  EZO_ALLOC(b->d_path_first, B);
-  EZO_ALLOC(b->d_contained, B * b->max_path_len);
-  EZO_ALLOC(b->d_st0, B);
-  EZO_ALLOC(b->d_A0, B * mc * n);
-  EZO_ALLOC(b->d_b0, B * mc);
-  // the bisection's projected candidate rows (c_proj, c - c_proj in FP32)
   b->view.s_ld = n <= 8 ? 8 : EZO_MAX_DOF;
-  EZO_ALLOC(b->view.s_p32, (long long)b->max_bisect_tiles * kTile * b->view.s_ld);
-  EZO_ALLOC(b->view.s_d32, (long long)b->max_bisect_tiles * kTile * b->view.s_ld);
-  EZO_ALLOC(b->view.sm_seats, kSeatSlots);
   // one claim per work unit of the largest launch: 8 passes per sample tile,
   // up to 32 per bisection tile
   b->claim_cap = std::max<long long>((long long)b->max_sample_tiles * 8, (long long)b->max_bisect_tiles * 32);
-  EZO_ALLOC(b->view.q_claim, b->claim_cap + 1);
   b->view.q_claim_cap = (int)b->claim_cap;
-#undef EZO_ALLOC
-  if (e == cudaSuccess) e = cudaMallocHost(&b->h_sum, sizeof(RoundSummary));
+  // One block: what starts from host values (uploaded in one copy), what
+  // starts zero (one memset), and the rest.
+  size_t image = 0, zeros = 0, total = 0;
+  auto layout = [&](char* base) {
+    size_t at = 0;
+    auto take = [&](auto*& p, long long count) {
+      p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(base + at);
+      at += ((size_t)std::max<long long>(1, count) * sizeof(*p) + 255) & ~(size_t)255;
+    };
+    take(b->d_st0, B);
+    take(b->d_v1, B * n);
+    take(b->d_v2, B * n);
+    take(b->d_envs, n_env);
+    take(b->d_path_first, B);
+    take(b->d_A0, (long long)m0 * n);
+    take(b->d_b0, m0);
+    image = at;
+    take(b->d_sum, 1);
+    take(b->view.sm_seats, kSeatSlots);
+    take(b->view.q_claim, b->claim_cap + 1);
+    take(b->d_flags, b->total_s);
+    zeros = at - image;
+    take(b->d_st, B);
+    take(b->d_A, B * mc * n);
+    take(b->d_b, B * mc);
+    take(b->d_S, b->total_s * n);
+    take(b->d_cidx, b->total_c);
+    take(b->d_cstar, b->total_c * n);
+    take(b->d_dist, b->total_c);
+    take(b->d_c32, b->total_c * n);
+    take(b->d_cn, b->total_c);
+    take(b->d_bits, b->total_c);
+    take(b->d_ga, b->total_c * n);
+    take(b->d_gb, b->total_c);
+    take(b->d_pidx, B * prm->n_f);
+    take(b->d_pdelta, B * prm->n_f);
+    take(b->d_stiles, b->max_sample_tiles);
+    take(b->d_btiles, b->max_bisect_tiles);
+    take(b->d_contained, B * b->max_path_len);
+    // the bisection's projected candidate rows (c_proj, c - c_proj in FP32)
+    take(b->view.s_p32, (long long)b->max_bisect_tiles * kTile * b->view.s_ld);
+    take(b->view.s_d32, (long long)b->max_bisect_tiles * kTile * b->view.s_ld);
+    total = at;
+  };
+  layout(nullptr);
+  cudaError_t e = cudaSuccess;
+  b->mem = (char*)device_pool().take(total, &e);
+  if (e == cudaSuccess) b->h_sum = (RoundSummary*)host_pool().take(sizeof(RoundSummary), &e);
   if (e != cudaSuccess) {
     batch_free_device(b);
     delete b;
     return cuda_fail(e, "ezo_batch_create: allocation");
   }
-  // initial contents
-  std::vector<double> Ah((size_t)B * mc * n, 0.0), bh((size_t)B * mc, 0.0);
-  for (long long g = 0; g < B; ++g) {
-    std::copy(A0v.begin(), A0v.end(), Ah.begin() + g * mc * n);
-    std::copy(b0v.begin(), b0v.end(), bh.begin() + g * mc);
-  }
-#define EZO_H2D(dst, src, bytes) \
-  if (e == cudaSuccess) e = cudaMemcpy((dst), (src), (bytes), cudaMemcpyHostToDevice)
-  EZO_H2D(b->d_st, b->st0.data(), sizeof(SegState) * B);
-  EZO_H2D(b->d_v1, v1, sizeof(double) * B * n);
-  EZO_H2D(b->d_v2, v2, sizeof(double) * B * n);
-  EZO_H2D(b->d_A, Ah.data(), sizeof(double) * Ah.size());
-  EZO_H2D(b->d_b, bh.data(), sizeof(double) * bh.size());
-  EZO_H2D(b->d_envs, b->envs.data(), sizeof(EnvDevFull) * n_env);
-  EZO_H2D(b->d_path_first, b->path_first.data(), sizeof(int) * B);
-  EZO_H2D(b->d_st0, b->st0.data(), sizeof(SegState) * B);
-  EZO_H2D(b->d_A0, Ah.data(), sizeof(double) * Ah.size());
-  EZO_H2D(b->d_b0, bh.data(), sizeof(double) * bh.size());
-#undef EZO_H2D
-  if (e == cudaSuccess) e = cudaMemset(b->d_sum, 0, sizeof(RoundSummary));
-  if (e == cudaSuccess) e = cudaMemset(b->view.sm_seats, 0, sizeof(int) * kSeatSlots);
-  if (e == cudaSuccess) e = cudaMemset(b->view.q_claim, 0, sizeof(int) * (b->claim_cap + 1));
-  if (e == cudaSuccess) e = cudaMemset(b->d_flags, 0, (size_t)std::max<long long>(1, b->total_s));
+  std::vector<char> host(image);
+  layout(host.data());
+  std::memcpy(b->d_st0, b->st0.data(), sizeof(SegState) * B);
+  std::memcpy(b->d_v1, v1, sizeof(double) * B * n);
+  std::memcpy(b->d_v2, v2, sizeof(double) * B * n);
+  std::memcpy(b->d_envs, b->envs.data(), sizeof(EnvDevFull) * n_env);
+  std::memcpy(b->d_path_first, b->path_first.data(), sizeof(int) * B);
+  std::memcpy(b->d_A0, A0v.data(), sizeof(double) * A0v.size());
+  std::memcpy(b->d_b0, b0v.data(), sizeof(double) * b0v.size());
+  layout(b->mem);
+  e = cudaMemcpy(b->mem, host.data(), image, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b->mem + image, 0, zeros, nullptr);
   if (e != cudaSuccess) {
     batch_free_device(b);
     delete b;
@@ -1530,6 +1570,14 @@ ezo_status ezo_batch_create(const ezo_robot* robot, int32_t n_env, const ezo_env
   v.path_first = b->d_path_first;
   v.max_path_len = b->max_path_len;
   v.graph_cond = 0;
+  // states and polytopes; complete before any stream uses the batch
+  e = launch_batch_reset(v, b->d_st0, b->d_A0, b->d_b0, m0, nullptr);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+  if (e != cudaSuccess) {
+    batch_free_device(b);
+    delete b;
+    return cuda_fail(e, "ezo_batch_create: initial state");
+  }
   // launch shapes: lanes per configuration from the work per round
   const int sms = sm_count();
   long long tot_np = 0, tot_s1 = 0;
@@ -1759,7 +1807,7 @@ ezo_status ezo_batch_reset(ezo_batch* b, const double* v1, const double* v2, voi
   if (v2) EZO_CUDA(cudaMemcpyAsync(b->d_v2, v2, sizeof(double) * B * n, cudaMemcpyHostToDevice, s));
   // states, starting polytopes and the summary in one kernel (the summary's
   // work-queue fields reset themselves at the end of every launch)
-  EZO_CUDA(launch_batch_reset(b->view, b->d_st0, b->d_A0, b->d_b0, s));
+  EZO_CUDA(launch_batch_reset(b->view, b->d_st0, b->d_A0, b->d_b0, b->m0, s));
   g_err.clear();
   return EZO_OK;
 }
@@ -1949,6 +1997,53 @@ ezo_status ezo_batch_get_polytopes(const ezo_batch* b, int32_t* status, int32_t*
   }
   g_err.clear();
   return EZO_OK;
+}
+
+// The segments segs[0 .. count) of a finished batch: their states' fields and
+// polytope rows (A and b with at most `rows` rows each are appended to the
+// vectors) with two copies and two synchronisations. Internal.
+extern "C++" __attribute__((visibility("hidden"))) ezo_status ezo_internal_batch_take(
+    const ezo_batch* b, const std::vector<int>& segs, std::vector<SegState>& states, std::vector<double>& A,
+    std::vector<double>& bv, int* rows, cudaStream_t s) {
+  states.clear();
+  std::vector<SegState> all;
+  EZO_CUDA(cudaStreamSynchronize(s));
+  all.resize(b->B);
+  EZO_CUDA(cudaMemcpyAsync(all.data(), b->d_st, sizeof(SegState) * b->B, cudaMemcpyDeviceToHost, s));
+  EZO_CUDA(cudaStreamSynchronize(s));
+  int m = 0;
+  for (int g : segs) {
+    states.push_back(all[g]);
+    m = std::max(m, all[g].m);
+  }
+  *rows = m;
+  const size_t n = b->n, mc = b->m_cap, k = segs.size();
+  A.resize(k * m * n);
+  bv.resize(k * m);
+  if (!k || !m) return EZO_OK;
+  cudaError_t e = cudaSuccess;
+  double* host = (double*)host_pool().take(sizeof(double) * k * m * (n + 1), &e);
+  if (e != cudaSuccess) return cuda_fail(e, "reading the polytopes");
+  double* hb = host + k * m * n;
+  // runs of consecutive segments, a strided copy each
+  for (size_t i = 0; i < k && e == cudaSuccess;) {
+    size_t j = i + 1;
+    while (j < k && segs[j] == segs[j - 1] + 1) ++j;
+    e = cudaMemcpy2DAsync(host + i * m * n, sizeof(double) * m * n, b->d_A + (size_t)segs[i] * mc * n,
+                          sizeof(double) * mc * n, sizeof(double) * m * n, j - i, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess)
+      e = cudaMemcpy2DAsync(hb + i * m, sizeof(double) * m, b->d_b + (size_t)segs[i] * mc, sizeof(double) * mc,
+                            sizeof(double) * m, j - i, cudaMemcpyDeviceToHost, s);
+    i = j;
+  }
+  const cudaError_t e2 = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = e2;
+  if (e == cudaSuccess) {
+    std::memcpy(A.data(), host, sizeof(double) * A.size());
+    std::memcpy(bv.data(), hb, sizeof(double) * bv.size());
+  }
+  host_pool().give(host);
+  return e == cudaSuccess ? EZO_OK : cuda_fail(e, "reading the polytopes");
 }
 
 ezo_status ezo_host_alloc(size_t bytes, void** out) {
@@ -2142,9 +2237,8 @@ ezo_status ezo_batch_reinflate(ezo_batch* b, const uint8_t* which, int32_t mode,
     r.sample_flops = sts[g].sample_flops;
     r.planes = 0;
     sts[g] = r;
-    EZO_CUDA(cudaMemcpyAsync(b->d_A + g * mc * n, b->d_A0 + g * mc * n, sizeof(double) * mc * n,
-                             cudaMemcpyDeviceToDevice, s));
-    EZO_CUDA(cudaMemcpyAsync(b->d_b + g * mc, b->d_b0 + g * mc, sizeof(double) * mc, cudaMemcpyDeviceToDevice, s));
+    EZO_CUDA(cudaMemcpyAsync(b->d_A + g * mc * n, b->d_A0, sizeof(double) * b->m0 * n, cudaMemcpyDeviceToDevice, s));
+    EZO_CUDA(cudaMemcpyAsync(b->d_b + g * mc, b->d_b0, sizeof(double) * b->m0, cudaMemcpyDeviceToDevice, s));
     any = 1;
   }
   if (!any) {
@@ -2202,24 +2296,34 @@ ezo_status ezo_check_path(const ezo_robot* robot, const ezo_env* env, const doub
     return EZO_OK;
   }
   for (int k = 0; k < K; ++k) off[k + 1] = off[k] + cnt[k];
-  // one scratch block: vertices (FP64), edge offsets, edge flags
-  const size_t vb = sizeof(double) * (size_t)n_verts * n, ob = sizeof(long long) * (size_t)(K + 1);
-  char* scratch = nullptr;
-  EZO_CUDA(cudaMallocAsync((void**)&scratch, vb + ob + (size_t)K, s));
-  double* d_verts = (double*)scratch;
-  long long* d_off = (long long*)(scratch + vb);
+  // one block on each side: vertices (FP64), edge offsets, edge flags (zero)
+  const size_t vb = sizeof(double) * (size_t)n_verts * n, ob = sizeof(long long) * (size_t)(K + 1),
+               bytes = vb + ob + (size_t)K;
+  cudaError_t e = cudaSuccess;
+  char *scratch = (char*)device_pool().take(bytes, &e), *host = nullptr;
+  if (e == cudaSuccess) host = (char*)host_pool().take(bytes, &e);
+  if (e != cudaSuccess) {
+    device_pool().give(scratch);
+    return cuda_fail(e, "ezo_check_path");
+  }
+  std::memcpy(host, verts, vb);
+  std::memcpy(host + vb, off.data(), ob);
+  std::memset(host + vb + ob, 0, (size_t)K);
   uint8_t* d_edge = (uint8_t*)(scratch + vb + ob);
-  cudaError_t e = cudaMemcpyAsync(d_verts, verts, vb, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_off, off.data(), ob, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_edge, 0, (size_t)K, s);
+  e = cudaMemcpyAsync(scratch, host, bytes, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) {
     const int lanes = ezo_internal_tuned_lanes(robot, env, N, s);
-    e = launch_check_path(robot->d_robot, n, robot->nsp_pad, robot->n_box, lane_code(robot, env), env->dev_for(robot), d_verts, K, d_off, N,
-                          point_flags_dev, d_edge, lanes, sm_count() * 32, s);
+    e = launch_check_path(robot->d_robot, n, robot->nsp_pad, robot->n_box, lane_code(robot, env), env->dev_for(robot),
+                          (const double*)scratch, K, (const long long*)(scratch + vb), N, point_flags_dev, d_edge, lanes,
+                          sm_count() * 32, s);
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(edge_flags, d_edge, (size_t)K, cudaMemcpyDeviceToHost, s);
-  cudaFreeAsync(scratch, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(host + vb + ob, d_edge, (size_t)K, cudaMemcpyDeviceToHost, s);
+  // the blocks are given back only when nothing uses them any more
+  const cudaError_t done = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = done;
+  if (e == cudaSuccess) std::memcpy(edge_flags, host + vb + ob, (size_t)K);
+  host_pool().give(host);
+  device_pool().give(scratch);
   if (e != cudaSuccess) return cuda_fail(e, "ezo_check_path");
   g_err.clear();
   return EZO_OK;

@@ -18,16 +18,16 @@ namespace ezo {
 __global__ void __launch_bounds__(1024) k_round_begin(BatchView v) { round_begin_block(v); }
 
 // Reset of a batch in one launch: every segment's state and the rows of its
-// starting polytope (st0[g].m rows; rows past a segment's m are never read),
+// starting polytope (the domain's m rows; rows past a segment's m are never read),
 // and the round summary's public part. One block per segment.
 __global__ void __launch_bounds__(256) k_batch_reset(BatchView v, const SegState* __restrict__ st0,
-                                                     const double* __restrict__ A0, const double* __restrict__ b0) {
+                                                     const double* __restrict__ A0, const double* __restrict__ b0,
+                                                     int m) {
   const int g = blockIdx.x;
   if (g >= v.B) return;
-  const int m = st0[g].m;
   const long long base = (long long)g * v.m_cap;
-  for (int i = threadIdx.x; i < m * v.n; i += blockDim.x) v.A[base * v.n + i] = A0[base * v.n + i];
-  for (int i = threadIdx.x; i < m; i += blockDim.x) v.b[base + i] = b0[base + i];
+  for (int i = threadIdx.x; i < m * v.n; i += blockDim.x) v.A[base * v.n + i] = A0[i];
+  for (int i = threadIdx.x; i < m; i += blockDim.x) v.b[base + i] = b0[i];
   if (threadIdx.x == 0) v.st[g] = st0[g];
   if (g == 0 && threadIdx.x == 0) {
     v.summary->active = 0;
@@ -308,10 +308,10 @@ cudaError_t launch_round_begin(const BatchView& v, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_batch_reset(const BatchView& v, const SegState* st0, const double* A0, const double* b0,
+cudaError_t launch_batch_reset(const BatchView& v, const SegState* st0, const double* A0, const double* b0, int m,
                                cudaStream_t s) {
   if (v.B <= 0) return cudaSuccess;
-  k_batch_reset<<<v.B, 256, 0, s>>>(v, st0, A0, b0);
+  k_batch_reset<<<v.B, 256, 0, s>>>(v, st0, A0, b0, m);
   return cudaGetLastError();
 }
 

@@ -25,6 +25,7 @@ extern "C" const ezo::RobotDev* ezo_internal_robot_dev(const ezo_robot* r, int* 
 extern "C" int ezo_internal_env_dev(const ezo_robot* r, const ezo_env* e, ezo::EnvDevFull* out);
 extern "C" void ezo_internal_set_error(const char* msg);
 extern "C" int ezo_internal_robot_boxes(const ezo_robot* r);
+extern "C" int ezo_internal_robot_self(const ezo_robot* r);
 extern "C" int ezo_internal_lane(const ezo_robot* r, const ezo_env* e);
 
 namespace {
@@ -78,12 +79,10 @@ extern "C" __attribute__((visibility("hidden"))) int ezo_internal_tuned_lanes(co
     return T;
   };
   if (!g_autotune || N <= 0) return fit_up(rule(N));
-  RobotDev head;
-  if (cudaMemcpy(&head, rd, sizeof(int) * 4, cudaMemcpyDeviceToHost) != cudaSuccess) return fit_up(rule(N));
   int dev = 0;
   cudaGetDevice(&dev);
   const int cls = size_class(N);
-  const auto key = std::make_tuple(dev, n, nsp, head.n_self, ef.e.n_obs_pad, cls, nrbox, ef.e.n_box, lane);
+  const auto key = std::make_tuple(dev, n, nsp, ezo_internal_robot_self(robot), ef.e.n_obs_pad, cls, nrbox, ef.e.n_box, lane);
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune_cache.find(key);
