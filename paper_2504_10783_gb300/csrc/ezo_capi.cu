@@ -1446,8 +1446,8 @@ ezo_status ezo_batch_create(const ezo_robot* robot, int32_t n_env, const ezo_env
   const long long B = n_seg, mc = b->m_cap;
   b->view.s_ld = n <= 8 ? 8 : EZO_MAX_DOF;
   // one claim per work unit of the largest launch: 8 passes per sample tile,
-  // up to 32 per bisection tile
-  b->claim_cap = std::max<long long>((long long)b->max_sample_tiles * 8, (long long)b->max_bisect_tiles * 32);
+  // one unit a candidate row in the two-halvings bisection
+  b->claim_cap = std::max<long long>((long long)b->max_sample_tiles * 8, (long long)b->max_bisect_tiles * kTile);
   b->view.q_claim_cap = (int)b->claim_cap;
   // One block: what starts from host values (uploaded in one copy), what
   // starts zero (one memset), and the rest.

@@ -51,3 +51,32 @@ def test_borrowed_memory_across_threads_and_handles():
     for j, g in enumerate(got):
         for a, b in zip(want[j % 6], g):
             assert np.array_equal(a, b), j
+
+
+def test_every_candidate_row_has_a_claim():
+    """The two-halvings bisection (96 lanes) takes one work unit per candidate
+    row, 128 a tile: with most of N_p = 1000 samples colliding its units
+    outnumber 32 a tile, and the claims still have room for all of them."""
+    from paper_2504_10783_gb300 import ezo
+    from paper_2504_10783_gb300 import workloads as wl
+    robot = ezo.Robot(wl.planar3_robot())
+    # disks all around the outstretched arm: nearly every configuration but
+    # the segment's surroundings collides
+    ang = np.linspace(0.35, 2 * np.pi - 0.35, 60)
+    disks = np.concatenate([np.column_stack([R * np.cos(ang), R * np.sin(ang), 0 * ang, 0.12 + 0 * ang])
+                            for R in (0.6, 1.2, 1.8, 2.4, 2.9)])
+    env = ezo.Env(disks)
+    prm = ezo.Params.make(eps=0.1, delta=0.05, n_p=1000, n_f=10, n_b=10, n_mix=10, n_it_max=6, seed=1)
+    got = {}
+    for lanes in (8, 96):
+        bt = ezo.Batch(robot, [env], np.zeros(3), np.full(3, 0.02), prm)
+        bt.set_shape(bt.shape()["sample_fill_tiles"], 2, lanes)
+        for step in (0, 1, 2, 3, 4):
+            bt.step(step)
+        bt.sync()
+        assert bt.state(0)["n_cand"] > 512  # more than four tiles of 128 rows
+        got[lanes] = bt.read(0, "bits")[: bt.state(0)["n_cand"]]
+        bt.reset()
+        bt.run()
+        got[lanes] = (got[lanes], bt.segment(0).A)
+    assert all(np.array_equal(a, b) for a, b in zip(got[8], got[96]))
