@@ -233,10 +233,13 @@ size_t check_smem_bytes(int n_spheres_pad, int n_obs_pad, int threads, int T, in
 // 0.033 at two, 0.036 at four, 0.047 at eight) unless that leaves schedulers
 // without a warp. A candidate's N_b checks depend on one another: eight lanes
 // are fastest at the few thousand candidates of a path's round (0.054 ms;
-// 0.060 at four and sixteen), four where a round holds hundreds of thousands
-// (24 paths: 3.0 ms; 3.2 at eight, 3.6 at one).
+// 0.060 at four and sixteen), sixteen at a segment's few hundred (0.039 ms;
+// 0.042 at eight), four where a round holds hundreds of thousands (24 paths:
+// 3.0 ms; 3.2 at eight, 3.6 at one).
 inline int lane_check_lanes(long long samples) { return samples >= (1ll << 16) ? 1 : (samples >= (1ll << 14) ? 2 : 4); }
-inline int lane_bisect_lanes(long long candidates) { return candidates >= (1ll << 20) ? 4 : 8; }
+inline int lane_bisect_lanes(long long candidates) {
+  return candidates >= (1ll << 20) ? 4 : (candidates >= (1ll << 15) ? 8 : 16);
+}
 // Dynamic shared memory a collision kernel may request: the opt-in maximum
 // per block (227 KB) less the static robot image and a margin. The sphere
 // centres take (spheres + 1) x 16 bytes per group of lanes, so more lanes per
