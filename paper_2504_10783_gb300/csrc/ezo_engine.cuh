@@ -99,7 +99,7 @@ struct BatchView {
   float* cnorm;      // [cand_off + c]
   uint32_t* bits;    // [cand_off + c]
   double* ga;        // plane normal grad dist_L(c*): [n*cand_off + d*n_p + c]
-  double* gb;        // plane offset a^T c*: [cand_off + c]
+  double* gb;        // plane offset a^T c* - Delta: [cand_off + c]
   int* placed_idx;   // [B][n_f]   candidate index of each plane of the last round
   double* placed_delta;  // [B][n_f]
   int2* sample_tiles;    // (segment, first sample)

@@ -58,7 +58,7 @@ __device__ __forceinline__ double bisect_hi(uint32_t bits, int n_b) {
 
 // c* = c_proj + hi (c - c_proj) of candidate c in FP64, its distance to L, the
 // FP32 copy and its norm, and the tangent plane of Eq. (10) at c*:
-// a = (c* - c_proj) / dist_L(c*), b = a^T c*
+// a = (c* - c_proj) / dist_L(c*), b = a^T c*, with its offset b - Delta
 template <int NDOF>
 __device__ __forceinline__ void bisect_end_point(const BatchView& v, const SegState& st, int g, int c,
                                                  double hi) {
@@ -102,7 +102,31 @@ __device__ __forceinline__ void bisect_end_point(const BatchView& v, const SegSt
       bval = fma(a, cst[j], bval);
     }
   }
-  v.gb[co + c] = bval;
+  // step back (Eqs. 11-12): r = max(a^T v1, a^T v2) - b + Delta_max, Delta =
+  // Delta_max - max(r, 0); the sums in pairs at distance 8, 4, 2, 1. Delta
+  // takes the rows of c - c_proj, which nothing reads after the halvings
+  // (a row of s_ld >= 8 floats per candidate at least).
+  double t1[NDOF], t2[NDOF];
+#pragma unroll
+  for (int j = 0; j < NDOF; ++j) {
+    const double a = j < n ? __dmul_rn(cst[j] - ps[j], inv) : 0.0;
+    t1[j] = j < n ? __dmul_rn(a, v1[j]) : 0.0;
+    t2[j] = j < n ? __dmul_rn(a, v2[j]) : 0.0;
+  }
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+#pragma unroll
+    for (int j = 0; j < o; ++j) {
+      if (j + o < NDOF) {
+        t1[j] = __dadd_rn(t1[j], t1[j + o]);
+        t2[j] = __dadd_rn(t2[j], t2[j + o]);
+      }
+    }
+  }
+  const double r = fmax(t1[0], t2[0]) - bval + v.step_back_max;
+  const double step_back = r > 0.0 ? v.step_back_max - r : v.step_back_max;
+  v.gb[co + c] = bval - step_back;
+  reinterpret_cast<double*>(v.s_d32)[co + c] = step_back;
 }
 
 #if !EZO_BOX_TU
@@ -348,10 +372,60 @@ __global__ void __launch_bounds__(96) k_round_bisect_pair(BatchView v) {
 // a_i^T c_j > b_i - Delta_i; at most N_f planes. One block per segment.
 // The discard test runs in FP32 with a rounding bound and falls back to FP64
 // inside the bound, so every decision equals the FP64 decision.
+//
+// A plane depends on the one before it, so the chain from one plane to the
+// next bounds the kernel. It holds one barrier: each thread keeps its first
+// candidates (coordinates, norm, distance and sample index) in registers, a
+// warp finds its closest by three integer reductions over (distance bits,
+// sample index) and publishes it with its plane (normal and offset b - Delta,
+// from the bisection's end point), and after the barrier every warp reduces
+// the records itself and tests its candidates. FP64 runs at 1/64 of the
+// FP32 rate, an instruction of a warp about 64 cycles, so none is on the chain:
+// distances compare as integers and normals narrow by integer arithmetic. What
+// no later plane needs (the rows of A and b, Delta) follows the last one.
 // CLOSE: the run loops' form, whose last block to finish also closes the
 // round (round_close_block), one launch fewer per round.
+
+// The lexicographic minimum of (hi, lo, si) over the warp and the lanes that
+// hold it; lanes without a candidate pass ~0, ~0, 0x7fffffff.
+__device__ __forceinline__ unsigned warp_closest(unsigned& hi, unsigned& lo, unsigned& si) {
+  const unsigned h = hi, l = lo, s = si;
+  hi = __reduce_min_sync(0xffffffffu, h);
+  lo = __reduce_min_sync(0xffffffffu, h == hi ? l : ~0u);
+  si = __reduce_min_sync(0xffffffffu, h == hi && l == lo ? s : ~0u);
+  return __ballot_sync(0xffffffffu, h == hi && l == lo && s == si);
+}
+
+// (float)d without the FP64 unit; below the normal range 0, which the discard
+// test's absolute term covers
+__device__ __forceinline__ float narrow(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e > 1149u) return (float)d;  // 2^127 and above, infinities, NaN
+  const unsigned sign = hi & 0x80000000u;
+  if (e < 897u) return __uint_as_float(sign);
+  const unsigned m = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const unsigned rest = lo & 0x1fffffffu;
+  return __uint_as_float(sign | (m + (rest + (m & 1u) > 0x10000000u ? 1u : 0u)));
+}
+
+// Ten segments, 646 candidates each, seven joints: 0.8 us a plane at 1024
+// threads with one held candidate each, 0.6 at 512 with two, 0.85 at 512 with
+// four and 0.8 at 256 with four (more reductions to issue, or more held words
+// to fill first); 2.45 us when two barriers, FP64 and a block-wide load lay
+// between planes. A placement of ten planes: 17 us, 30 before; with thousands
+// of candidates a segment (24 paths) 31 us, 43 before.
+constexpr int kPlaceThreads = 512;
+
 template <int NDOF>
 __device__ __forceinline__ void place_segment(const BatchView& v) {
+  // candidates threadIdx.x + kPlaceThreads k: k < kHeld in registers, up to 8
+  // joints with their planes, the others in L1/L2
+  constexpr int kHeld = NDOF <= 8 ? 2 : 1;
+  constexpr int kBatch = NDOF <= 8 ? 4 : 2;  // passes of the others whose loads are in flight together
+  constexpr int kWarps = kPlaceThreads / 32;
+  constexpr bool kPlanes = NDOF <= 8;
+  constexpr int kRec = (NDOF + 4) & ~3;  // a plane: normal, offset at NDOF
   const int g = blockIdx.x;
   SegState& st = v.st[g];
   if (st.status != SEG_ACTIVE) return;
@@ -359,193 +433,203 @@ __device__ __forceinline__ void place_segment(const BatchView& v) {
   const int n = v.n;
   const int np = st.n_p;
   const long long co = st.cand_off;
-  extern __shared__ uint32_t alive[];  // nc bits
-  __shared__ unsigned long long red_key[32];
-  __shared__ int red_sidx[32];
-  __shared__ int red_idx[32];
-  __shared__ int s_best;
-  __shared__ double s_a[EZO_MAX_DOF];
-  __shared__ float s_a32[EZO_MAX_DOF];
-  __shared__ double s_beta;
-  __shared__ float s_beta32;
-  __shared__ int s_stop;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int nwords = (nc + 31) >> 5;
-  for (int w = threadIdx.x; w < nwords; w += blockDim.x) {
-    const int rem = nc - (w << 5);
-    alive[w] = rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u);
-  }
-  if (threadIdx.x == 0) s_stop = 0;
-  __syncthreads();
+  const int m0 = st.m;
+  extern __shared__ uint32_t alive[];  // a bit per candidate past the held ones
+  __shared__ uint4 red[2][kWarps];     // per warp its closest: distance bits, sample index, candidate
+  __shared__ __align__(16) float rec[2][kWarps][kRec];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const double* dist = v.dist + co;
   const int* cidx = v.cand_idx + co;
-  const double* v1 = v.v1 + (long long)g * n;
-  const double* v2 = v.v2 + (long long)g * n;
-  double* A = v.A + (long long)g * v.m_cap * n;
-  double* bb = v.b + (long long)g * v.m_cap;
-  int placed = 0;
+  const double* ga = v.ga + (long long)n * co;
+  const float* c32 = v.c32 + (long long)n * co;
+  const float* cnorm = v.cnorm + co;
   const float u = 5.9604644775390625e-8f;
-  // per-thread best survivor (distance bits, sample index, candidate)
-  unsigned long long best_key = ~0ull;
-  int best_i = 0x7fffffff;
-  int best_c = -1;
-  for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-    const unsigned long long key = (unsigned long long)__double_as_longlong(dist[c]);
-    const int si = cidx[c];
-    if (key < best_key || (key == best_key && si < best_i)) {
-      best_key = key;
-      best_i = si;
-      best_c = c;
+  // dist <= t_col as integers: dist is a square root, so +0 or above (or NaN);
+  // a negative t_col (-0 aside) or NaN is below all
+  unsigned long long t_key = (unsigned long long)__double_as_longlong(v.t_col);
+  if (t_key == 0x8000000000000000ull) t_key = 0ull;
+  const bool t_any = t_key <= 0x7ff0000000000000ull;
+
+  // the thread's closest survivor
+  unsigned b_hi = ~0u, b_lo = ~0u, b_si = 0x7fffffffu;
+  int b_c = -1;
+  auto closer = [&](unsigned hi, unsigned lo, unsigned si, int c) {
+    if (hi < b_hi || (hi == b_hi && (lo < b_lo || (lo == b_lo && si < b_si)))) {
+      b_hi = hi;
+      b_lo = lo;
+      b_si = si;
+      b_c = c;
+    }
+  };
+  float x[kHeld][NDOF], xn[kHeld], own_pl[kHeld][kPlanes ? kRec : 1];
+  unsigned hi[kHeld], lo[kHeld], si[kHeld];
+  bool live[kHeld];
+#pragma unroll
+  for (int k = 0; k < kHeld; ++k) {
+    const int c = threadIdx.x + k * kPlaceThreads;
+    live[k] = c < nc;
+    hi[k] = lo[k] = ~0u;
+    si[k] = 0x7fffffffu;
+    xn[k] = 0.f;
+#pragma unroll
+    for (int j = 0; j < NDOF; ++j) x[k][j] = live[k] && j < n ? c32[(long long)j * np + c] : 0.f;
+    if constexpr (kPlanes) {
+      double a[kRec];
+#pragma unroll
+      for (int j = 0; j < kRec; ++j) a[j] = live[k] && j < n ? ga[(long long)j * np + c] : 0.0;
+      if (live[k]) a[NDOF] = v.gb[co + c];
+#pragma unroll
+      for (int j = 0; j < kRec; ++j) own_pl[k][j] = narrow(a[j]);
+    }
+    if (live[k]) {
+      const long long d = __double_as_longlong(dist[c]);
+      hi[k] = (unsigned)((unsigned long long)d >> 32);
+      lo[k] = (unsigned)d;
+      si[k] = (unsigned)cidx[c];
+      xn[k] = cnorm[c];
     }
   }
-  // warp 0's lane j < n keeps the segment's endpoints' coordinate j
-  const double my_v1 = (wid == 0 && lane < n) ? v1[lane] : 0.0;
-  const double my_v2 = (wid == 0 && lane < n) ? v2[lane] : 0.0;
+#pragma unroll
+  for (int k = 0; k < kHeld; ++k)
+    if (live[k]) closer(hi[k], lo[k], si[k], threadIdx.x + k * kPlaceThreads);
+  // word kWarps k + wid holds this warp's candidates of pass k, and only its own
+  for (int k = kHeld; k * kPlaceThreads + wid * 32 < nc; ++k) {
+    const int c = threadIdx.x + k * kPlaceThreads;
+    const unsigned w = __ballot_sync(0xffffffffu, c < nc);
+    if (lane == 0) alive[k * kWarps + wid] = w;
+    if (c < nc) {
+      const long long d = __double_as_longlong(dist[c]);
+      closer((unsigned)((unsigned long long)d >> 32), (unsigned)d, (unsigned)cidx[c], c);
+    }
+  }
+  __syncwarp();
+
+  int placed = 0, stop = 0, held_c = -1;
+  float held = 0.f;  // lane j < n: the warp's closest candidate's normal; lane n its offset
   for (int f = 0; f < v.n_f; ++f) {
-    // block arg-min of (distance, sample index) over the survivors
+    const int par = f & 1;
+    unsigned r_hi = b_hi, r_lo = b_lo, r_si = b_si;
+    const int own = __ffs(warp_closest(r_hi, r_lo, r_si)) - 1;
+    const int wc = __shfl_sync(0xffffffffu, b_c, own);
+    if (lane == own) red[par][wid] = make_uint4(r_hi, r_lo, r_si, (unsigned)wc);
+    if (kPlanes && wc < kHeld * kPlaceThreads) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, best_key, o);
-      const int i2 = __shfl_xor_sync(0xffffffffu, best_i, o);
-      const int c2 = __shfl_xor_sync(0xffffffffu, best_c, o);
-      if (k2 < best_key || (k2 == best_key && i2 < best_i)) {
-        best_key = k2;
-        best_i = i2;
-        best_c = c2;
-      }
-    }
-    if (lane == 0) {
-      red_key[wid] = best_key;
-      red_sidx[wid] = best_i;
-      red_idx[wid] = best_c;
-    }
-    __syncthreads();
-    if (wid == 0) {
-      unsigned long long bk = lane < nw ? red_key[lane] : ~0ull;
-      int bi = lane < nw ? red_sidx[lane] : 0x7fffffff;
-      int bc = lane < nw ? red_idx[lane] : -1;
+      for (int k = 0; k < kHeld; ++k)
+        if (lane == own && wc / kPlaceThreads == k)
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, bk, o);
-        const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-        const int c2 = __shfl_xor_sync(0xffffffffu, bc, o);
-        if (k2 < bk || (k2 == bk && i2 < bi)) {
-          bk = k2;
-          bi = i2;
-          bc = c2;
-        }
-      }
-      // the plane, with the loads of warp 0's lanes in flight together: lane
-      // j < n holds a_j = (grad dist_L(c*))_j (Eq. 10, from the bisection
-      // kernel) and v1_j, v2_j; lane 0 the distance and b = a^T c*
-      const bool have = bc >= 0;
-      double a = 0.0, dbc = 0.0, bval = 0.0;
-      if (have && lane < n) a = v.ga[(long long)n * co + (long long)lane * np + bc];
-      if (have && lane == 0) {
-        dbc = dist[bc];
-        bval = v.gb[co + bc];
-      }
-      double av1 = a * my_v1, av2 = a * my_v2;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        av1 += __shfl_xor_sync(0xffffffffu, av1, o);
-        av2 += __shfl_xor_sync(0xffffffffu, av2, o);
-      }
-      int stop = 0;
-      double beta = 0.0, delta = 0.0;
-      int row = 0;
-      if (lane == 0) {
-        if (!have) {
-          stop = 1;
-        } else if (dbc <= v.t_col) {
-          stop = 2;  // segment likely in collision (Sec. IV-C)
-        } else if (st.m >= v.m_cap) {
-          stop = 3;
-        } else {
-          // step back (Eqs. 11-12): r = max(a^T v1, a^T v2) - b + Delta_max
-          const double r = fmax(av1, av2) - bval + v.step_back_max;
-          delta = r > 0.0 ? v.step_back_max - r : v.step_back_max;
-          beta = bval - delta;
-          row = st.m;
-        }
-      }
-      stop = __shfl_sync(0xffffffffu, stop, 0);
-      row = __shfl_sync(0xffffffffu, row, 0);
-      if (stop == 0 && lane < n) {
-        s_a[lane] = a;
-        s_a32[lane] = (float)a;
-        A[(long long)row * n + lane] = a;
-      }
-      if (lane == 0) {
-        s_best = bc;
-        s_stop = stop;
-        if (stop == 0) {
-          s_beta = beta;
-          s_beta32 = (float)beta;
-          bb[row] = beta;
-          st.m = row + 1;
-          v.placed_idx[g * v.n_f + f] = bc;
-          v.placed_delta[g * v.n_f + f] = delta;
-        }
-      }
+          for (int j = 0; j < (kPlanes ? kRec : 0); j += 4)
+            *reinterpret_cast<float4*>(&rec[par][wid][j]) =
+                make_float4(own_pl[k][j], own_pl[k][j + 1], own_pl[k][j + 2], own_pl[k][j + 3]);
+    } else if (wc >= 0) {
+      if (wc != held_c && lane <= n) held = narrow(lane < n ? ga[(long long)lane * np + wc] : v.gb[co + wc]);
+      held_c = wc;
+      if (lane <= n) rec[par][wid][lane < n ? lane : NDOF] = held;
     }
     __syncthreads();
-    if (s_stop) break;
+    // two buffers: a warp can write the other one while this one is read, and
+    // writes this one again only after the next barrier
+    const uint4 e = lane < kWarps ? red[par][lane] : make_uint4(~0u, ~0u, 0x7fffffffu, ~0u);
+    r_hi = e.x;
+    r_lo = e.y;
+    r_si = e.z;
+    const int w = __ffs(warp_closest(r_hi, r_lo, r_si)) - 1;
+    const int bc = (int)__shfl_sync(0xffffffffu, e.w, w);
+    if (bc < 0) {
+      stop = 1;
+    } else if (t_any && (((unsigned long long)r_hi << 32) | r_lo) <= t_key) {
+      stop = 2;  // segment likely in collision (Sec. IV-C)
+    } else if (m0 + placed >= v.m_cap) {
+      stop = 3;
+    }
+    if (stop) break;  // the same in every thread
+    if (threadIdx.x == 0) v.placed_idx[g * v.n_f + f] = bc;
     ++placed;
-    const int bc = s_best;
-    const double beta = s_beta;
-    const float beta32 = s_beta32;
+    float pl[kRec];
+#pragma unroll
+    for (int j = 0; j < kRec; j += 4) {
+      const float4 q = *reinterpret_cast<const float4*>(&rec[par][w][j]);
+      pl[j] = q.x;
+      pl[j + 1] = q.y;
+      pl[j + 2] = q.z;
+      pl[j + 3] = q.w;
+    }
+    const float beta32 = pl[NDOF];
+    auto outside = [&](int c, const float (&cj)[NDOF], float cn) {
+      if (c == bc) return true;
+      float s32 = 0.f;
+#pragma unroll
+      for (int j = 0; j < NDOF; ++j)
+        if (j < n) s32 = fmaf(pl[j], cj[j], s32);
+      const float bound = 2.f * (float)(n + 4) * u * (cn + fabsf(beta32)) + 1e-30f;
+      if (fabsf(s32 - beta32) > bound) return s32 > beta32;
+      double sd = 0.0;
+      for (int j = 0; j < n; ++j)
+        sd = fma(ga[(long long)j * np + bc], v.cstar[(long long)n * co + (long long)j * np + c], sd);
+      return sd > v.gb[co + bc];
+    };
     // one pass: discard candidates outside the new half space and find the
-    // best survivor for the next plane
-    best_key = ~0ull;
-    best_i = 0x7fffffff;
-    best_c = -1;
-    for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-      if (!((alive[c >> 5] >> (c & 31)) & 1u)) continue;
-      bool out;
-      if (c == bc) {
-        out = true;
-      } else {
-        // the candidate's coordinates in one batch of loads, then the dot product
-        float cj[NDOF];
+    // closest survivor for the next plane
+    b_hi = b_lo = ~0u;
+    b_si = 0x7fffffffu;
+    b_c = -1;
 #pragma unroll
-        for (int j = 0; j < NDOF; ++j) cj[j] = (j < n) ? v.c32[(long long)n * co + (long long)j * np + c] : 0.f;
-        float s32 = 0.f;
+    for (int k = 0; k < kHeld; ++k) {
+      const int c = threadIdx.x + k * kPlaceThreads;
+      if (live[k] && outside(c, x[k], xn[k])) live[k] = false;
+      if (live[k]) closer(hi[k], lo[k], si[k], c);
+    }
+    for (int k0 = kHeld; k0 * kPlaceThreads + wid * 32 < nc; k0 += kBatch) {
+      unsigned word[kBatch], any = 0u;
 #pragma unroll
-        for (int j = 0; j < NDOF; ++j)
-          if (j < n) s32 = fmaf(s_a32[j], cj[j], s32);
-        const float bound = 2.f * (float)(n + 4) * u * (v.cnorm[co + c] + fabsf(beta32)) + 1e-30f;
-        if (fabsf(s32 - beta32) > bound) {
-          out = s32 > beta32;
-        } else {
-          double sd = 0.0;
-          for (int j = 0; j < n; ++j) sd = fma(s_a[j], v.cstar[(long long)n * co + (long long)j * np + c], sd);
-          out = sd > beta;
-        }
+      for (int i = 0; i < kBatch; ++i) {
+        word[i] = (k0 + i) * kPlaceThreads + wid * 32 < nc ? alive[(k0 + i) * kWarps + wid] : 0u;
+        any |= word[i];
       }
-      if (out) {
-        atomicAnd(&alive[c >> 5], ~(1u << (c & 31)));
-      } else {
-        const unsigned long long key = (unsigned long long)__double_as_longlong(dist[c]);
-        const int si = cidx[c];
-        if (key < best_key || (key == best_key && si < best_i)) {
-          best_key = key;
-          best_i = si;
-          best_c = c;
-        }
+      if (!any) continue;  // the whole warp
+      float cj[kBatch][NDOF], cn[kBatch];
+      long long d[kBatch];
+      int ci[kBatch];
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        const int c = threadIdx.x + (k0 + i) * kPlaceThreads;
+        const bool in = (word[i] >> lane) & 1u;
+#pragma unroll
+        for (int j = 0; j < NDOF; ++j) cj[i][j] = in && j < n ? c32[(long long)j * np + c] : 0.f;
+        cn[i] = in ? cnorm[c] : 0.f;
+        d[i] = in ? __double_as_longlong(dist[c]) : 0;
+        ci[i] = in ? cidx[c] : 0;
+      }
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        const int c = threadIdx.x + (k0 + i) * kPlaceThreads;
+        const bool in = ((word[i] >> lane) & 1u) && !outside(c, cj[i], cn[i]);
+        if (in) closer((unsigned)((unsigned long long)d[i] >> 32), (unsigned)d[i], (unsigned)ci[i], c);
+        const unsigned now = __ballot_sync(0xffffffffu, in);
+        if (lane == 0 && now != word[i]) alive[(k0 + i) * kWarps + wid] = now;
       }
     }
-    // no barrier needed here: warp 0 read red_* before the barrier above, and
-    // the shared plane is rewritten only after the next iteration's first
-    // barrier, which every thread reaches after this pass
+    __syncwarp();
+  }
+  __syncthreads();  // placed_idx
+  // the planes' rows, a warp each
+  const double* gd = reinterpret_cast<const double*>(v.s_d32);
+  for (int f = wid; f < placed; f += kWarps) {
+    const int bc = v.placed_idx[g * v.n_f + f];
+    const long long row = (long long)g * v.m_cap + m0 + f;
+    if (lane < n) v.A[row * n + lane] = ga[(long long)lane * np + bc];
+    if (lane == 0) {
+      v.b[row] = v.gb[co + bc];
+      v.placed_delta[g * v.n_f + f] = gd[co + bc];
+    }
   }
   if (threadIdx.x == 0) {
+    st.m = m0 + placed;
     st.n_placed = placed;
     st.planes += placed;
-    if (s_stop == 2) {
+    if (stop == 2) {
       st.status = SEG_IN_COLLISION;
       st.rounds = st.k;
-    } else if (s_stop == 3) {
+    } else if (stop == 3) {
       st.status = SEG_CAPACITY;
       st.rounds = st.k;
     }
@@ -553,7 +637,15 @@ __device__ __forceinline__ void place_segment(const BatchView& v) {
 }
 
 template <int NDOF, bool CLOSE>
-__global__ void __launch_bounds__(1024) k_round_place(BatchView v) {
+__global__ void __launch_bounds__(kPlaceThreads) k_round_place(BatchView v) {
+  // the next round's test size (FP64 logarithm) beside the placement, which
+  // leaves the FP64 unit idle, for the block that closes the round
+  __shared__ int s_size[2];
+  if (CLOSE && threadIdx.x == blockDim.x - 1) {
+    const int k = v.st[blockIdx.x].k + 1;
+    s_size[0] = k;
+    s_size[1] = round_test_size(k, v.eps, v.delta, v.tau);
+  }
   place_segment<NDOF>(v);
   if constexpr (CLOSE) {
     // every block reports when its segment is placed; the last one closes
@@ -568,7 +660,7 @@ __global__ void __launch_bounds__(1024) k_round_place(BatchView v) {
     if (s_last) {
       __threadfence();
       if (threadIdx.x == 0) v.summary->left_place = 0;
-      round_close_block(v);
+      round_close_block(v, s_size);
     }
   }
 }
@@ -803,11 +895,11 @@ cudaError_t launch_round_place(const BatchView& v, cudaStream_t s, bool close) {
     if (close) {
       err = set_smem(k_round_place<ND, true>, smem);
       if (err != cudaSuccess) return err;
-      k_round_place<ND, true><<<v.B, 1024, smem, s>>>(v);
+      k_round_place<ND, true><<<v.B, kPlaceThreads, smem, s>>>(v);
     } else {
       err = set_smem(k_round_place<ND, false>, smem);
       if (err != cudaSuccess) return err;
-      k_round_place<ND, false><<<v.B, 1024, smem, s>>>(v);
+      k_round_place<ND, false><<<v.B, kPlaceThreads, smem, s>>>(v);
     }
   });
   return cudaGetLastError();

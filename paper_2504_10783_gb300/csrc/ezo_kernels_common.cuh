@@ -500,8 +500,9 @@ __device__ __forceinline__ int round_test_size(int k, double eps, double delta, 
 }
 
 // Round size of every active segment and the round's list of sample tiles
-// (block-wide exclusive scan over the segments). Runs in one block.
-__device__ __forceinline__ void round_begin_block(const BatchView& v) {
+// (block-wide exclusive scan over the segments). Runs in one block. size, if
+// given, is (k, M_k) of one round.
+__device__ __forceinline__ void round_begin_block(const BatchView& v, const int* size = nullptr) {
   __shared__ int warp_sum[32];
   __shared__ int carry;
   if (threadIdx.x == 0) carry = 0;
@@ -520,7 +521,7 @@ __device__ __forceinline__ void round_begin_block(const BatchView& v) {
         st.n_placed = 0;
         tiles = (st.n_samples + kTile - 1) / kTile;
       } else if (st.status == SEG_ACTIVE) {
-        const int M = round_test_size(st.k, v.eps, v.delta, v.tau);
+        const int M = size && size[0] == st.k ? size[1] : round_test_size(st.k, v.eps, v.delta, v.tau);
         int S = M > st.n_p ? M : st.n_p;
         if (S > st.s_cap) S = st.s_cap;  // capacity is sized for M at N_it; never hit
         st.m_test = M;
@@ -574,14 +575,14 @@ __device__ __forceinline__ void round_begin_block(const BatchView& v) {
 // active segment that reached N_it stops (Sec. IV-C), the others go to round
 // k + 1, the next round's sample tiles are listed, and the round summary (and
 // a graph's WHILE condition) is set.
-__device__ __forceinline__ void round_close_block(const BatchView& v) {
+__device__ __forceinline__ void round_close_block(const BatchView& v, const int* size = nullptr) {
   __shared__ int s_active;
   if (threadIdx.x == 0) s_active = 0;
   __syncthreads();
   const int act = round_end_segments(v);
   if (act) atomicAdd(&s_active, act);
   __syncthreads();
-  round_begin_block(v);
+  round_begin_block(v, size);
   __syncthreads();
   if (threadIdx.x == 0) round_summary_close(v, s_active);
 }
