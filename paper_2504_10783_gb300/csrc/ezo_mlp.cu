@@ -91,8 +91,8 @@ struct ezo_surrogate {
   uint8_t *wimg = nullptr, *wtimg = nullptr;
   int* tc_err = nullptr;
   float* loss = nullptr;
-  // one block for a training batch of up to cap rows: operand images,
-  // pre-activations, the partial sums of the gradients
+  // one block for a training batch of up to cap rows: operand images, the
+  // outputs' errors, the partial sums of the gradients
   int cap = 0;
   uint8_t* train = nullptr;
 };
@@ -105,8 +105,8 @@ int blocks_for(long long n, int t) { return (int)std::max<long long>(1, std::min
 
 // The training block's parts for `rows` batch rows.
 struct TrainBufs {
-  uint8_t *Xt, *H1, *H2, *H1t, *H2t, *H3t, *dZ3, *dZ2, *dZ1t, *dZ2t, *dZ3t;
-  float *Z1, *Z2, *Z3, *part, *ws;
+  uint8_t *Xt, *H1t, *H2t, *H3t, *dZ1t, *dZ2t, *dZ3t;
+  float *e, *part, *ws;
   size_t bytes;
 };
 TrainBufs train_bufs(uint8_t* base, int rows) {
@@ -119,8 +119,8 @@ TrainBufs train_bufs(uint8_t* base, int rows) {
     return p;
   };
   b.Xt = take(tiles * 128 * 128);
-  for (uint8_t** p : {&b.H1, &b.H2, &b.H1t, &b.H2t, &b.H3t, &b.dZ3, &b.dZ2, &b.dZ1t, &b.dZ2t, &b.dZ3t}) *p = take(op);
-  for (float** p : {&b.Z1, &b.Z2, &b.Z3}) *p = reinterpret_cast<float*>(take(2 * op));
+  for (uint8_t** p : {&b.H1t, &b.H2t, &b.H3t, &b.dZ1t, &b.dZ2t, &b.dZ3t}) *p = take(op);
+  b.e = reinterpret_cast<float*>(take(tiles * 128 * sizeof(float)));
   b.ws = reinterpret_cast<float*>(take(tiles * kMlpWeights * sizeof(float)));
   b.part = reinterpret_cast<float*>(take(sizeof(float) * kOutBlocks * kOutPart));
   b.bytes = at;
@@ -147,30 +147,17 @@ cudaError_t train_step(ezo_surrogate* S, const float* q, long long ldq, const fl
   cudaError_t e = ensure_train_cap(S, B, s);
   if (e != cudaSuccess) return e;
   const TrainBufs b = train_bufs(S->train, S->cap);
-  LayerArgs a{};
-  a.rows = B;
-  a.err = S->tc_err;
-  a.q = q; a.ldq = ldq; a.n = S->n; a.Xt = b.Xt;
-  a.B = S->wimg; a.bias = S->p + kOffB1; a.Z = b.Z1; a.H = b.H1; a.Ht = b.H1t;
-  if ((e = mlp_layer_first(a, s)) != cudaSuccess) return e;
-  a.A = b.H1; a.B = S->wimg + kMlpChunk; a.bias = S->p + kOffB2; a.Z = b.Z2; a.H = b.H2; a.Ht = b.H2t;
-  if ((e = mlp_layer_forward(a, s)) != cudaSuccess) return e;
-  a.A = b.H2; a.B = S->wimg + 5 * kMlpChunk; a.bias = S->p + kOffB3; a.Z = b.Z3; a.H = nullptr; a.Ht = b.H3t;
-  if ((e = mlp_layer_forward(a, s)) != cudaSuccess) return e;
-  const OutputArgs o{b.H3t, b.Z3, S->p + kOffW4, S->p + kOffB4, t, B, b.dZ3, b.dZ3t, b.part};
-  if ((e = mlp_output(o, s)) != cudaSuccess) return e;
-  // dZ2 = (dZ3 W3) SiLU'(Z2), dZ1 = (dZ2 W2) SiLU'(Z1)
-  a.A = b.dZ3; a.B = S->wtimg + 4 * kMlpChunk; a.Z = b.Z2; a.H = b.dZ2; a.Ht = b.dZ2t;
-  if ((e = mlp_layer_backward(a, s)) != cudaSuccess) return e;
-  a.A = b.dZ2; a.B = S->wtimg; a.Z = b.Z1; a.H = nullptr; a.Ht = b.dZ1t;
-  if ((e = mlp_layer_backward(a, s)) != cudaSuccess) return e;
-  const WgradArgs w{b.Xt, b.H1t, b.H2t, b.dZ1t, b.dZ2t, b.dZ3t, B, b.ws, S->tc_err};
+  const ChainArgs c{B, q, ldq, S->n, t, S->wimg, S->wtimg, {S->p + kOffB1, S->p + kOffB2, S->p + kOffB3},
+                    S->p + kOffW4, S->p + kOffB4, b.Xt, {b.H1t, b.H2t, b.H3t, b.dZ3t, b.dZ2t, b.dZ1t}, b.e, S->tc_err};
+  if ((e = mlp_chain(c, s)) != cudaSuccess) return e;
+  const WgradArgs w{b.Xt, b.H1t, b.H2t, b.H3t, b.dZ1t, b.dZ2t, b.dZ3t, b.e, B, mlp_splits(B), mlp_out_blocks(B),
+                    b.ws, b.part, S->tc_err};
   if ((e = mlp_wgrad(w, s)) != cudaSuccess) return e;
   UpdateArgs u{};
-  u.ws = b.ws; u.splits = mlp_splits(B);
+  u.ws = b.ws; u.splits = w.splits;
   u.dZ1t = b.dZ1t; u.dZ2t = b.dZ2t; u.dZ3t = b.dZ3t;
   u.rows = B;
-  u.part = b.part; u.out_blocks = mlp_out_blocks(B);
+  u.part = b.part; u.out_blocks = w.out_blocks;
   u.g = S->g; u.loss = S->loss;
   u.p = S->p; u.m = S->m; u.v = S->v;
   u.img = S->wimg; u.timg = S->wtimg;

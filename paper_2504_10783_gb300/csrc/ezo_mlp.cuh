@@ -3,11 +3,9 @@
 //
 // An operand image holds rows of 64 BF16 values (one K-chunk) in the K-major
 // 128-byte swizzled layout of the tensor cores (sw128, ezo_tc.cuh), so a
-// range of its rows is one contiguous copy. Batch-major operands (features x
-// rows of the next product's K) are [tile of 128 batch rows][K-chunk of 64
-// features][128 rows]; transposed ones [chunk of 64 batch rows][feature];
-// weights [K-chunk][256 rows]. Pre-activations are FP32 [tile][feature][128
-// batch rows].
+// range of its rows is one contiguous copy. Transposed operands (batch rows
+// are the product's K) are [chunk of 64 batch rows][feature], weights
+// [K-chunk][256 rows].
 #pragma once
 
 #include <cuda_bf16.h>
@@ -24,38 +22,32 @@ constexpr int kMlpWeights = 2 * 65536 + 256 * 64;    // hidden weights: W3, W2, 
 constexpr long long kOffW1 = 0, kOffB1 = kOffW1 + 256 * 64, kOffW2 = kOffB1 + 256, kOffB2 = kOffW2 + 65536,
                     kOffW3 = kOffB2 + 256, kOffB3 = kOffW3 + 65536, kOffW4 = kOffB3 + 256, kOffB4 = kOffW4 + 256,
                     kNumParams = kOffB4 + 1;
-constexpr int kOutPart = 258;    // a block's partial sums: dw4, db4, loss
-constexpr int kOutBlocks = 256;  // blocks of the output layer's kernel at most
+constexpr int kOutPart = 258;    // partial sums of the output layer: dw4, db4, loss
+constexpr int kOutBlocks = 256;  // of them at most
 
 inline int mlp_splits(int rows) { return (rows + 127) / 128; }
 inline int mlp_out_blocks(int rows) { return rows / 8 < kOutBlocks ? rows / 8 : kOutBlocks; }
 
-struct LayerArgs {
-  const uint8_t* A;   // batch-major image of the input (not the first layer)
-  const uint8_t* B;   // weight image (backward: the transposed one)
+struct ChainArgs {
   int rows;           // batch rows, a multiple of 64
-  const float* bias;  // forward
-  float* Z;           // pre-activations: written forward, read backward
-  uint8_t* H;         // batch-major image of the result, or null
-  uint8_t* Ht;        // transposed image of the result
-  const float* q;     // first layer: configurations, value j of row i at q[j * ldq + i]
+  const float* q;     // configurations, value j of row i at q[j * ldq + i]
   long long ldq;
   int n;
-  uint8_t* Xt;        // first layer: transposed feature image, 64 features a chunk
+  const float* t;     // targets
+  const uint8_t *img, *timg;  // weight images
+  const float *bias[3], *w4, *b4;
+  uint8_t *Xt;        // transposed feature image, 64 features a chunk
+  uint8_t* Ht[6];     // transposed images of H1, H2, H3, dZ3, dZ2, dZ1
+  float* e;           // output minus target
   int* err;           // set when a bounded wait gave up
 };
 struct WgradArgs {
-  const uint8_t *Xt, *H1t, *H2t, *dZ1t, *dZ2t, *dZ3t;
-  int rows;
-  float* ws;  // [128 batch rows][kMlpWeights]
+  const uint8_t *Xt, *H1t, *H2t, *H3t, *dZ1t, *dZ2t, *dZ3t;
+  const float* e;
+  int rows, splits, out_blocks;
+  float* ws;    // [128 batch rows][kMlpWeights]
+  float* part;  // [out_blocks][kOutPart]
   int* err;
-};
-struct OutputArgs {
-  const uint8_t* H3t;
-  const float *Z3, *w4, *b4, *t;
-  int rows;
-  uint8_t *dZ3, *dZ3t;
-  float* part;  // [block][kOutPart]
 };
 struct UpdateArgs {
   const float* ws;
@@ -71,10 +63,7 @@ struct UpdateArgs {
   uint8_t *img, *timg;  // weight images
 };
 
-cudaError_t mlp_layer_first(const LayerArgs& g, cudaStream_t s);
-cudaError_t mlp_layer_forward(const LayerArgs& g, cudaStream_t s);
-cudaError_t mlp_layer_backward(const LayerArgs& g, cudaStream_t s);
-cudaError_t mlp_output(const OutputArgs& g, cudaStream_t s);
+cudaError_t mlp_chain(const ChainArgs& g, cudaStream_t s);
 cudaError_t mlp_wgrad(const WgradArgs& g, cudaStream_t s);
 cudaError_t mlp_update(const UpdateArgs& u, cudaStream_t s);
 cudaError_t mlp_weight_images(const float* p, void* img, void* timg, cudaStream_t s);
