@@ -623,8 +623,9 @@ def measure_checker(ezo, torch, robot, env, rd, stream, flush, props, sm_max, fl
                                        "self pair, plus the kinematics); the obstacle pairs of the first "
                                        "static_spheres robot spheres, "
                                        "on the fixed base frame and clear of every obstacle, are decided once "
-                                       "per obstacle set, so the pair tests run per configuration come to "
-                                       "flops_per_config_tested",
+                                       "per obstacle set, which leaves flops_per_config_tested; the obstacle grid "
+                                       "decides most of either count's pairs without evaluating them, so both "
+                                       "fractions are label rates in counted pairs and can exceed 1",
                          "traffic": traffic},
             "paper_context": "paper: ~8.6 M configs/s, Franka (1187 pairs), RTX 3090, same batch size",
             "launches": reps + 3}

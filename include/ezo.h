@@ -152,12 +152,12 @@ void ezo_env_free(ezo_env* env);
  * below the squared sum of radii), else 0. Robot spheres on the fixed base
  * frame have the same centre for every configuration: when they all clear
  * every obstacle sphere by more than 1e-4 m (checked on the host at each
- * call) their obstacle pairs are not swept again; the flags are the same.
+ * call) their obstacle pairs are not tested again; the flags are the same.
  * Stream-ordered, asynchronous.
  * lanes_per_config selects 1, 2, 4 or 8 cooperating lanes per configuration
- * (0 = choose from N, among the counts that fit). Each group of lanes keeps
- * its sphere centres in shared memory, so large robots with many obstacles
- * need more lanes: at the maximum sizes (256 spheres, 4096 obstacles) only 4
+ * (0 = choose from N, among the counts that fit). What fits is decided as if
+ * each group of lanes kept its sphere centres, and the block the obstacles,
+ * in shared memory, so large robots with many obstacles need more lanes: at the maximum sizes (256 spheres, 4096 obstacles) only 4
  * and 8 fit. Errors: EZO_ERR_INVALID_ARG (null handle, N < 0, ldq < N, bad
  * lanes value, spheres and obstacles beyond shared memory at that lanes
  * value; nothing is launched), EZO_ERR_CUDA (launch failure). */
@@ -656,7 +656,7 @@ ezo_status ezo_probe_fp32_fma(double* tflops, void* cuda_stream);
  * used for rooflines. */
 double ezo_check_flops(const ezo_robot* robot, const ezo_env* env);
 /* The robot spheres (the first ones, on the fixed base frame) whose obstacle
- * pairs the checker's sweep decides once for this obstacle set instead of per
+ * pairs the checker decides once for this obstacle set instead of per
  * configuration: every such sphere clears every obstacle sphere by more than
  * 1e-4 m, whole chunks of eight spheres; 0 when none qualifies or for NULL
  * handles. Their 8 x count x n_obs flops per configuration are part of

@@ -146,8 +146,8 @@ struct ezo_env {
 // them; the clearance is checked in
 // FP64 on the FP32 values the kernels use, against 1e-4 m, far above the
 // rounding band of the FP32 test (the kernels place a base sphere exactly at
-// its FP32 local coordinates), so every label is what the full sweep gives.
-// Any base sphere within 1e-4 m of an obstacle keeps the full sweep.
+// its FP32 local coordinates), so every label is what all spheres' tests give.
+// With a base sphere within 1e-4 m of an obstacle all spheres are tested.
 static int sweep_first(const ezo_robot* r, const ezo_env* e, int cut) {
   if (cut == 0) return 0;
   // apart along an axis by the box around the base spheres and the one around

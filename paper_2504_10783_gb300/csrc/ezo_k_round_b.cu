@@ -838,7 +838,7 @@ cudaError_t launch_round_bisect_box(const BatchView& v, int T, int grid, cudaStr
   return cudaGetLastError();
 }
 #else
-// T = 16 or 32 lanes per candidate take the wide check (sphere scenes; box
+// T = 16 or 32 lanes per candidate are for sphere scenes (box
 // scenes run at 8)
 cudaError_t launch_round_bisect(const BatchView& v, int T, int grid, cudaStream_t s) {
   if (v.n_rbox || v.max_ebox) return launch_round_bisect_box(v, T > 8 ? 8 : T, grid, s);
