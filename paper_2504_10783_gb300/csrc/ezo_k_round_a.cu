@@ -159,11 +159,12 @@ __global__ void __launch_bounds__(128) k_round_check(BatchView v, int stage_lb) 
     queue_leave(v, q, &v.summary->left_check, units);
     return;
   }
-  // the bounds are copied to shared memory (where the launch has room) when a
-  // block of this round looks up enough of them, the flat check's rule: a
-  // single segment's round of 1000 samples copied 32 KB in each of 32 blocks
-  // for 400 lookups (16.6 -> 13.9 us; a path's and 24 paths' rounds copy them as
-  // before)
+  // collide_group's bounds are copied to shared memory (where the launch has
+  // room) when a block of this round looks up enough of them, the flat check's
+  // rule. collide_lane reads them through L1: without the copy six blocks of a
+  // round are resident on an SM instead of four, and 782 units are one wave (a
+  // path's check 28 -> 24.5 us a round, 24 paths' 36 -> 30; a segment's 1000
+  // samples 16.6 us copied, 13.9 not)
   const int per_block = (units + (int)gridDim.x - 1) / (int)gridDim.x * (128 / T);
   const bool stage = stage_lb && (long long)per_block * v.nsp_pad >= 4096;
   Checker<NDOF, T, BOX, LANE> chk(rs, smem4, v.robot, v.max_ebox, stage);
@@ -356,7 +357,7 @@ cudaError_t launch_round_check_box(const BatchView& v, int T, int grid, cudaStre
 cudaError_t launch_round_check(const BatchView& v, int T, int grid, cudaStream_t s) {
   if (v.n_rbox || v.max_ebox) return launch_round_check_box(v, T, grid, s);
   cudaError_t err = cudaSuccess;
-  const CheckPlan pl = check_plan(v.nsp_pad, v.n, 128, T, v.n_rbox, v.max_ebox, v.lane, true);
+  const CheckPlan pl = check_plan(v.nsp_pad, v.n, 128, T, v.n_rbox, v.max_ebox, v.lane, v.lane < 0);
   EZO_DISPATCH_NDOF(v.n, EZO_DISPATCH_T(T, EZO_DISPATCH_LANE(pl.lane, {
     auto kern = k_round_check<ND, TT, false, LL>;
     err = set_smem(kern, pl.smem);
