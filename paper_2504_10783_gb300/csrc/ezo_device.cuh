@@ -1199,7 +1199,7 @@ __device__ __forceinline__ void pair_distance(float cx, float cy, float cz, floa
 // the sphere of the smallest one against every obstacle, a few each. Links of
 // self pairs are taken sphere by sphere where the other segment's distance
 // allows less than the best. Of the 2788 pairs of the 7-DOF arm with 64
-// obstacles some 90 are left: 131071 distances 0.416 -> 0.137 ms (one lane a
+// obstacles some 90 are left: 131071 distances 0.416 -> 0.139 ms (one lane a
 // configuration over all pairs before), 2000 0.130 -> 0.021; among 1024
 // obstacles 131071 7.9 -> 0.88 ms. Bound by instruction issue; the chain is a
 // quarter of it.
@@ -1214,8 +1214,7 @@ __device__ __forceinline__ float distance_lane(const float (&q)[NDOF], const Lan
   float best = cap;
   bool left = false;  // some sphere of this lane keeps a bound
   // from the arm's tip: where the spheres near the obstacles usually are
-  const int first = e.n_obs > 0 ? e.s_first : ns;  // base-frame spheres are in cap (k_sd_lane)
-  for (int s = ns - 1 - lg; s >= first; s -= T) {
+  for (int s = ns - 1 - lg; s >= 0 && e.n_obs > 0; s -= T) {
     const int f = frame[s];
     const LanePose P = lane_pose<T>(ls.slot[f], general, mine, stride);
     const float r = sph[s].w;
@@ -1273,7 +1272,7 @@ __device__ __forceinline__ float distance_lane(const float (&q)[NDOF], const Lan
   while (__any_sync(0xffffffffu, left)) {
     float b = 3.0e38f;
     int s = 0;
-    for (int k = ns - 1 - lg; k >= first; k -= T)
+    for (int k = ns - 1 - lg; k >= 0 && e.n_obs > 0; k -= T)
       if (bnd[k] < b) b = bnd[k], s = k;
 #pragma unroll
     for (int o = 1; o < T; o <<= 1) {

@@ -86,11 +86,7 @@ __global__ void __launch_bounds__(128) k_sd_flat(const RobotDev* __restrict__ ro
   }
 }
 
-// Signed distances by groups of T lanes (distance_lane). The base-frame
-// spheres that the collision tests leave out (EnvDev::s_first) stand still, so
-// a block measures them once and its configurations start from the smallest
-// of their distances: 131071 distances of the 7-DOF arm (11 of its 40 spheres)
-// 141 -> 137 us a call.
+// Signed distances by groups of T lanes (distance_lane).
 template <int NDOF, int T>
 __global__ void __launch_bounds__(128) k_sd_lane(const RobotDev* __restrict__ robot, EnvDev env, WideGrid wide,
                                                  const float* __restrict__ q, long long ldq, long long N,
@@ -101,20 +97,7 @@ __global__ void __launch_bounds__(128) k_sd_lane(const RobotDev* __restrict__ ro
   chk.set_env(env);
   // the groups' bounds follow the check's shared memory
   float* bnd = reinterpret_cast<float*>(chk.frame + robot->n_spheres_pad) + (threadIdx.x / T) * robot->n_spheres_pad;
-  __shared__ float base[4];
   __syncthreads();
-  if (env.s_first > 0 && env.n_obs > 0) {
-    for (int p = threadIdx.x; p < env.s_first * env.n_obs; p += blockDim.x) {
-      const int s = p / env.n_obs;
-      const float4 l = chk.gs.sph[s];
-      pair_distance(l.x, l.y, l.z, l.w, __ldg(env.obs + (p - s * env.n_obs)), cap);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cap = fminf(cap, __shfl_xor_sync(0xffffffffu, cap, o));
-    if ((threadIdx.x & 31) == 0) base[threadIdx.x >> 5] = cap;
-    __syncthreads();
-    cap = fminf(fminf(base[0], base[1]), fminf(base[2], base[3]));
-  }
   const int groups = blockDim.x / T, gi = threadIdx.x / T;
   for (long long base = (long long)blockIdx.x * groups; base < N; base += (long long)gridDim.x * groups) {
     const long long i = base + gi;
