@@ -1,6 +1,6 @@
 """Signed distances where spheres on the fixed base frame count: nearest of
-all, near one obstacle of many, touching, and with no obstacle. Within the 2e-5 m of the other signed
-distance tests."""
+all, near one obstacle of many, touching, and with no obstacle. Within the 2e-5 m
+of the other signed distance tests."""
 import numpy as np
 import pytest
 
