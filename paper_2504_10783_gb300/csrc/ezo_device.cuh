@@ -825,8 +825,9 @@ __device__ __forceinline__ void lane_world(const LanePose& P, int axis, const fl
 
 // The self pairs from the kept poses, links lg, lg + T, ..: the squared
 // distance of the two segments (any point pair on them bounds it from above,
-// and the pair found is the nearest to second order in its rounding, which
-// r2's margin covers); the pairs of links nearer than their radii one by one.
+// and the pair found is the nearest to second order in its rounding and in the
+// angle of nearly parallel segments, which r2's margin covers); the pairs of
+// links nearer than their radii one by one.
 template <int T>
 __device__ __forceinline__ bool links_hit(const LaneSmem& ls, const float4* __restrict__ sph,
                                           const float2* __restrict__ sa, const float* mine, int stride, int lg) {
@@ -857,14 +858,22 @@ __device__ __forceinline__ bool links_hit(const LaneSmem& ls, const float4* __re
     const float uv = fmaf(ux, vx, fmaf(uy, vy, uz * vz));
     const float ur = fmaf(ux, rx, fmaf(uy, ry, uz * rz)), vr = fmaf(vx, rx, fmaf(vy, ry, vz * rz));
     const float det = fmaf(uu, vv, -uv * uv);
-    // s on the first segment for the nearest points of the two lines (0 when
-    // they are parallel), t the nearest on the second to it, then s to t
+    // from s on the first segment: t the nearest on the second to it, then s to t
     const float iu = uu > 0.f ? __fdividef(1.f, uu) : 0.f, iv = vv > 0.f ? __fdividef(1.f, vv) : 0.f;
-    float s = det > 1e-6f * uu * vv ? __saturatef(__fdividef(fmaf(uv, vr, -ur * vv), det)) : 0.f;
-    const float t = __saturatef(fmaf(s, uv, vr) * iv);
-    s = __saturatef(fmaf(t, uv, -ur) * iu);
-    const float dx = rx + fmaf(s, ux, -t * vx), dy = ry + fmaf(s, uy, -t * vy), dz = rz + fmaf(s, uz, -t * vz);
-    if (!(fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < L.r2)) continue;
+    auto squared = [&](float s) {
+      const float t = __saturatef(fmaf(s, uv, vr) * iv);
+      s = __saturatef(fmaf(t, uv, -ur) * iu);
+      const float dx = rx + fmaf(s, ux, -t * vx), dy = ry + fmaf(s, uy, -t * vy), dz = rz + fmaf(s, uz, -t * vz);
+      return fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+    };
+    // Start at the nearest point of the two lines. Nearly parallel segments
+    // (an angle a up to 1e-3 by det) are nearest at an end of their overlap,
+    // which the two ends of the first lead to, or within (a |u|)^2 / 4 of the
+    // squared distance there, a fortieth of r2's margin.
+    float d2;
+    if (det > 1e-6f * uu * vv) d2 = squared(__saturatef(__fdividef(fmaf(uv, vr, -ur * vv), det)));
+    else d2 = fminf(squared(0.f), squared(1.f));
+    if (!(d2 < L.r2)) continue;
     for (int j = L.b0; j < L.b0 + L.nb; ++j) {
       const float4 lj = sph[j];
       float cx, cy, cz;
