@@ -237,8 +237,12 @@ cudaError_t launch_check_flat(const RobotDev* robot, int n, int nsp_pad, int n_r
   if (n_rbox || env.n_box) return launch_check_flat_box(robot, n, nsp_pad, n_rbox, env, q, ldq, N, flags, T, grid_cap, s);
   if (N <= 0) return cudaSuccess;
   cudaError_t err = cudaSuccess;
-  // 256 threads where a block shares the staged bounds and has work for them
-  const int threads = lane >= 0 && N * T >= 256ll * 152 ? 256 : 128;
+  // 256 threads where a block shares the staged bounds, has work for them and
+  // holds the poses of all of them (one lane of 16 joints with general spheres
+  // on 17 frames takes 880 bytes); the acceptance rule counts 128
+  const bool wide = lane >= 0 && N * T >= 256ll * 152 &&
+                    lane_smem_layout(nsp_pad, n, 256, T, lane, false) <= kSmemBudget;
+  const int threads = wide ? 256 : 128;
   const long long groups = threads / T;
   long long grid = (N + groups - 1) / groups;
   if (grid_cap > 0 && grid > grid_cap) grid = grid_cap;
