@@ -166,10 +166,15 @@ ezo_status ezo_check_collision(const ezo_robot* robot, const ezo_env* env, const
 
 /* Signed distance per configuration: min over the same pairs of
  * ||c_i - c_j|| - r_i - r_j in FP32 (negative iff in collision). Used to
- * label data and to bound ambiguous decisions. Stream-ordered.
+ * label data and to bound ambiguous decisions. Stream-ordered, asynchronous.
+ * The first call of at least 16384 configurations on an obstacle set, outside
+ * a capture, allocates a grid of its own for the set (3 MB for 1024
+ * obstacles, freed with it) and queues its build on the call's stream; calls
+ * on other streams wait for the build on the device.
  * EZO_ERR_INVALID_ARG when the robot or env has boxes, or when its spheres
- * and obstacles exceed the kernel's shared memory (one lane per
- * configuration: (spheres + 1) x 64 centres plus the obstacles). */
+ * and obstacles exceed shared memory by the rule of one lane per
+ * configuration: (spheres + 1) x 64 centres plus the obstacles (the kernels
+ * need less). */
 ezo_status ezo_signed_distance(const ezo_robot* robot, const ezo_env* env, const float* q_dev, int64_t N,
                                int64_t ldq, float* sd_dev, void* cuda_stream);
 

@@ -128,9 +128,13 @@ struct ezo_env {
   GridBuild build{};  // what the grid was built from
   double lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0}, ext = 0.0;
   bool gridded = false;
+  // signed_distance_grid's, under wide_mu
+  enum WideState { kWideNone, kWideQueued, kWideComplete, kWideNoMemory };
   mutable std::mutex wide_mu;
+  mutable WideState wide_state = kWideNone;
   mutable char* d_wide = nullptr;
   mutable WideGrid wide_full{};
+  mutable cudaEvent_t wide_ready = nullptr;  // recorded behind the build
   int n_obs = 0, n_obs_pad = 0;
   float4* d_box = nullptr;  // obstacle boxes, 4 float4 each
   int n_box = 0;
@@ -138,6 +142,7 @@ struct ezo_env {
   EnvDev dev() const { return EnvDev{d_obs, n_obs, n_obs_pad, d_box, n_box, 0, grid}; }
   EnvDev dev_for(const ezo_robot* r) const;
   WideGrid signed_distance_grid(long long N, cudaStream_t s) const;
+  bool build_wide(cudaStream_t s) const;
 };
 
 // The robot spheres on the fixed base frame sit where they are for every
@@ -182,52 +187,66 @@ static void wide_params(WideGrid& w, const GridBuild& b, float inv, double r_obs
 }
 
 // The wide grid for N signed distances on stream s. The first call of at
-// least 16384 builds the wide grid (about 0.15 ms for 64 obstacles, 0.5 ms
-// for 1024, of which the allocation is most; 131071 distances of the 7-DOF
-// arm take 0.36 ms without it and 0.136 ms with it), unless s is capturing or
-// there is no memory for it. The build is complete before the lock is given
-// up, so calls on other streams and threads may use it at once.
+// least 16384 allocates it and queues its build on s (about 0.15 ms for 64
+// obstacles, 0.5 ms for 1024, of which the allocation is most; 131071
+// distances of the 7-DOF arm take 0.36 ms without it and 0.136 ms with it),
+// unless s is capturing or there is no memory for it. Nothing here waits on
+// the host: until the build has completed, calls on other streams wait for it
+// on the device, and calls on a capturing stream, which cannot, take the
+// coarse grid's bounds.
 WideGrid ezo_env::signed_distance_grid(long long N, cudaStream_t s) const {
   if (!gridded) return wide;
   std::lock_guard<std::mutex> lock(wide_mu);
-  if (!d_wide) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (N < 16384 || cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-      (void)cudaGetLastError();
-      return wide;
-    }
-    GridBuild b = build;
-    const float inv = (float)((kGridC - 1) / (3.0 * ext));
-    for (int k = 0; k < 3; ++k) {
-      b.k0[k] = (int)std::floor((lo[k] - ext) * inv);
-      b.n[k] = std::min(kGridC, (int)std::floor((hi[k] + ext) * inv) - b.k0[k] + 1);
-    }
-    b.sub = 1;
-    b.h = (float)(1.0 / inv);
-    b.step = (float)(2.0 * ext / 255.0);
-    b.far = 3.0e38f;
-    b.ids_cap = 262144u + 1024u * (unsigned)n_obs;
-    const size_t o_cell = 256, cells = (size_t)b.n[2] * kGridC * kGridC, o_ids = o_cell + cells * sizeof(unsigned long long);
-    char* mem = nullptr;
-    if (cudaMalloc(&mem, o_ids + b.ids_cap * sizeof(uint16_t)) == cudaSuccess) {
-      b.used = (unsigned*)mem;
-      b.lb = nullptr;
-      b.cell = (unsigned long long*)(mem + o_cell);
-      b.ids = (uint16_t*)(mem + o_ids);
-      if (cudaMemsetAsync(mem, 0, 256, s) == cudaSuccess && launch_grid_build(b, s) == cudaSuccess &&
-          cudaStreamSynchronize(s) == cudaSuccess) {
-        wide_full = WideGrid{};
-        wide_full.cell = b.cell;
-        wide_full.ids = b.ids;
-        wide_params(wide_full, b, inv, wide.r_obs);
-        d_wide = mem;
-      } else {
-        cudaFree(mem);
-      }
-    }
-    (void)cudaGetLastError();
+  if (wide_state == kWideComplete) return wide_full;
+  if (wide_state == kWideNoMemory || (wide_state == kWideNone && N < 16384)) return wide;
+  RelaxedCapture relaxed;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool capturing = cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  bool use = false;
+  if (wide_state == kWideQueued) {
+    use = cudaEventQuery(wide_ready) == cudaSuccess;
+    if (use) wide_state = kWideComplete;
+    else use = !capturing && cudaStreamWaitEvent(s, wide_ready, 0) == cudaSuccess;
+  } else if (!capturing) {
+    use = build_wide(s);
+    wide_state = use ? kWideQueued : kWideNoMemory;
   }
-  return d_wide ? wide_full : wide;
+  (void)cudaGetLastError();
+  return use ? wide_full : wide;
+}
+
+// Queues the wide grid's build on s; false when a call failed.
+bool ezo_env::build_wide(cudaStream_t s) const {
+  GridBuild b = build;
+  const float inv = (float)((kGridC - 1) / (3.0 * ext));
+  for (int k = 0; k < 3; ++k) {
+    b.k0[k] = (int)std::floor((lo[k] - ext) * inv);
+    b.n[k] = std::min(kGridC, (int)std::floor((hi[k] + ext) * inv) - b.k0[k] + 1);
+  }
+  b.sub = 1;
+  b.h = (float)(1.0 / inv);
+  b.step = (float)(2.0 * ext / 255.0);
+  b.far = 3.0e38f;
+  b.ids_cap = 262144u + 1024u * (unsigned)n_obs;
+  const size_t o_cell = 256, cells = (size_t)b.n[2] * kGridC * kGridC, o_ids = o_cell + cells * sizeof(unsigned long long);
+  char* mem = nullptr;
+  if (cudaMalloc(&mem, o_ids + b.ids_cap * sizeof(uint16_t)) != cudaSuccess) return false;
+  b.used = (unsigned*)mem;
+  b.lb = nullptr;
+  b.cell = (unsigned long long*)(mem + o_cell);
+  b.ids = (uint16_t*)(mem + o_ids);
+  if (cudaEventCreateWithFlags(&wide_ready, cudaEventDisableTiming) != cudaSuccess ||
+      cudaMemsetAsync(mem, 0, 256, s) != cudaSuccess || launch_grid_build(b, s) != cudaSuccess ||
+      cudaEventRecord(wide_ready, s) != cudaSuccess) {
+    cudaFree(mem);  // waits for what was queued
+    return false;
+  }
+  wide_full = WideGrid{};
+  wide_full.cell = b.cell;
+  wide_full.ids = b.ids;
+  wide_params(wide_full, b, inv, wide.r_obs);
+  d_wide = mem;
+  return true;
 }
 
 EnvDev ezo_env::dev_for(const ezo_robot* r) const {
@@ -714,6 +733,7 @@ void ezo_env_free(ezo_env* e) {
   if (!e) return;
   cudaFree(e->d_mem);
   cudaFree(e->d_wide);
+  if (e->wide_ready) cudaEventDestroy(e->wide_ready);
   cudaFree(e->d_box);
   delete e;
 }

@@ -16,6 +16,23 @@
 
 namespace ezo {
 
+// While in scope, this thread's allocations and event queries are allowed
+// beside a stream capture that any thread has begun in global mode; without
+// it they fail and invalidate that capture, which they have no part in.
+class RelaxedCapture {
+ public:
+  RelaxedCapture() { ok_ = cudaThreadExchangeStreamCaptureMode(&mode_) == cudaSuccess; }
+  ~RelaxedCapture() {
+    if (ok_) cudaThreadExchangeStreamCaptureMode(&mode_);
+  }
+  RelaxedCapture(const RelaxedCapture&) = delete;
+  RelaxedCapture& operator=(const RelaxedCapture&) = delete;
+
+ private:
+  cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+  bool ok_;
+};
+
 class BlockPool {
  public:
   explicit BlockPool(bool host) : host_(host) {}
