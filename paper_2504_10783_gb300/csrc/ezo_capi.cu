@@ -997,6 +997,7 @@ struct ezo_batch {
   SegState* d_st0 = nullptr;    // initial state, for resets
   double *d_A0 = nullptr, *d_b0 = nullptr;  // the domain, m0 rows: every segment's initial polytope
   char* mem = nullptr;  // one block of the device pool: all of the above
+  int dev = 0;          // the device it was taken on
   std::vector<double> v1h, v2h;
   BatchView view{};
   int T_check = 1, T_bisect = 4, split_below = 0;
@@ -1043,9 +1044,9 @@ ezo_status batch_free_device(ezo_batch* b) {
   for (void* p : ptrs)
     if (p) cudaFree(p);
   // work queued on the batch's buffers ends before they are handed on
-  if (b->mem) cudaDeviceSynchronize();
-  device_pool().give(b->mem);
-  host_pool().give(b->h_sum);
+  const bool idle = b->mem && device_idle(b->dev);
+  device_pool().give(b->mem, idle);
+  host_pool().give(b->h_sum, idle);
   for (auto e : b->events.ev) cudaEventDestroy(e);
   return EZO_OK;
 }
@@ -1515,7 +1516,8 @@ ezo_status ezo_batch_create(const ezo_robot* robot, int32_t n_env, const ezo_env
   };
   layout(nullptr);
   cudaError_t e = cudaSuccess;
-  b->mem = (char*)device_pool().take(total, &e);
+  e = cudaGetDevice(&b->dev);
+  if (e == cudaSuccess) b->mem = (char*)device_pool().take(total, &e);
   if (e == cudaSuccess) b->h_sum = (RoundSummary*)host_pool().take(sizeof(RoundSummary), &e);
   if (e != cudaSuccess) {
     batch_free_device(b);
@@ -2062,7 +2064,7 @@ extern "C++" __attribute__((visibility("hidden"))) ezo_status ezo_internal_batch
     std::memcpy(A.data(), host, sizeof(double) * A.size());
     std::memcpy(bv.data(), hb, sizeof(double) * bv.size());
   }
-  host_pool().give(host);
+  host_pool().give(host, e2 == cudaSuccess);
   return e == cudaSuccess ? EZO_OK : cuda_fail(e, "reading the polytopes");
 }
 
@@ -2323,7 +2325,7 @@ ezo_status ezo_check_path(const ezo_robot* robot, const ezo_env* env, const doub
   char *scratch = (char*)device_pool().take(bytes, &e), *host = nullptr;
   if (e == cudaSuccess) host = (char*)host_pool().take(bytes, &e);
   if (e != cudaSuccess) {
-    device_pool().give(scratch);
+    device_pool().give(scratch, true);
     return cuda_fail(e, "ezo_check_path");
   }
   std::memcpy(host, verts, vb);
@@ -2338,12 +2340,12 @@ ezo_status ezo_check_path(const ezo_robot* robot, const ezo_env* env, const doub
                           sm_count() * 32, s);
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(host + vb + ob, d_edge, (size_t)K, cudaMemcpyDeviceToHost, s);
-  // the blocks are given back only when nothing uses them any more
+  // the blocks are kept only when nothing uses them any more
   const cudaError_t done = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = done;
   if (e == cudaSuccess) std::memcpy(edge_flags, host + vb + ob, (size_t)K);
-  host_pool().give(host);
-  device_pool().give(scratch);
+  host_pool().give(host, done == cudaSuccess);
+  device_pool().give(scratch, done == cudaSuccess);
   if (e != cudaSuccess) return cuda_fail(e, "ezo_check_path");
   g_err.clear();
   return EZO_OK;

@@ -5,6 +5,7 @@
 // keeps at most kKeep blocks and kBytes bytes, only of sizes up to kMaxBlock,
 // hands a block out on the device it was made on and to one taker at a time,
 // and frees what it holds when the last robot, obstacle set and batch are gone.
+// A block whose work may not have completed is freed, not kept.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -32,6 +33,20 @@ class RelaxedCapture {
   cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
   bool ok_;
 };
+
+// Waits for everything queued on device `dev`, whichever device is current;
+// false when that could not be done.
+inline bool device_idle(int dev) {
+  int current = -1;
+  bool ok = cudaGetDevice(&current) == cudaSuccess && (current == dev || cudaSetDevice(dev) == cudaSuccess);
+  if (ok) {
+    RelaxedCapture relaxed;
+    ok = cudaDeviceSynchronize() == cudaSuccess;
+  }
+  if (current >= 0 && current != dev) cudaSetDevice(current);
+  if (!ok) (void)cudaGetLastError();
+  return ok;
+}
 
 class BlockPool {
  public:
@@ -73,8 +88,8 @@ class BlockPool {
     return p;
   }
 
-  // a block from take() whose work has completed
-  void give(void* p) {
+  // a block from take(); idle: its work has completed
+  void give(void* p, bool idle) {
     if (!p) return;
     {
       std::lock_guard<std::mutex> lock(mu_);
@@ -82,7 +97,7 @@ class BlockPool {
         if (out_[i].p == p) {
           const Block b = out_[i];
           out_.erase(out_.begin() + i);
-          if (b.bytes <= kMaxBlock && held_.size() < kKeep && total_ + b.bytes <= kBytes) {
+          if (idle && b.bytes <= kMaxBlock && held_.size() < kKeep && total_ + b.bytes <= kBytes) {
             held_.push_back(b);
             total_ += b.bytes;
             return;
