@@ -133,7 +133,11 @@ int32_t ezo_robot_dof(const ezo_robot* robot);
 
 /* -------------------------------------------------------------- obstacles --
  * Obstacle spheres (Sec. V-B: perceived voxels become circumscribing
- * spheres): n_obs rows (x, y, z, radius) of host FP64, n_obs <= 4096.
+ * spheres): n_obs rows (x, y, z, radius) of host FP64, n_obs <= 4096. The
+ * call builds the grid that collision tests look spheres up in and returns
+ * when it is complete; ezo_env_free waits for the device. Memory of freed
+ * sets, batches and path checks is kept for the next ones (at most 64 MB)
+ * until the last robot, obstacle set and batch are freed.
  * Errors: EZO_ERR_INVALID_ARG, EZO_ERR_CUDA. */
 ezo_status ezo_env_create(int32_t n_obs, const double* xyzr, ezo_env** out);
 /* Oriented obstacle boxes (at most 64): one row of 15 doubles per box,
@@ -388,7 +392,8 @@ ezo_status ezo_batch_write_samples(ezo_batch* batch, int32_t seg, const float* s
  * the path. Each call builds a batch (ezo_batch_create), runs it with the
  * batch kernels, copies the results into host objects owned by the caller
  * and frees the batch; it blocks until they are on the host. The device
- * memory is allocated and freed inside the call.
+ * memory is taken and given back inside the call (ezo_env_create says where
+ * to).
  *
  * Per-polytope statistics (the segment's outcome and work). */
 typedef struct {

@@ -120,8 +120,10 @@ struct ezo_robot {
 
 struct ezo_env {
   HandleCount alive;
-  // one block: obstacles, the grid's list counter, coarse bounds, cells, lists
+  // one block of the device pool: obstacles, the grid's list counter, coarse
+  // bounds, cells, lists
   char* d_mem = nullptr;
+  int device = 0;  // the device it was taken on
   float4* d_obs = nullptr;
   ObsGrid grid{};
   WideGrid wide{};  // the coarse collision grid; signed_distance_grid's own once it is built
@@ -187,10 +189,10 @@ static void wide_params(WideGrid& w, const GridBuild& b, float inv, double r_obs
 }
 
 // The wide grid for N signed distances on stream s. The first call of at
-// least 16384 allocates it and queues its build on s (about 0.15 ms for 64
-// obstacles, 0.5 ms for 1024, of which the allocation is most; 131071
-// distances of the 7-DOF arm take 0.36 ms without it and 0.136 ms with it),
-// unless s is capturing or there is no memory for it. Nothing here waits on
+// least 16384 takes a block for it and queues its build on s (0.02 ms for 64
+// obstacles and 0.12 ms for 1024, or 0.1 to 0.4 ms more where the pool has no
+// block; 131071 distances of the 7-DOF arm take 0.36 ms without it and 0.136
+// ms with it), unless s is capturing or there is no memory for it. Nothing here waits on
 // the host: until the build has completed, calls on other streams wait for it
 // on the device, and calls on a capturing stream, which cannot, take the
 // coarse grid's bounds.
@@ -229,8 +231,9 @@ bool ezo_env::build_wide(cudaStream_t s) const {
   b.far = 3.0e38f;
   b.ids_cap = 262144u + 1024u * (unsigned)n_obs;
   const size_t o_cell = 256, cells = (size_t)b.n[2] * kGridC * kGridC, o_ids = o_cell + cells * sizeof(unsigned long long);
-  char* mem = nullptr;
-  if (cudaMalloc(&mem, o_ids + b.ids_cap * sizeof(uint16_t)) != cudaSuccess) return false;
+  cudaError_t err = cudaSuccess;
+  char* mem = (char*)device_pool().take(o_ids + b.ids_cap * sizeof(uint16_t), &err);
+  if (!mem) return false;
   b.used = (unsigned*)mem;
   b.lb = nullptr;
   b.cell = (unsigned long long*)(mem + o_cell);
@@ -238,7 +241,7 @@ bool ezo_env::build_wide(cudaStream_t s) const {
   if (cudaEventCreateWithFlags(&wide_ready, cudaEventDisableTiming) != cudaSuccess ||
       cudaMemsetAsync(mem, 0, 256, s) != cudaSuccess || launch_grid_build(b, s) != cudaSuccess ||
       cudaEventRecord(wide_ready, s) != cudaSuccess) {
-    cudaFree(mem);  // waits for what was queued
+    device_pool().give(mem, false);  // freed, which waits for what was queued
     return false;
   }
   wide_full = WideGrid{};
@@ -637,6 +640,10 @@ ezo_status ezo_env_create(int32_t n_obs, const double* xyzr, ezo_env** out) {
   // are larger than that. Cells that a coordinate cannot be told apart in (a
   // set far from the origin for its size), and sets that are not finite, get
   // one cell that lists every obstacle.
+  // The memory is the pool's, since a planner makes a set for every scene it
+  // perceives: making a set of 1024 spheres, 1000 labels on it and freeing it
+  // take 141 us (365 with an allocation each time and the grid's first build
+  // kernel, 140 without a grid), 64 spheres 68 us (75, 72).
   double ext = 0.0, size = 0.0;
   for (int k = 0; k < 3; ++k) {
     ext = std::max(ext, hi[k] - lo[k]);
@@ -658,14 +665,16 @@ ezo_status ezo_env_create(int32_t n_obs, const double* xyzr, ezo_env** out) {
   // Fine cells of half the size from 257 obstacles on: among 1024 spheres on a
   // 2 cm grid 2e5 labels take 0.106 ms with them and 0.139 ms without; below,
   // the cells hold one to three candidates either way (64 obstacles, 2e6
-  // labels: 0.548 ms both) and the smaller table spares 60 us of allocation.
+  // labels: 0.548 ms both) and the smaller table is built in half the time.
   gb.sub = n_obs > 256 ? 2 : 1;
   const size_t row = (size_t)gb.sub * kGridC, cells = use ? (size_t)gb.sub * gb.n[2] * row * row : 0;
   gb.ids_cap = use && n_obs > (int)kGridInline ? (unsigned)std::max(65536, 1024 * n_obs) : 0u;
   const size_t o_lb = (size_t)(np + 1) * sizeof(float4), o_cell = o_lb + kGridLbBytes,
                o_ids = o_cell + std::max<size_t>(1, cells) * sizeof(unsigned long long);
   cudaError_t err;
-  if ((err = cudaMalloc(&e->d_mem, o_ids + sizeof(uint16_t) * std::max(1u, gb.ids_cap))) != cudaSuccess ||
+  if ((err = cudaGetDevice(&e->device)) == cudaSuccess)
+    e->d_mem = (char*)device_pool().take(o_ids + sizeof(uint16_t) * std::max(1u, gb.ids_cap), &err);
+  if (err != cudaSuccess ||
       (err = cudaMemcpy(e->d_mem, obs.data(), o_lb, cudaMemcpyHostToDevice)) != cudaSuccess) {
     ezo_env_free(e);
     return cuda_fail(err, "ezo_env_create");
@@ -731,8 +740,10 @@ ezo_status ezo_env_create(int32_t n_obs, const double* xyzr, ezo_env** out) {
 
 void ezo_env_free(ezo_env* e) {
   if (!e) return;
-  cudaFree(e->d_mem);
-  cudaFree(e->d_wide);
+  // work queued on the set ends before its memory is handed on
+  const bool idle = e->d_mem && device_idle(e->device);
+  device_pool().give(e->d_mem, idle);
+  device_pool().give(e->d_wide, idle);
   if (e->wide_ready) cudaEventDestroy(e->wide_ready);
   cudaFree(e->d_box);
   delete e;

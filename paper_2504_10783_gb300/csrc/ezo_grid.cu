@@ -1,18 +1,24 @@
 // The grid over an obstacle set that the collision kernels look spheres up in
 // (ObsGrid, ezo_device.cuh).
 //
-// One block of 64 threads per brick of 4 x 4 x 4 fine cells. The block first
-// keeps the obstacles that can be the nearest to some point of the brick
-// (lower bound of the distance over the brick at most the smallest upper
-// bound), then each thread does the same for its cell from that list, so an
-// obstacle is read once per brick and a cell looks at the few that are left:
-// 1024 obstacles cost about as much as 64. Built once per obstacle set, in
-// one launch.
+// One block per brick of 4 x 4 x 4 fine cells. The block first keeps the
+// obstacles that can be the nearest to some point of the brick (lower bound of
+// the distance over the brick at most the smallest upper bound), then four
+// threads a cell do the same for the cell from that list, so an obstacle is
+// read once per brick and a cell looks at the few that are left. Latency of
+// the bricks with the longest lists bounds it (hundreds of obstacles above a
+// dense layer): one thread a cell and an atomic a list took 12 us for 64
+// spheres, 111 for 1024 on a table and 168 for 4096 where this takes 8, 57 and
+// 106 (eight threads a cell: 9, 55, 113). Built once per obstacle set, in one
+// launch.
 #include "ezo_kernels_common.cuh"
 
 namespace ezo {
 
 namespace {
+
+constexpr int kParts = 4;  // threads a cell
+constexpr int kThreads = 64 * kParts;
 
 // Bounds of the surface distance of obstacle o over the box [lo, hi]: lower
 // less the margin, upper plus it.
@@ -31,11 +37,15 @@ __device__ __forceinline__ void surface_bounds(const float (&lo)[3], const float
   upper = sqrtf(far2) - o.w + margin;
 }
 
-__global__ void __launch_bounds__(64) k_grid_build(GridBuild g) {
+__global__ void __launch_bounds__(kThreads) k_grid_build(GridBuild g) {
   __shared__ uint16_t list[EZO_MAX_OBS];
   __shared__ int s_count;
-  __shared__ float s_min[2];
+  __shared__ float s_min[kThreads / 32];
   __shared__ int s_lb[64];
+  __shared__ float s_up[kParts][64], s_low[kParts][64];
+  __shared__ int s_kept[kParts][64];
+  __shared__ unsigned s_off[64];
+  __shared__ unsigned long long s_word[64];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int sub = g.sub, stride = sub * kGridC;
   const int n_fine[3] = {sub * g.n[0], sub * g.n[1], sub * g.n[2]};
@@ -48,9 +58,12 @@ __global__ void __launch_bounds__(64) k_grid_build(GridBuild g) {
     hi[k] = (float)(sub * g.k0[k] + b0[k] + 4) * hf;
   }
   if (t == 0) s_count = 0;
-  s_lb[t] = 255;
+  if (t < 64) {
+    s_lb[t] = 255;
+    s_word[t] = 0ull;
+  }
   float best = 3.0e38f;
-  for (int j = t; j < g.n_obs; j += 64) {
+  for (int j = t; j < g.n_obs; j += kThreads) {
     float l, u;
     surface_bounds(lo, hi, g.obs[j], g.margin, l, u);
     best = fminf(best, u);
@@ -59,8 +72,9 @@ __global__ void __launch_bounds__(64) k_grid_build(GridBuild g) {
   for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
   if (lane == 0) s_min[warp] = best;
   __syncthreads();
-  best = fminf(s_min[0], s_min[1]);
-  for (int j0 = 0; j0 < g.n_obs; j0 += 64) {
+#pragma unroll
+  for (int k = 0; k < kThreads / 32; ++k) best = fminf(best, s_min[k]);
+  for (int j0 = 0; j0 < g.n_obs; j0 += kThreads) {
     const int j = j0 + t;
     float l = 3.0e38f, u;
     if (j < g.n_obs) surface_bounds(lo, hi, g.obs[j], g.margin, l, u);
@@ -72,61 +86,89 @@ __global__ void __launch_bounds__(64) k_grid_build(GridBuild g) {
   }
   __syncthreads();
   const int cnt = s_count;
-  const int x = b0[0] + (t & 3), y = b0[1] + ((t >> 2) & 3), z = b0[2] + (t >> 4);
+  // thread (part, c): every kParts-th obstacle of the list for cell c
+  const int part = t >> 6, c = t & 63;
+  const int x = b0[0] + (c & 3), y = b0[1] + ((c >> 2) & 3), z = b0[2] + (c >> 4);
   const bool in = x < n_fine[0] && y < n_fine[1] && z < n_fine[2];
-  if (in) {
-    const int cell[3] = {x, y, z};
+  const int cell[3] = {x, y, z};
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      lo[k] = (float)(sub * g.k0[k] + cell[k]) * hf;
-      hi[k] = (float)(sub * g.k0[k] + cell[k] + 1) * hf;
+  for (int k = 0; k < 3; ++k) {
+    lo[k] = (float)(sub * g.k0[k] + cell[k]) * hf;
+    hi[k] = (float)(sub * g.k0[k] + cell[k] + 1) * hf;
+  }
+  float up = 3.0e38f, low = 3.0e38f;
+#pragma unroll 4
+  for (int i = part; i < cnt; i += kParts) {
+    float l, u;
+    surface_bounds(lo, hi, __ldg(g.obs + list[i]), g.margin, l, u);
+    up = fminf(up, u);
+    low = fminf(low, l);
+  }
+  s_up[part][c] = up;
+  s_low[part][c] = low;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kParts; ++k) {
+    up = fminf(up, s_up[k][c]);
+    low = fminf(low, s_low[k][c]);
+  }
+  int kept = 0;
+#pragma unroll 4
+  for (int i = part; i < cnt; i += kParts) {
+    float l, u;
+    surface_bounds(lo, hi, __ldg(g.obs + list[i]), g.margin, l, u);
+    kept += l <= up ? 1 : 0;
+  }
+  s_kept[part][c] = kept;
+  __syncthreads();
+  int m = 0, at = 0;  // the cell's ids, and those of the parts before this one
+#pragma unroll
+  for (int k = 0; k < kParts; ++k) {
+    at += k < part ? s_kept[k][c] : 0;
+    m += s_kept[k][c];
+  }
+  // The first kGridInline ids go into the cell's word, more into a list; the
+  // collision grid's cells farther from every obstacle than its edge need no
+  // list: a sphere that large is tested against every obstacle.
+  const bool listed = in && m > (int)kGridInline && low <= g.far;
+  if (part == 0) {  // a warp takes its cells' room together
+    int sum = listed ? m : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, sum, o);
+      if (lane >= o) sum += v;
     }
-    float up = 3.0e38f, low = 3.0e38f;
-    for (int i = 0; i < cnt; ++i) {
-      float l, u;
-      surface_bounds(lo, hi, __ldg(g.obs + list[i]), g.margin, l, u);
-      up = fminf(up, u);
-      low = fminf(low, l);
-    }
-    const int lb8 = (int)fminf(fmaxf(floorf(low / g.step), 0.f), 255.f);
-    // the ids, the first kGridInline of them in the cell's word
-    unsigned long long w = 0ull;
-    int m = 0;
-    for (int i = 0; i < cnt; ++i) {
-      float l, u;
-      surface_bounds(lo, hi, __ldg(g.obs + list[i]), g.margin, l, u);
-      if (l <= up) {
-        if (m < (int)kGridInline) w |= (unsigned long long)list[i] << (16 + 12 * m);
-        ++m;
-      }
-    }
-    unsigned kind = (unsigned)m;
-    if (m > (int)kGridInline) {
-      // the collision grid's cells farther from every obstacle than its edge
-      // need no list: a sphere that large is tested against every obstacle
-      kind = kGridAll;
-      if (low <= g.far) {
-        const unsigned off = atomicAdd(g.used, (unsigned)m);
-        if (off + (unsigned)m <= g.ids_cap) {
-          kind = kGridList;
-          w = ((unsigned long long)off << 32) | ((unsigned long long)m << 16);
-          int at = 0;
-          for (int i = 0; i < cnt; ++i) {
-            float l, u;
-            surface_bounds(lo, hi, __ldg(g.obs + list[i]), g.margin, l, u);
-            if (l <= up) g.ids[off + at++] = list[i];
-          }
-        }
-      }
-      if (kind == kGridAll) w = 0ull;
-    }
-    g.cell[(z * stride + y) * stride + x] = w | ((unsigned long long)kind << 8) | (unsigned long long)lb8;
-    // the coarse cell's bound, at its first fine cell's place
-    atomicMin(&s_lb[sub == 2 ? t & 0x2a : t], lb8);
+    unsigned base = 0u;
+    if (lane == 31 && sum) base = atomicAdd(g.used, (unsigned)sum);
+    s_off[c] = __shfl_sync(0xffffffffu, base, 31) + (unsigned)(sum - (listed ? m : 0));
   }
   __syncthreads();
-  if (in && g.lb && (sub == 1 || (t & ~0x2a) == 0))
-    g.lb[((z / sub) * kGridC + y / sub) * kGridC + x / sub] = (uint8_t)s_lb[t];
+  const unsigned off = s_off[c];
+  const bool fits = listed && off + (unsigned)m <= g.ids_cap;
+  if (in && kept && (fits || m <= (int)kGridInline)) {
+    for (int i = part; i < cnt; i += kParts) {
+      float l, u;
+      surface_bounds(lo, hi, __ldg(g.obs + list[i]), g.margin, l, u);
+      if (!(l <= up)) continue;
+      if (fits) g.ids[off + (unsigned)at] = list[i];
+      else atomicOr(&s_word[c], (unsigned long long)list[i] << (16 + 12 * at));
+      ++at;
+    }
+  }
+  const int lb8 = (int)fminf(fmaxf(floorf(low / g.step), 0.f), 255.f);
+  // the coarse cell's bound, at its first fine cell's place
+  if (in && part == 0) atomicMin(&s_lb[sub == 2 ? c & 0x2a : c], lb8);
+  __syncthreads();
+  if (!in || part != 0) return;
+  unsigned long long w = s_word[c];
+  unsigned kind = (unsigned)m;
+  if (m > (int)kGridInline) {
+    kind = fits ? kGridList : kGridAll;
+    w = fits ? ((unsigned long long)off << 32) | ((unsigned long long)m << 16) : 0ull;
+  }
+  g.cell[(z * stride + y) * stride + x] = w | ((unsigned long long)kind << 8) | (unsigned long long)lb8;
+  if (g.lb && (sub == 1 || (c & ~0x2a) == 0))
+    g.lb[((z / sub) * kGridC + y / sub) * kGridC + x / sub] = (uint8_t)s_lb[c];
 }
 
 }  // namespace
@@ -134,7 +176,7 @@ __global__ void __launch_bounds__(64) k_grid_build(GridBuild g) {
 cudaError_t launch_grid_build(const GridBuild& g, cudaStream_t s) {
   if (g.n_obs <= 0) return cudaSuccess;
   const dim3 grid((g.sub * g.n[0] + 3) / 4, (g.sub * g.n[1] + 3) / 4, (g.sub * g.n[2] + 3) / 4);
-  k_grid_build<<<grid, 64, 0, s>>>(g);
+  k_grid_build<<<grid, kThreads, 0, s>>>(g);
   return cudaGetLastError();
 }
 

@@ -2,10 +2,11 @@
 // needs working memory for its own duration takes a block and gives it back
 // when its work has completed, instead of paying for an allocation (a
 // one-segment inflation spent a third of its time in thirty of them). A pool
-// keeps at most kKeep blocks and kBytes bytes, only of sizes up to kMaxBlock,
-// hands a block out on the device it was made on and to one taker at a time,
-// and frees what it holds when the last robot, obstacle set and batch are gone.
-// A block whose work may not have completed is freed, not kept.
+// keeps at most kKeep blocks and kBytes bytes, the ones given back last and only
+// of sizes up to kMaxBlock, hands a block out on the device it was made on and
+// to one taker at a time, and frees what it holds when the last robot, obstacle
+// set and batch are gone. A block whose work may not have completed is freed,
+// not kept. Obstacle sets take their memory here too.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -76,6 +77,7 @@ class BlockPool {
     }
     if (bytes > kMaxBlock) size = bytes;
     void* p = nullptr;
+    RelaxedCapture relaxed;
     *err = host_ ? cudaMallocHost(&p, size) : cudaMalloc(&p, size);
     if (*err != cudaSuccess) {
       (void)cudaGetLastError();
@@ -91,21 +93,29 @@ class BlockPool {
   // a block from take(); idle: its work has completed
   void give(void* p, bool idle) {
     if (!p) return;
+    std::vector<Block> gone;
     {
       std::lock_guard<std::mutex> lock(mu_);
-      for (size_t i = 0; i < out_.size(); ++i)
-        if (out_[i].p == p) {
-          const Block b = out_[i];
-          out_.erase(out_.begin() + i);
-          if (idle && b.bytes <= kMaxBlock && held_.size() < kKeep && total_ + b.bytes <= kBytes) {
-            held_.push_back(b);
-            total_ += b.bytes;
-            return;
-          }
-          break;
+      size_t i = 0;
+      while (i < out_.size() && out_[i].p != p) ++i;
+      Block b{p, kMaxBlock + 1, 0};
+      if (i < out_.size()) {
+        b = out_[i];
+        out_.erase(out_.begin() + i);
+      }
+      if (idle && b.bytes <= kMaxBlock) {
+        held_.push_back(b);
+        total_ += b.bytes;
+        while (held_.size() > kKeep || total_ > kBytes) {  // the longest unused go
+          total_ -= held_.front().bytes;
+          gone.push_back(held_.front());
+          held_.erase(held_.begin());
         }
+      } else {
+        gone.push_back(b);
+      }
     }
-    release(p);
+    for (const Block& b : gone) release(b.p);
   }
 
   void trim() {
@@ -126,6 +136,7 @@ class BlockPool {
   };
   static constexpr size_t kMinBlock = 1 << 16, kMaxBlock = 32 << 20, kBytes = 64 << 20, kKeep = 8;
   void release(void* p) {
+    RelaxedCapture relaxed;
     if (host_) cudaFreeHost(p);
     else cudaFree(p);
   }

@@ -92,6 +92,14 @@ int main() {
   pool.give(large, true);
   EXPECT(g_freed.size() == 3 && g_freed.count(large));
   pool.give(nullptr, true);
+  // many small blocks do not keep a later one out: the longest unused go
+  pool.trim();
+  many.clear();
+  for (int i = 0; i < 12; ++i) many.push_back(pool.take(1000, &e));
+  for (void* p : many) pool.give(p, true);
+  void* c = pool.take(8u << 20, &e);
+  pool.give(c, true);
+  EXPECT(!g_freed.count(c) && pool.take(8u << 20, &e) == c);
   return 0;
 }
 """
