@@ -1502,6 +1502,7 @@ ezo_status ezo_batch_create(const ezo_robot* robot, int32_t n_env, const ezo_env
     take(b->view.sm_seats, kSeatSlots);
     take(b->view.q_claim, b->claim_cap + 1);
     take(b->d_flags, b->total_s);
+    take(b->d_bits, b->total_c);
     zeros = at - image;
     take(b->d_st, B);
     take(b->d_A, B * mc * n);
@@ -1512,7 +1513,6 @@ ezo_status ezo_batch_create(const ezo_robot* robot, int32_t n_env, const ezo_env
     take(b->d_dist, b->total_c);
     take(b->d_c32, b->total_c * n);
     take(b->d_cn, b->total_c);
-    take(b->d_bits, b->total_c);
     take(b->d_ga, b->total_c * n);
     take(b->d_gb, b->total_c);
     take(b->d_pidx, B * prm->n_f);

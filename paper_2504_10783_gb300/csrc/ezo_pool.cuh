@@ -53,7 +53,8 @@ class BlockPool {
  public:
   explicit BlockPool(bool host) : host_(host) {}
 
-  // at least `bytes`; null when there is no memory
+  // at least `bytes`, of the smallest that fit the one given back last; null
+  // when there is no memory
   void* take(size_t bytes, cudaError_t* err) {
     int dev = 0;
     *err = cudaGetDevice(&dev);
@@ -65,7 +66,7 @@ class BlockPool {
       size_t best = held_.size();
       for (size_t i = 0; i < held_.size(); ++i)
         if (held_[i].dev == dev && held_[i].bytes >= bytes && held_[i].bytes <= 4 * size &&
-            (best == held_.size() || held_[i].bytes < held_[best].bytes))
+            (best == held_.size() || held_[i].bytes <= held_[best].bytes))
           best = i;
       if (best < held_.size()) {
         const Block b = held_[best];
