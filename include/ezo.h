@@ -154,15 +154,15 @@ void ezo_env_free(ezo_env* env);
  * every robot sphere against every obstacle sphere and of every listed self
  * pair; flags_dev[i] = 1 iff some pair overlaps (squared centre distance
  * below the squared sum of radii), else 0. Robot spheres on the fixed base
- * frame have the same centre for every configuration: when they all clear
- * every obstacle sphere by more than 1e-4 m (checked on the host at each
- * call) their obstacle pairs are not tested again; the flags are the same.
- * Stream-ordered, asynchronous.
+ * frame have the same centre for every configuration: the obstacle pairs of
+ * the leading ones that clear every obstacle sphere by more than 1e-4 m
+ * (checked on the host at each call) are not tested again; the flags are the
+ * same. Stream-ordered, asynchronous.
  * lanes_per_config selects 1, 2, 4 or 8 cooperating lanes per configuration
  * (0 = choose from N, among the counts that fit). What fits is decided as if
  * each group of lanes kept its sphere centres, and the block the obstacles,
- * in shared memory, so large robots with many obstacles need more lanes: at the maximum sizes (256 spheres, 4096 obstacles) only 4
- * and 8 fit. Errors: EZO_ERR_INVALID_ARG (null handle, N < 0, ldq < N, bad
+ * in shared memory, so large robots with many obstacles need more lanes: at
+ * the maximum sizes (256 spheres, 4096 obstacles) only 4 and 8 fit. Errors: EZO_ERR_INVALID_ARG (null handle, N < 0, ldq < N, bad
  * lanes value, spheres and obstacles beyond shared memory at that lanes
  * value; nothing is launched), EZO_ERR_CUDA (launch failure). */
 ezo_status ezo_check_collision(const ezo_robot* robot, const ezo_env* env, const float* q_dev, int64_t N,
@@ -665,12 +665,14 @@ ezo_status ezo_probe_fp32_fma(double* tflops, void* cuda_stream);
  * plus 8 flops per obstacle pair and per self pair, every pair counted), as
  * used for rooflines. */
 double ezo_check_flops(const ezo_robot* robot, const ezo_env* env);
-/* The robot spheres (the first ones, on the fixed base frame) whose obstacle
- * pairs the checker decides once for this obstacle set instead of per
- * configuration: every such sphere clears every obstacle sphere by more than
- * 1e-4 m, whole chunks of eight spheres; 0 when none qualifies or for NULL
- * handles. Their 8 x count x n_obs flops per configuration are part of
- * ezo_check_flops but are not executed per configuration. */
+/* Robot spheres on the fixed base frame whose obstacle pairs the checker
+ * decides once for this obstacle set instead of per configuration: the whole
+ * chunks of eight of them when each sphere in these clears every obstacle
+ * sphere by more than 1e-4 m, else 0 (and 0 for NULL handles). The checker
+ * itself leaves out every leading base sphere that is clear, so this count is
+ * rounded down: 8 of the 7-DOF arm's 11. Their 8 x count x n_obs flops per
+ * configuration are part of ezo_check_flops but are not executed per
+ * configuration. */
 int32_t ezo_check_static_spheres(const ezo_robot* robot, const ezo_env* env);
 
 #ifdef __cplusplus

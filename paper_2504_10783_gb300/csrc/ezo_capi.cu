@@ -148,27 +148,25 @@ struct ezo_env {
 };
 
 // The robot spheres on the fixed base frame sit where they are for every
-// configuration, so their pairs with a static obstacle set need no test per
-// configuration when every such pair is clear. The tests then start past
-// them; the clearance is checked in
+// configuration, so the pairs of one with a static obstacle set need no test
+// per configuration when all of them are clear. The tests start past the
+// leading ones for which that holds; the clearance is checked in
 // FP64 on the FP32 values the kernels use, against 1e-4 m, far above the
 // rounding band of the FP32 test (the kernels place a base sphere exactly at
 // its FP32 local coordinates), so every label is what all spheres' tests give.
-// With a base sphere within 1e-4 m of an obstacle all spheres are tested.
-static int sweep_first(const ezo_robot* r, const ezo_env* e, int cut) {
-  if (cut == 0) return 0;
+static int sweep_first(const ezo_robot* r, const ezo_env* e) {
   // apart along an axis by the box around the base spheres and the one around
   // the obstacles: clear without a look at the pairs
   for (int k = 0; k < 3 && e->n_obs > 0; ++k)
-    if (e->lo[k] - r->base_hi[k] > 1e-4 || r->base_lo[k] - e->hi[k] > 1e-4) return cut;
-  for (int s = 0; s < cut; ++s) {
+    if (e->lo[k] - r->base_hi[k] > 1e-4 || r->base_lo[k] - e->hi[k] > 1e-4) return r->n_base;
+  for (int s = 0; s < r->n_base; ++s) {
     const float4 l = r->host.sph[s];
     for (const float4& o : e->h_obs) {
       const double dx = (double)l.x - o.x, dy = (double)l.y - o.y, dz = (double)l.z - o.z;
-      if (std::sqrt(dx * dx + dy * dy + dz * dz) - (double)l.w - (double)o.w <= 1e-4) return 0;
+      if (std::sqrt(dx * dx + dy * dy + dz * dz) - (double)l.w - (double)o.w <= 1e-4) return s;
     }
   }
-  return cut;
+  return r->n_base;
 }
 
 // The wide grid's cells and box from a build (its own coarse cells).
@@ -254,7 +252,7 @@ bool ezo_env::build_wide(cudaStream_t s) const {
 
 EnvDev ezo_env::dev_for(const ezo_robot* r) const {
   EnvDev d = dev();
-  d.s_first = sweep_first(r, this, r->n_base);
+  d.s_first = sweep_first(r, this);
   return d;
 }
 
@@ -971,7 +969,9 @@ double ezo_check_flops(const ezo_robot* robot, const ezo_env* env) {
 }
 
 int32_t ezo_check_static_spheres(const ezo_robot* robot, const ezo_env* env) {
-  return (robot && env) ? sweep_first(robot, env, (robot->n_base / EZO_CH) * EZO_CH) : 0;
+  if (!robot || !env) return 0;
+  const int whole = robot->n_base / EZO_CH * EZO_CH;
+  return sweep_first(robot, env) >= whole ? whole : 0;
 }
 
 // ------------------------------------------------------------------ batch --

@@ -258,11 +258,10 @@ struct EnvDev {
   int n_obs_pad;
   const float4* box;  // obstacle boxes, 4 float4 each: (centre, h_x), (axis 0, h_y), (axis 1, h_z), (axis 2, 0)
   int n_box;
-  // first robot sphere of the obstacle tests: the
-  // spheres before it sit on the fixed base frame, so their pairs with these
-  // obstacles are the same for every configuration, and they were found
-  // clear of every obstacle by more than any rounding band when the pair
-  // (robot, obstacle set) was set up; 0 when that does not hold
+  // first robot sphere of the obstacle tests: the spheres before it sit on the
+  // fixed base frame, so their pairs with these obstacles are the same for
+  // every configuration, and they were found clear of every obstacle by more
+  // than any rounding band when the pair (robot, obstacle set) was set up
   int s_first;
   ObsGrid grid;
 };
