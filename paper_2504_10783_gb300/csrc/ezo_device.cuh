@@ -207,8 +207,8 @@ __device__ __forceinline__ void stage_robot_boxes(float4* rbox_l, const RobotDev
 // Grid over an obstacle set (built once per set by k_grid_build): up to 32
 // coarse cells an axis and as many or twice as many fine ones. For a point of coarse
 // cell i, lb[i] step is a lower bound of its distance to the nearest obstacle
-// surface; a point outside the grid takes the cell of its projection, whose
-// bound holds for it as well (the grid contains every obstacle). A fine cell
+// surface; a point outside the grid is at least as far from all of them as from
+// the box around them. A fine cell
 // lists the obstacles that can be the nearest to some point of it: obstacle j
 // is left out when another one is nearer to every point of the cell, so a
 // sphere of any radius whose centre lies in the cell collides with the set
@@ -223,6 +223,9 @@ constexpr int kGridLbBytes = kGridC * kGridC * kGridC;
 constexpr unsigned kGridInline = 4, kGridList = 0xFE, kGridAll = 0xFF;
 
 struct ObsGrid {
+  // before the bounds, two float4: the box around the obstacles (its least and
+  // largest coordinates; the first one's w is added to a radius that is
+  // compared with the distance to the box)
   const uint8_t* lb;
   const unsigned long long* cell;
   const uint16_t* ids;
@@ -232,10 +235,9 @@ struct ObsGrid {
   // fx) likewise for the fine cells
   float inv, finv, inv_step;
   float bx, by, bz, fx, fy, fz;
-  float tx, ty, tz;  // 2^23 + last coarse cell
   float ex, ey, ez;  // 2^23 + fine cells
   int fbits;         // log2 of the fine cells' row stride: 5 or 6
-  float r_out;       // a smaller sphere whose centre lies outside the grid is free
+  int large;         // whether the robot has spheres that can be hit with their centres outside the grid
   float step;        // metres a unit of lb
 };
 
@@ -486,39 +488,66 @@ __device__ __forceinline__ bool cell_hit(const EnvDev& e, float cx, float cy, fl
     if (__fmaf_ru(r, g.inv_step, kGridBias) < __uint_as_float(0x4B000000u | (unsigned)(d & 0xffu))) return false;
   }
   const unsigned kind = (unsigned)(d >> 8) & 0xffu;
+  unsigned id[kGridInline];
+  float4 o[kGridInline];
+  bool hit = false;
   if (kind <= kGridInline) {
     // the word's one to four ids, their obstacles loaded together
-    unsigned id[kGridInline];
-    bool hit = false;
 #pragma unroll
     for (unsigned k = 0; k < kGridInline; ++k)
       id[k] = (k < kind ? (unsigned)(d >> (16 + 12 * k)) : (unsigned)(d >> 16)) & 0xfffu;
-    float4 o[kGridInline];
 #pragma unroll
     for (unsigned k = 0; k < kGridInline; ++k) o[k] = __ldg(e.obs + id[k]);
 #pragma unroll
     for (unsigned k = 0; k < kGridInline; ++k) hit = pair_hit(cx, cy, cz, r, o[k]) || hit;
     return hit;
   }
+  // four at a time; past the last one the last again
   const bool list = kind == kGridList;
   const int cnt = list ? (int)((d >> 16) & 0xffffu) : e.n_obs;
   const uint16_t* ids = g.ids + (list ? (unsigned)(d >> 32) : 0u);
-  for (int k = 0; k < cnt; ++k) {
-    const unsigned id = list ? (unsigned)__ldg(ids + k) : (unsigned)k;
-    if (pair_hit(cx, cy, cz, r, __ldg(e.obs + id))) return true;
+  for (int k0 = 0; k0 < cnt && !hit; k0 += (int)kGridInline) {
+#pragma unroll
+    for (int k = 0; k < (int)kGridInline; ++k) {
+      const int at = min(k0 + k, cnt - 1);
+      id[k] = list ? (unsigned)__ldg(ids + at) : (unsigned)at;
+    }
+#pragma unroll
+    for (unsigned k = 0; k < kGridInline; ++k) o[k] = __ldg(e.obs + id[k]);
+#pragma unroll
+    for (unsigned k = 0; k < kGridInline; ++k) hit = pair_hit(cx, cy, cz, r, o[k]) || hit;
   }
-  return false;
+  return hit;
+}
+
+// Whether a sphere whose centre lies outside the grid can touch an obstacle:
+// it is free when the box around them is farther than its radius, by more than
+// the roundings of this test and of the pair test.
+__device__ __forceinline__ bool box_within(const ObsGrid& g, float cx, float cy, float cz, float r) {
+  const float4* box = reinterpret_cast<const float4*>(g.lb);
+  const float4 lo = __ldg(box - 2), hi = __ldg(box - 1);
+  const float ox = fmaxf(fmaxf(lo.x - cx, cx - hi.x), 0.f), oy = fmaxf(fmaxf(lo.y - cy, cy - hi.y), 0.f),
+              oz = fmaxf(fmaxf(lo.z - cz, cz - hi.z), 0.f);
+  const float reach = fmaf(r, 1.00001f, lo.w);
+  return !(fmaf(ox, ox, fmaf(oy, oy, oz * oz)) > reach * reach);
+}
+
+// The coarse cell of a point as an index into lb; false outside the grid: all
+// three coordinates in [2^23, 2^23 + 32) have no bit but the low five different
+// from 2^23's.
+__device__ __forceinline__ bool coarse_cell(const ObsGrid& g, float cx, float cy, float cz, unsigned& cell) {
+  const unsigned ix = __float_as_uint(__fmaf_rd(cx, g.inv, g.bx)), iy = __float_as_uint(__fmaf_rd(cy, g.inv, g.by)),
+                 iz = __float_as_uint(__fmaf_rd(cz, g.inv, g.bz));
+  cell = ((iz * kGridC + iy) * kGridC + ix) & (kGridLbBytes - 1);
+  return ((ix ^ 0x4B000000u) | (iy ^ 0x4B000000u) | (iz ^ 0x4B000000u)) < (unsigned)kGridC;
 }
 
 // Whether the coarse bound leaves a sphere to be tested: it is free when
-// ceil(r / step) < lb (a bound of 0 may stand for a negative one). fmaxf and
-// fminf put an out-of-range (or NaN) coordinate into the grid.
+// ceil(r / step) < lb (a bound of 0 may stand for a negative one).
 __device__ __forceinline__ bool coarse_near(const ObsGrid& g, const uint8_t* __restrict__ lb, float cx, float cy,
                                             float cz, float r) {
-  const unsigned ix = __float_as_uint(fminf(fmaxf(__fmaf_rd(cx, g.inv, g.bx), kGridBias), g.tx));
-  const unsigned iy = __float_as_uint(fminf(fmaxf(__fmaf_rd(cy, g.inv, g.by), kGridBias), g.ty));
-  const unsigned iz = __float_as_uint(fminf(fmaxf(__fmaf_rd(cz, g.inv, g.bz), kGridBias), g.tz));
-  const unsigned i = ((iz & (kGridC - 1)) * kGridC + (iy & (kGridC - 1))) * kGridC + (ix & (kGridC - 1));
+  unsigned i;
+  if (!coarse_cell(g, cx, cy, cz, i)) return box_within(g, cx, cy, cz, r);
   const float bound = __uint_as_float(0x4B000000u | (unsigned)lb[i]);
   return !(__fmaf_ru(r, g.inv_step, kGridBias) < bound);
 }
@@ -798,14 +827,15 @@ struct LaneChain {
 };
 
 // Whether the coarse bound leaves a sphere (centre c, q = ceil(r / step)) to
-// be tested: its centre in the grid and its radius not below the bound.
+// be tested: its centre in the grid and its radius not below the bound, or,
+// with LARGE, a centre outside and a radius that can reach in from there.
+template <bool LARGE>
 __device__ __forceinline__ bool lane_near(const ObsGrid& g, const uint8_t* __restrict__ lb, float cx, float cy,
-                                          float cz, int q) {
-  const unsigned ix = __float_as_uint(__fmaf_rd(cx, g.inv, g.bx)), iy = __float_as_uint(__fmaf_rd(cy, g.inv, g.by)),
-                 iz = __float_as_uint(__fmaf_rd(cz, g.inv, g.bz));
-  // all three in [2^23, 2^23 + 32): no bit but the low five differs from 2^23's
-  const unsigned off = (ix ^ 0x4B000000u) | (iy ^ 0x4B000000u) | (iz ^ 0x4B000000u);
-  return off < (unsigned)kGridC && q >= (int)lb[((iz * kGridC + iy) * kGridC + ix) & (kGridLbBytes - 1)];
+                                          float cz, int q, const float4* __restrict__ l) {
+  unsigned i;
+  const bool in = coarse_cell(g, cx, cy, cz, i);
+  if constexpr (LARGE) return in ? q >= (int)lb[i] : q >= 0 && box_within(g, cx, cy, cz, l->w);
+  return in && q >= (int)lb[i];
 }
 
 // Point or vector (w = 1 or 0 for the origin) of a run's segment in the world.
@@ -977,8 +1007,7 @@ __device__ __forceinline__ void lane_walk(const float (&q)[NDOF], const LaneSmem
 // cosines), lane 0 writes the poses, and the spheres of all frames are dealt
 // to the lanes; the rolled form was a quarter slower there, where few warps
 // hide its latency.
-// Needs the robot's largest sphere to be smaller than the grid's edge: a
-// centre outside the grid is then free. All lanes of the warp call it
+// All lanes of the warp call it
 // together; returns the group-wide OR.
 // Measured at one lane, 7-DOF arm of 40 spheres (kernel time, collide_group at
 // its best lane count before): 2e6 labels among 64 obstacles 0.53 -> 0.179 ms,
@@ -1021,12 +1050,22 @@ __device__ __forceinline__ bool collide_lane(const float (&q)[NDOF], const LaneS
       for (int s0 = f == 0 ? max(ls.frame_first[0], e.s_first) : ls.frame_first[f]; s0 < s_end; s0 += 32) {
         unsigned near = 0u, bit = 1u;
         const int cnt = min(32, s_end - s0);
+        if (!g.large) {
 #pragma unroll 4
-        for (int k = 0; k < cnt; ++k, bit += bit) {
-          const float2 a = sa[s0 + k];
-          float cx, cy, cz;
-          lane_centre(P, axis, a.x, sph + s0 + k, cx, cy, cz);
-          if (lane_near(g, lb, cx, cy, cz, __float_as_int(a.y))) near |= bit;
+          for (int k = 0; k < cnt; ++k, bit += bit) {
+            const float2 a = sa[s0 + k];
+            float cx, cy, cz;
+            lane_centre(P, axis, a.x, sph + s0 + k, cx, cy, cz);
+            if (lane_near<false>(g, lb, cx, cy, cz, __float_as_int(a.y), sph + s0 + k)) near |= bit;
+          }
+        } else {
+#pragma unroll 1
+          for (int k = 0; k < cnt; ++k, bit += bit) {
+            const float2 a = sa[s0 + k];
+            float cx, cy, cz;
+            lane_centre(P, axis, a.x, sph + s0 + k, cx, cy, cz);
+            if (lane_near<true>(g, lb, cx, cy, cz, __float_as_int(a.y), sph + s0 + k)) near |= bit;
+          }
         }
         if (hit) near = 0u;
         while (__any_sync(0xffffffffu, near != 0u)) {
@@ -1046,16 +1085,23 @@ __device__ __forceinline__ bool collide_lane(const float (&q)[NDOF], const LaneS
     for (int s1 = e.s_first; s1 < ns; s1 += 32 * T) {
       const int s0 = s1 + lg;
       unsigned near = 0u;
-#pragma unroll 2
-      for (int k = 0; k < 32; ++k) {
-        const int s = s0 + k * T;
-        if (s >= ns) break;
-        const int f = frame[s];
+      auto look = [&](int k, auto near_of) {
+        const int s = s0 + k * T, f = frame[s];
         const LanePose P = lane_pose<T>(ls.slot[f], general, mine, stride);
         const float2 a = sa[s];
         float cx, cy, cz;
         lane_centre(P, ls.axis[f], a.x, sph + s, cx, cy, cz);
-        if (lane_near(g, lb, cx, cy, cz, __float_as_int(a.y))) near |= 1u << k;
+        if (near_of(cx, cy, cz, __float_as_int(a.y), sph + s)) near |= 1u << k;
+      };
+      const int cnt = min(32, (ns - s0 + T - 1) / T);
+      if (!g.large) {
+#pragma unroll 2
+        for (int k = 0; k < cnt; ++k)
+          look(k, [&](float x, float y, float z, int w, const float4* l) { return lane_near<false>(g, lb, x, y, z, w, l); });
+      } else {
+#pragma unroll 1
+        for (int k = 0; k < cnt; ++k)
+          look(k, [&](float x, float y, float z, int w, const float4* l) { return lane_near<true>(g, lb, x, y, z, w, l); });
       }
       if (hit) near = 0u;
       while (__any_sync(0xffffffffu, near != 0u)) {

@@ -144,8 +144,9 @@ __global__ void __launch_bounds__(128, NDOF <= 7 ? (SPLIT ? 5 : 7) : 4)
 
 #endif  // !EZO_BOX_TU
 
+// (one lane: 80 registers, so that the six blocks below fit)
 template <int NDOF, int T, bool BOX, bool LANE>
-__global__ void __launch_bounds__(128) k_round_check(BatchView v, int stage_lb) {
+__global__ void __launch_bounds__(128, LANE && T == 1 ? 6 : 1) k_round_check(BatchView v, int stage_lb) {
   extern __shared__ float4 smem4[];
   __shared__ typename CheckRobot<LANE>::type rs;
   const int n_tiles = v.summary->n_sample_tiles;
