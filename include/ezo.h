@@ -493,7 +493,8 @@ ezo_status ezo_path_points(const double* verts, int32_t n_verts, int32_t n, doub
  * edge_flags (host, n_verts - 1 bytes): 1 when any point of the edge
  * collides. point_flags_dev (nullable, device, point_cap bytes): 1 per
  * colliding point, in edge order. *n_points (nullable) receives the point
- * count. Synchronous; uses stream-ordered scratch (cudaMallocAsync).
+ * count. Synchronous; working memory is borrowed from a pool, or allocated
+ * for the call above 32 MB.
  * EZO_ERR_CAPACITY when point_cap is below the point count;
  * EZO_ERR_INVALID_ARG when spheres and obstacles exceed shared memory even at
  * 8 lanes per point (the lane count is chosen as in ezo_check_collision). */
