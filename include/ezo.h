@@ -162,9 +162,10 @@ void ezo_env_free(ezo_env* env);
  * (0 = choose from N, among the counts that fit). What fits is decided as if
  * each group of lanes kept its sphere centres, and the block the obstacles,
  * in shared memory, so large robots with many obstacles need more lanes: at
- * the maximum sizes (256 spheres, 4096 obstacles) only 4 and 8 fit. Errors: EZO_ERR_INVALID_ARG (null handle, N < 0, ldq < N, bad
- * lanes value, spheres and obstacles beyond shared memory at that lanes
- * value; nothing is launched), EZO_ERR_CUDA (launch failure). */
+ * the maximum sizes (256 spheres, 4096 obstacles) only 4 and 8 fit. Errors:
+ * EZO_ERR_INVALID_ARG (null handle, N < 0, ldq < N, bad lanes value, spheres
+ * and obstacles beyond shared memory at that lanes value; nothing is
+ * launched), EZO_ERR_CUDA (launch failure). */
 ezo_status ezo_check_collision(const ezo_robot* robot, const ezo_env* env, const float* q_dev, int64_t N,
                                int64_t ldq, uint8_t* flags_dev, int32_t lanes_per_config, void* cuda_stream);
 

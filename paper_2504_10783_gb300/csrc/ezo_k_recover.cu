@@ -15,13 +15,9 @@
 
 namespace ezo {
 
-#if !EZO_BOX_TU
-
 // Point i of the discretised path: edge k with off[k] <= i < off[k + 1],
 // t = (i - off[k]) / N_k with N_k = off[k + 1] - off[k] - 1 pieces, and
 // q = v_k + t (v_{k+1} - v_k) with separately rounded FP64 products and sums.
-#endif  // !EZO_BOX_TU
-
 template <int NDOF, int T, bool BOX, bool LANE>
 __global__ void __launch_bounds__(128) k_check_path(const RobotDev* __restrict__ robot, EnvDev env, int stage_lb,
                                                     const double* __restrict__ verts, int n_edges,
