@@ -112,7 +112,7 @@ struct ezo_robot {
   int n_base = 0;  // sorted spheres on frame 0 (the fixed base), the first n_base
   double base_lo[3] = {0, 0, 0}, base_hi[3] = {0, 0, 0};  // the box around them
   std::vector<double> q_lo, q_hi;
-  double r_max = 0.0;
+  double reach = 0.0, r_max = 0.0;  // reach: no sphere centre lies farther from the base
   double fk_flops = 0.0;
   bool prismatic = false;  // any prismatic joint
   int n_box = 0, n_sbp = 0, n_bbp = 0;
@@ -364,8 +364,33 @@ static int lane_code(const ezo_robot* r, const ezo_env* e) {
   return 2 * l.n_slot + l.general;
 }
 
-// The same for the signed distance, which takes any obstacle set.
-static int sd_lane(const ezo_robot* r) { return r->host.lane.ok ? 2 * r->host.lane.n_slot + r->host.lane.general : -1; }
+// The same for the signed distance of N configurations, which takes any obstacle
+// set; -1 also where one lane a configuration over all pairs is the faster form:
+// few pairs for the joints that every lane of a group walks. The lines lie where
+// the two are equal (us a call with its synchronisation, in groups and over all
+// pairs; up to 48 pairs a joint of the compiled chain, 24 where a call has few
+// configurations or there are only self pairs): 131071 configurations, 1 obstacle
+// 10 joints 193, 63, 3 joints 68, 32; 32000, 16 obstacles, 10 joints 79, 52; 4,
+// 7 joints 53, 56; 64, 10 joints 87, 99; 8000, 8, 10 joints 52, 46; 16, 53, 53;
+// 131071, no obstacle, 7 joints 68, 100. A robot of one sphere: 131071 among 256
+// obstacles 95, 47. Sets without a grid, or with all of their wide grid out of
+// reach, have no candidates to look up, only bounds that lie close together:
+// 32000, 16 obstacles, 7 joints 130, 79; 32, 138, 108; 64, 162, 166.
+static int sd_lane(const ezo_robot* r, const ezo_env* e, long long N) {
+  if (!r->host.lane.ok) return -1;
+  const int lane = 2 * r->host.lane.n_slot + r->host.lane.general;
+  if (check_smem_bytes(r->nsp_pad, e->n_obs_pad, 64, 1) > kSmemBudget) return lane;
+  const int joints = r->n <= 3 ? 3 : (r->n <= 7 ? 7 : EZO_MAX_DOF);
+  const long long pairs = (long long)r->n_spheres * e->n_obs + r->n_self;
+  long long most = (e->n_obs == 0 || N < 16000 ? 24 : 48) * joints;
+  if (e->n_obs > 0 && N >= 24000) {
+    double d2 = 0.0;  // from the base to the wide grid
+    for (int k = 0; k < 3; ++k) d2 += std::pow(std::max({e->lo[k] - e->ext, -(e->hi[k] + e->ext), 0.0}), 2.0);
+    if (!e->gridded || d2 > r->reach * r->reach) most = 288 * joints;
+    else if (r->n_spheres < 4) most = 512;
+  }
+  return pairs <= most ? -1 : lane;
+}
 
 extern "C" {
 
@@ -547,6 +572,7 @@ ezo_status ezo_robot_create(int32_t n, const double* a, const double* alpha, con
       h.n_sblk = 0;
     }
     plan_lane(h, ok ? norm : std::vector<std::pair<int, int>>(), ok || norm.empty(), chain + loc_max);
+    r->reach = chain + loc_max;
     const double a2 = 2.0 * (chain + loc_max), b2 = 2.0 * r->r_max;
     h.E_self = (float)(8.0 * kU32 * (a2 * a2 + b2 * b2));
   }
@@ -878,8 +904,9 @@ ezo_status ezo_signed_distance(const ezo_robot* robot, const ezo_env* env, const
     return fail(EZO_ERR_INVALID_ARG, "ezo_signed_distance: sphere geometries only (the robot or env has boxes)");
   if (check_smem_bytes(robot->nsp_pad, env->n_obs_pad, 64, 1) > kSmemBudget)
     return fail(EZO_ERR_INVALID_ARG, "ezo_signed_distance: robot and obstacle spheres exceed shared memory");
-  cudaError_t e = launch_sd_flat(robot->d_robot, robot->n, robot->nsp_pad, sd_lane(robot), env->dev(),
-                                 sd_lane(robot) >= 0 ? env->signed_distance_grid(N, (cudaStream_t)stream) : WideGrid{},
+  const int lane = sd_lane(robot, env, N);
+  cudaError_t e = launch_sd_flat(robot->d_robot, robot->n, robot->nsp_pad, lane, env->dev(),
+                                 lane >= 0 ? env->signed_distance_grid(N, (cudaStream_t)stream) : WideGrid{},
                                  q_dev, ldq, N, sd_dev, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "ezo_signed_distance");
   g_err.clear();
@@ -955,7 +982,9 @@ __attribute__((visibility("hidden"))) ezo::WideGrid ezo_internal_sd_grid(const e
   return e->signed_distance_grid(N, s);
 }
 
-__attribute__((visibility("hidden"))) int ezo_internal_sd_lane(const ezo_robot* r) { return sd_lane(r); }
+__attribute__((visibility("hidden"))) int ezo_internal_sd_lane(const ezo_robot* r, const ezo_env* e, long long N) {
+  return sd_lane(r, e, N);
+}
 
 __attribute__((visibility("hidden"))) void ezo_internal_set_error(const char* msg) { g_err = msg ? msg : ""; }
 

@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(128) k_sd_flat(const RobotDev* __restrict__ ro
   float4* obs_s = sph_s + nsp;
   float4* cen_all = obs_s + env.n_obs_pad;
   stage_robot(rs, sph_s, robot);
-  for (int i = threadIdx.x; i < env.n_obs_pad; i += blockDim.x) obs_s[i] = env.obs[i];
+  stage_obs(obs_s, env);
   __syncthreads();
   float4* cen = cen_all + threadIdx.x * (nsp + 1);
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
@@ -287,7 +287,7 @@ cudaError_t launch_sd_flat(const RobotDev* robot, int n, int nsp_pad, int lane, 
     });
     return e;
   }
-  // self pairs that distance_lane cannot order
+  // few pairs, or self pairs that distance_lane cannot order
   cudaError_t err = cudaSuccess;
   const int threads = 64;
   const size_t smem = check_smem_rule(nsp_pad, env.n_obs_pad, threads, 1);

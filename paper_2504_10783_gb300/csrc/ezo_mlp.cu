@@ -73,7 +73,7 @@ cudaError_t dal(T** p, size_t n) {
 
 extern "C" int ezo_internal_robot_boxes(const ezo_robot* r);
 extern "C" int ezo_internal_env_boxes(const ezo_env* e);
-extern "C" int ezo_internal_sd_lane(const ezo_robot* r);
+extern "C" int ezo_internal_sd_lane(const ezo_robot* r, const ezo_env* e, long long N);
 extern "C" int ezo_internal_env_dev(const ezo_robot* r, const ezo_env* e, ezo::EnvDevFull* out);
 extern "C" ezo::WideGrid ezo_internal_sd_grid(const ezo_env* e, long long N, cudaStream_t s);
 extern "C" int ezo_internal_robot_prismatic(const ezo_robot* r);
@@ -356,8 +356,8 @@ ezo_status ezo_surrogate_train(ezo_surrogate* S, const ezo_env* env, int64_t n_s
   const RobotDev* rd = ezo_internal_robot_dev(S->robot, &n, &nsp, lo, hi);
   EnvDevFull ef{};
   ezo_internal_env_dev(S->robot, env, &ef);
-  const int lane = ezo_internal_sd_lane(S->robot);
   const long long N = n_samples / batch * batch;
+  const int lane = ezo_internal_sd_lane(S->robot, env, N);
   // one block: the configurations, their labels, the joint limits
   float* q = nullptr;
   cudaError_t e = dal(&q, (size_t)(n + 1) * N + 2 * EZO_MAX_DOF);
