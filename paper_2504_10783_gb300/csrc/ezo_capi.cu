@@ -1661,7 +1661,7 @@ ezo_status ezo_batch_create(const ezo_robot* robot, int32_t n_env, const ezo_env
     if (envs[e2]->n_obs > envs[e_big]->n_obs) e_big = e2;
   if (v.lane >= 0) {
     b->T_check = lane_check_lanes(tot_s1);
-    b->T_bisect = lane_bisect_lanes(tot_np);
+    b->T_bisect = lane_bisect_lanes(tot_np, b->n, robot->nsp_pad);
   } else {
     // collide_group: two lanes per label below ~1e6 samples a round (whole
     // inflations ran faster than at the flat tuner's pick there), and for the

@@ -674,7 +674,8 @@ __device__ __forceinline__ bool box_pairs_hit(const RobotSmem& rs, const float4*
 struct LaneSmem {
   float4 joint[2 * EZO_MAX_DOF];  // (ca, sa, a, d), (toff, kth, kd, 0)
   int frame_first[EZO_MAX_DOF + 2], axis[EZO_MAX_DOF + 2], slot[EZO_MAX_DOF + 2];
-  int n, n_spheres, last, n_link, general;
+  int n, n_spheres, last, n_link, general, n_self;
+  const ushort2* self_pairs;  // in global memory
   LinkPair link[kLinkPairs];
 };
 
@@ -707,6 +708,8 @@ __device__ __forceinline__ void stage_lane_robot(LaneSmem& ls, float4* sph, int*
     ls.last = lr.last;
     ls.n_link = lr.n_link;
     ls.general = lr.general;
+    ls.n_self = rd->n_self;
+    ls.self_pairs = rd->self_pairs;
   }
   for (int i = threadIdx.x; i < rd->n_spheres; i += blockDim.x) {
     sph[i] = rd->sph[i];
@@ -917,6 +920,29 @@ __device__ __forceinline__ bool links_hit(const LaneSmem& ls, const float4* __re
   return false;
 }
 
+// The listed self pairs one by one, lg, lg + T, ..: where the group has a lane or
+// two for each, their one or two links would keep as many lanes busy while the
+// others wait. The planar arm's 16 pairs (one link): a round's bisection of 2500
+// candidates at sixteen lanes 62 -> 52 us, of 5000 at eight 51 -> 45. In the
+// kernels of up to 3 joints; the others' robots have more pairs.
+template <int T>
+__device__ __forceinline__ bool pairs_hit(const LaneSmem& ls, const float4* __restrict__ sph,
+                                          const float2* __restrict__ sa, const int* __restrict__ frame,
+                                          const float* mine, int stride, int lg) {
+  bool hit = false;
+  for (int p = lg; p < ls.n_self; p += T) {
+    const ushort2 pr = __ldg(ls.self_pairs + p);
+    const int fa = frame[pr.x], fb = frame[pr.y];
+    const LanePose A = lane_pose<T>(ls.slot[fa], ls.general, mine, stride),
+                   B = lane_pose<T>(ls.slot[fb], ls.general, mine, stride);
+    float ax, ay, az, bx, by, bz;
+    lane_centre(A, ls.axis[fa], sa[pr.x].x, sph + pr.x, ax, ay, az);
+    lane_centre(B, ls.axis[fb], sa[pr.y].x, sph + pr.y, bx, by, bz);
+    hit = pair_hit(ax, ay, az, sph[pr.x].w, make_float4(bx, by, bz, sph[pr.y].w)) || hit;
+  }
+  return hit;
+}
+
 // A warp's queue of spheres to test against their cells: the lanes put in
 // those that the coarse bound did not free, and 32 at a time are tested, one
 // a lane, from their owner's kept pose. Few spheres are left (0.7 of 29 a
@@ -1112,7 +1138,11 @@ __device__ __forceinline__ bool collide_lane(const float (&q)[NDOF], const LaneS
       }
     }
     if (nq.count && nq.test(ls, sph, sa, frame, e, mine, stride)) hit = true;
-    if (!hit) hit = links_hit<T>(ls, sph, sa, mine, stride, lg);
+    if (NDOF <= 3 && ls.n_self <= 2 * T) {
+      if (!hit) hit = pairs_hit<T>(ls, sph, sa, frame, mine, stride, lg);
+    } else if (!hit) {
+      hit = links_hit<T>(ls, sph, sa, mine, stride, lg);
+    }
     unsigned h = hit ? 1u : 0u;
 #pragma unroll
     for (int off = 1; off < T; off <<= 1) h |= __shfl_xor_sync(0xffffffffu, h, off, T);

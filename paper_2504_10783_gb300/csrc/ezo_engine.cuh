@@ -235,9 +235,13 @@ size_t check_smem_bytes(int n_spheres_pad, int n_obs_pad, int threads, int T, in
 // are fastest at the few thousand candidates of a path's round (0.054 ms;
 // 0.060 at four and sixteen), sixteen at a segment's few hundred (0.039 ms;
 // 0.042 at eight), four where a round holds hundreds of thousands (24 paths:
-// 3.0 ms; 3.2 at eight, 3.6 at one).
+// 3.0 ms; 3.2 at eight, 3.6 at one). Arms of up to three joints and sixteen
+// spheres leave lanes idle sooner (planar arm, a round of one segment at sixteen,
+// eight and four lanes: 1000 candidates 30, 31, 35 us; 5000 32, 33, 37, the whole
+// inflation 256, 262 and 271; 20000 52, 45, 40; six segments of 5000 66, 52, 46).
 inline int lane_check_lanes(long long samples) { return samples >= (1ll << 16) ? 1 : (samples >= (1ll << 14) ? 2 : 4); }
-inline int lane_bisect_lanes(long long candidates) {
+inline int lane_bisect_lanes(long long candidates, int n, int nsp_pad) {
+  if (n <= 3 && nsp_pad <= 16) return candidates >= (1ll << 14) ? 4 : (candidates >= (1ll << 12) ? 8 : 16);
   return candidates >= (1ll << 20) ? 4 : (candidates >= (1ll << 15) ? 8 : 16);
 }
 // Dynamic shared memory a collision kernel may request: the opt-in maximum

@@ -292,7 +292,7 @@ extern "C" ezo_status ezo_inflate_segment_noalloc(const ezo_robot* robot, const 
   const bool lane = v.lane >= 0;
   const int T_check = std::max(lane ? lane_check_lanes(s_cap) : check_lanes(s_cap), t_min);
   const int T_bis = std::max(
-      lane ? lane_bisect_lanes(np) : bisect_lanes(np, ezo_internal_robot_boxes(robot) || envf.e.n_box), t_min);
+      lane ? lane_bisect_lanes(np, n, nsp_pad) : bisect_lanes(np, ezo_internal_robot_boxes(robot) || envf.e.n_box), t_min);
   const int grid_s = (int)std::max<long long>(1, std::min<long long>(st_tiles * 8, (long long)sms * 16));
   const int grid_c = (int)std::max<long long>(1, std::min<long long>(st_tiles * T_check, (long long)sms * 16));
   const int grid_b = (int)std::max<long long>(1, std::min<long long>(bi_tiles * T_bis, (long long)sms * 16));
