@@ -173,9 +173,10 @@ ezo_status ezo_check_collision(const ezo_robot* robot, const ezo_env* env, const
  * ||c_i - c_j|| - r_i - r_j in FP32 (negative iff in collision). Used to
  * label data and to bound ambiguous decisions. Stream-ordered, asynchronous.
  * The first call of at least 16384 configurations on an obstacle set, outside
- * a capture, allocates a grid of its own for the set (3 MB for 1024
- * obstacles, freed with it) and queues its build on the call's stream; calls
- * on other streams wait for the build on the device.
+ * a capture, may allocate a grid of its own for the set (3 MB for 1024
+ * obstacles, freed with it; robots and sets of few pairs need none) and queue
+ * its build on the call's stream; calls on other streams wait for the build on
+ * the device.
  * EZO_ERR_INVALID_ARG when the robot or env has boxes, or when its spheres
  * and obstacles exceed shared memory by the rule of one lane per
  * configuration: (spheres + 1) x 64 centres plus the obstacles (the kernels

@@ -1033,8 +1033,7 @@ __device__ __forceinline__ void lane_walk(const float (&q)[NDOF], const LaneSmem
 // cosines), lane 0 writes the poses, and the spheres of all frames are dealt
 // to the lanes; the rolled form was a quarter slower there, where few warps
 // hide its latency.
-// All lanes of the warp call it
-// together; returns the group-wide OR.
+// All lanes of the warp call it together; returns the group-wide OR.
 // Measured at one lane, 7-DOF arm of 40 spheres (kernel time, collide_group at
 // its best lane count before): 2e6 labels among 64 obstacles 0.53 -> 0.179 ms,
 // of which the chain takes 0.05, the 29 lookups 0.04, the spheres left to
